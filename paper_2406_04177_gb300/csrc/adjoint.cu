@@ -22,7 +22,9 @@
 #include <cmath>
 #include <vector>
 
+#include "pdl.cuh"
 #include "physics.cuh"
+#include "sparse_pass.cuh"
 #include "stencil.cuh"
 #include "vga_internal.cuh"
 
@@ -183,44 +185,18 @@ __global__ void __launch_bounds__(kThreads) k_fused_rec_vec(int64_t n, NbrTable 
     table_vec<1, WM, 0, PREC, TF, 4, true>(i0, (uint32_t)n, tb, bt, p, io, rec);
 }
 
-// Sparse fused pass with recording, first half: the forward's MODE 4 body (every node's DOM diffused,
-// marked nodes left for the second half), writing h + l of every node's diffused DOM to rec.y2.  At
-// an unmarked node the transformation is the identity, so that value is both X^k_2 and y2^k.
-template <int WM, int PREC, int TF>
-__global__ void __launch_bounds__(kThreads) k_dom_rec_vec(int64_t n, NbrTable tb, BlockTable bt, StepParams p,
-                                                          StateIO io, PassRecord rec, SparseState ss) {
-    const uint32_t i0 = 4u * ((uint32_t)blockIdx.x * blockDim.x + threadIdx.x);
-    table_vec<4, WM, 0, PREC, TF, 4, true>(i0, (uint32_t)n, tb, bt, p, io, rec, ss);
-}
-
-// Second half: the marked nodes in rank order (k_transform_compact's arithmetic), recording their
-// X^k (MB, DOM, SOM, FOM, FP32 h + l; xc row q at q * xcap) and overwriting y2^k with the
-// transformed DOM.
-template <int PREC>
-__global__ void __launch_bounds__(kThreads) k_transform_compact_rec(int64_t m, SparseState ss, StepParams p,
-                                                                    StateIO io, float *__restrict__ y2,
-                                                                    float *__restrict__ xc, int64_t xcap) {
-    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= m) return;
-    const uint32_t i = __ldg(ss.list + r);
-    V x2;
-    x2.h = io.out[1][i];
-    x2.l = PREC == P_COMP ? res_decode(io.lout[1][i], x2.h) : 0.0f;
-    V v[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        v[q].h = ss.h[q][r];
-        v[q].l = PREC == P_COMP ? res_decode(ss.l[q][r], v[q].h) : 0.0f;
-    }
-    xc[r] = __fadd_rn(v[0].h, v[0].l);
-    xc[xcap + r] = __fadd_rn(x2.h, x2.l);
-    xc[2 * xcap + r] = __fadd_rn(v[1].h, v[1].l);
-    xc[3 * xcap + r] = __fadd_rn(v[2].h, v[2].l);
-    transform_sync<PREC>(v[0], x2, v[1], v[2], v[3], p);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) vstore<PREC>(ss.h[q], ss.l[q], r, v[q]);
-    vstore<PREC>(io.out[1], io.lout[1], i, x2);
-    y2[i] = __fadd_rn(x2.h, x2.l);
+// Sparse fused pass with recording (sparse_pass.cuh): y2^k of every node and X^k of the marked nodes.
+// At an unmarked node the transformation is the identity, so its diffused DOM is both X^k_2 and y2^k.
+template <int WM, int PREC, int TF, bool AHEAD>
+__global__ void __launch_bounds__(kSparseThreads, 5)
+    k_sparse_pass_rec(int64_t n, NbrTable tb, BlockTable bt, StepParams p, StateIO io, SparseState ss, SparseRecord rec,
+                      int ahead) {
+    __shared__ SparseShared sm;
+    pdl_wait();
+    pdl_trigger();
+    const uint32_t blk = AHEAD && ahead < 0 ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
+    sparse_pass_block<WM, 0, PREC, TF, true, AHEAD>(sm, blk * kSparseNodes, (uint32_t)n, (n + 31) >> 5, p.c, tb, bt, io,
+                                                    ss, rec, ahead, [&](uint32_t) -> const StepParams & { return p; });
 }
 
 // Compensated FP32 accumulator (TwoSum into a second float): GB300 issues FP64 at a small fraction of
@@ -819,6 +795,23 @@ static vga_status copy_state(vga_sim *s, PairBuf p, bool to_sim) {
     return VGA_OK;
 }
 
+// Where recorded step j of a segment goes (sparse records).
+static SparseRecord sparse_record(const AdjointBuffers *a, int64_t j) {
+    SparseRecord r;
+    r.y2 = a->rec_y2 + (size_t)j * a->npad;
+    r.xc = a->rec_xc + (size_t)j * 4 * a->xcap;
+    r.xcap = a->xcap;
+    return r;
+}
+
+template <int WM, int PREC>
+static void launch_sparse_rec(vga_sim *s, const NbrTable &tb, const BlockTable &bt, const StateIO &io,
+                              const SparseState &ss, const SparseRecord &rec, int pass, cudaStream_t st) {
+    auto kern = tb.tz ? (sparse_streams(s->n) ? k_sparse_pass_rec<WM, PREC, 1, true> : k_sparse_pass_rec<WM, PREC, 1, false>)
+                      : (sparse_streams(s->n) ? k_sparse_pass_rec<WM, PREC, 0, true> : k_sparse_pass_rec<WM, PREC, 0, false>);
+    launch_pdl(kern, grid_for(s->n, kSparseNodes), kSparseThreads, st, s->n, tb, bt, s->sp, io, ss, rec, sparse_ahead(pass));
+}
+
 // The steps of the last segment in the forward sweep, written as the backward sweep's
 // recomputation would write them: the same passes as sim_step_explicit (transformation pass, fused
 // passes on the four-node body, diffusion-only pass) with the records of X^k and y2^k, so the
@@ -849,17 +842,11 @@ static vga_status forward_recording(vga_sim *s, AdjointBuffers *a, int64_t len) 
         const int64_t m = a->act.n_active;
         if (m > 0) VGA_TRY(activity_copy(a->act, s->n, state_io_inplace(s), true, true, st));
         for (int64_t j = 1; j < len; ++j) {
-            const PassRecord pr = {nullptr, a->rec_y2 + (size_t)j * npad, npad};
-            const StateIO io = state_io(s);
             timing_begin(s, VGA_KERNEL_FUSED_STEP);
-            if (tb.tz) k_dom_rec_vec<WM, PREC, 1><<<Gv, kThreads, 0, st>>>(s->n, tb, bt, s->sp, io, pr, ss);
-            else k_dom_rec_vec<WM, PREC, 0><<<Gv, kThreads, 0, st>>>(s->n, tb, bt, s->sp, io, pr, ss);
-            if (m > 0)
-                k_transform_compact_rec<PREC><<<grid_for(m, kThreads), kThreads, 0, st>>>(
-                    m, ss, s->sp, io, pr.y2, a->rec_xc + (size_t)j * 4 * a->xcap, a->xcap);
+            launch_sparse_rec<WM, PREC>(s, tb, bt, state_io(s), ss, sparse_record(a, j), (int)j, st);
             timing_end(s);
             VGA_CHECK_LAUNCH();
-            s->launches += m > 0 ? 2 : 1;
+            ++s->launches;
             s->cur[1] ^= 1;
         }
         if (m > 0) VGA_TRY(activity_copy(a->act, s->n, state_io_inplace(s), false, true, st));
@@ -1062,14 +1049,9 @@ static vga_status adjoint_backward_impl(vga_sim *s, const double *d_lamN, double
                 auto issue = [&](cudaStream_t cs) -> vga_status {
                     int w = 0;
                     for (int64_t j = 1; j < len; ++j) {
-                        const PassRecord pr = {nullptr, a->rec_y2 + (size_t)j * npad, npad};
                         const StateIO io = io_from(a->work[w], a->work[1 - w], npad);
                         timing_begin(s, VGA_KERNEL_FUSED_STEP);
-                        if (tb.tz) k_dom_rec_vec<WM, PREC, 1><<<Gv, kThreads, 0, cs>>>(s->n, tb, bt, s->sp, io, pr, ss);
-                        else k_dom_rec_vec<WM, PREC, 0><<<Gv, kThreads, 0, cs>>>(s->n, tb, bt, s->sp, io, pr, ss);
-                        if (m > 0)
-                            k_transform_compact_rec<PREC><<<grid_for(m, kThreads), kThreads, 0, cs>>>(
-                                m, ss, s->sp, io, pr.y2, a->rec_xc + (size_t)j * 4 * a->xcap, a->xcap);
+                        launch_sparse_rec<WM, PREC>(s, tb, bt, io, ss, sparse_record(a, j), (int)j, cs);
                         timing_end(s);
                         VGA_CHECK_LAUNCH();
                         w = 1 - w;
@@ -1077,7 +1059,7 @@ static vga_status adjoint_backward_impl(vga_sim *s, const double *d_lamN, double
                     return VGA_OK;
                 };
                 VGA_TRY(graphs.run(0, len, issue));
-                s->launches += (len - 1) * (m > 0 ? 2 : 1);
+                s->launches += len - 1;
             }
             for (int64_t j = 1; j < len && !sparse; ++j) {
                 rec.x = a->rec_x + (size_t)j * 5 * npad;

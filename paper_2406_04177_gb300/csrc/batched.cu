@@ -20,6 +20,7 @@
 
 #include "grid_sync.cuh"
 #include "physics.cuh"
+#include "sparse_pass.cuh"
 #include "stencil.cuh"
 #include "vga_internal.cuh"
 
@@ -35,11 +36,25 @@ struct BInst {
     StepParams p;
 };
 
+static_assert(kTile == kSparseThreads && kSparseNodes % kTile == 0, "a warp of a sparse pass lies in one tile");
+
+// Diffusion coefficient D dt of a tile's instance and one past that instance's last node.
+struct ChunkInfo {
+    float c;
+    uint32_t end;
+};
+
+__device__ __forceinline__ ChunkInfo __ldg_chunk(const ChunkInfo *p) {
+    const float2 v = __ldg(reinterpret_cast<const float2 *>(p));
+    return ChunkInfo{v.x, __float_as_uint(v.y)};
+}
+
 struct BatchArgs {
     int64_t ntiles;
     int64_t npad;
     const int32_t *tile_inst;  // instance of every tile
     const BInst *inst;
+    const ChunkInfo *tile_info;
     NbrTable tb;
     float *h[2];
     res_t *l[2];
@@ -47,7 +62,6 @@ struct BatchArgs {
     int32_t *err;
     StateIO io[2];  // a pass whose input is state buffer k reads io[k] (kept as kernel parameters)
     SparseState ss;    // the sparse fused pass of the SPARSE instantiations (compact state, rank list)
-    int64_t n_active;  // marked nodes (ranks of the compact state)
     int32_t skip_block;   // test of the bounded waits: this block leaves before any barrier (-1: none)
     uint32_t spin_limit;  // polls of a grid barrier before it gives up
 };
@@ -57,7 +71,7 @@ struct BatchArgs {
 // belong to one instance, whose parameters the warp reads from shared memory (per-thread copies
 // would hold a dozen registers); every thread of a block runs the same number of iterations (the
 // warp-wide shuffles need all lanes).
-template <int TR, int PREC, int TF, bool SPARSE>
+template <int TR, int PREC, int TF>
 __device__ __forceinline__ void batch_fused_pass(const BatchArgs &a, const StateIO &io) {
     constexpr int KG = kBatchGroup;
     __shared__ StepParams wp[kTile / 32];
@@ -75,35 +89,23 @@ __device__ __forceinline__ void batch_fused_pass(const BatchArgs &a, const State
         __syncwarp();
         if ((threadIdx.x & 31) == 0) wp[w] = k >= 0 ? a.inst[k].p : StepParams{};
         __syncwarp();
-        if (SPARSE) table_vec<4, W_UNIT, TR, PREC, TF, KG>(i0, end, a.tb, BlockTable{}, wp[w], io, PassRecord{}, a.ss);
-        else table_vec<1, W_UNIT, TR, PREC, TF, KG>(i0, end, a.tb, BlockTable{}, wp[w], io);
+        table_vec<1, W_UNIT, TR, PREC, TF, KG>(i0, end, a.tb, BlockTable{}, wp[w], io);
     }
 }
 
-// Second half of a sparse fused pass, after a grid barrier: the marked nodes in rank order, each with
-// its instance's parameters, MB, SOM, FOM, CO2 from the compact state (updated in place) and its DOM
-// as the first half (MODE 4) stored it; stores the DOM as the dense fused pass does.  The DOM and
-// the compact state were written inside this launch, so they are read with coherent loads.
-template <int TR, int PREC>
-__device__ __forceinline__ void batch_transform_marked(const BatchArgs &a, const StateIO &io) {
-    const SparseState &ss = a.ss;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < a.n_active; r += stride) {
-        const uint32_t i = __ldg(ss.list + r);
-        const StepParams p = a.inst[__ldg(a.tile_inst + i / kTile)].p;
-        V x2;
-        x2.h = io.out[1][i];
-        x2.l = PREC == P_COMP ? res_decode(io.lout[1][i], x2.h) : 0.0f;
-        V v[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            v[q].h = ss.h[q][r];
-            v[q].l = PREC == P_COMP ? res_decode(ss.l[q][r], v[q].h) : 0.0f;
-        }
-        transform_n<TR, PREC>(v[0], x2, v[1], v[2], v[3], p);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) vstore<PREC>(ss.h[q], ss.l[q], r, v[q]);
-        vstore<PREC>(io.out[1], io.lout[1], i, x2);
+// The sparse fused pass (sparse_pass.cuh) over the whole batch: the 128 nodes of a warp lie in one tile,
+// hence in one instance.
+template <int TR, int PREC, int TF>
+__device__ __forceinline__ void batch_sparse_pass(const BatchArgs &a, const StateIO &io) {
+    __shared__ SparseShared sm;
+    const int64_t nsuper = (a.ntiles + 3) / 4, words = a.ntiles * (kTile / 32);
+    for (int64_t s = blockIdx.x; s < nsuper; s += gridDim.x) {
+        const int64_t v0 = s * kSparseNodes, tile = (v0 + 4 * threadIdx.x) / kTile;
+        const ChunkInfo ci = tile < a.ntiles ? __ldg_chunk(a.tile_info + tile) : ChunkInfo{0.0f, 0u};
+        sparse_pass_block<W_UNIT, TR, PREC, TF, false, false>(
+            sm, (uint32_t)v0, ci.end, words, ci.c, a.tb, BlockTable{}, io, a.ss, SparseRecord{}, 0,
+            [&](uint32_t i) -> const StepParams & { return a.inst[__ldg(a.tile_inst + i / kTile)].p; });
+        __syncthreads();  // the next turn reuses the shared pairs
     }
 }
 
@@ -122,12 +124,11 @@ __global__ void __launch_bounds__(kTile, SPARSE ? 5 : 1) k_batch(BatchArgs a, in
             // fused pass: kBatchGroup consecutive nodes per thread (table_vec).  Instances start on
             // tile boundaries, so a group never straddles two; every thread of a block runs the
             // same number of iterations (the warp-wide shuffles need all lanes).
-            if (bi == 0) batch_fused_pass<TR, PREC, TF, SPARSE>(a, a.io[0]);
-            else batch_fused_pass<TR, PREC, TF, SPARSE>(a, a.io[1]);
             if constexpr (SPARSE) {
-                if (!grid_barrier(a.bar, a.err, a.spin_limit)) return;
-                if (bi == 0) batch_transform_marked<TR, PREC>(a, a.io[0]);
-                else batch_transform_marked<TR, PREC>(a, a.io[1]);
+                batch_sparse_pass<TR, PREC, TF>(a, a.io[bi]);
+            } else {
+                if (bi == 0) batch_fused_pass<TR, PREC, TF>(a, a.io[0]);
+                else batch_fused_pass<TR, PREC, TF>(a, a.io[1]);
             }
             if (pass + 1 < pass1 && !grid_barrier(a.bar, a.err, a.spin_limit)) return;
             continue;
@@ -246,6 +247,7 @@ struct vga_batch {
     uint32_t *tz = nullptr;     // compact z offsets (npad) when they fit in 16 bits
     int32_t *tile_inst = nullptr;
     BInst *inst = nullptr;
+    ChunkInfo *tile_info = nullptr;
     unsigned *bar = nullptr;
     int32_t *err = nullptr;
     double *stage = nullptr;
@@ -312,6 +314,7 @@ vga_status launch_batch(vga_batch *b, int32_t pass0, int32_t pass1, int32_t npas
     a.npad = b->npad;
     a.tile_inst = b->tile_inst;
     a.inst = b->inst;
+    a.tile_info = b->tile_info;
     a.tb.ty = b->table;
     a.tb.tzm = b->table + b->npad;
     a.tb.tzp = b->table + 2 * b->npad;
@@ -323,7 +326,6 @@ vga_status launch_batch(vga_batch *b, int32_t pass0, int32_t pass1, int32_t npas
     a.bar = b->bar;
     a.err = b->err;
     a.ss = activity_state(b->act);
-    a.n_active = b->act.n_active;
     a.skip_block = b->wait_test_block;
     a.spin_limit = b->wait_test_spin ? b->wait_test_spin : kBarrierSpin;
     for (int k = 0; k < 2; ++k) {
@@ -432,6 +434,7 @@ vga_status vga_batch_free(vga_batch *b) {
     dfree(b->tz);
     dfree(b->tile_inst);
     dfree(b->inst);
+    dfree(b->tile_info);
     dfree(b->bar);
     activity_free(&b->act);
     dfree(b->err);
@@ -470,6 +473,7 @@ vga_status vga_batch_create(const vga_graph *const *graphs, const vga_params *pa
         st = fail(VGA_ERR_CUDA, "cudaStreamCreate failed");
     int64_t off = 0;
     std::vector<int32_t> tinst;
+    std::vector<ChunkInfo> tinfo;
     std::vector<BInst> hinst(count);
     for (int k = 0; k < count && st == VGA_OK; ++k) {
         b->start.push_back(off);
@@ -480,7 +484,10 @@ vga_status vga_batch_create(const vga_graph *const *graphs, const vga_params *pa
         sim_prepare_params(&tmp, &params[k]);
         hinst[k].p = tmp.sp;
         const int64_t tiles = (graphs[k]->n + kTile - 1) / kTile;
-        for (int64_t t = 0; t < tiles; ++t) tinst.push_back(k);
+        for (int64_t t = 0; t < tiles; ++t) {
+            tinst.push_back(k);
+            tinfo.push_back(ChunkInfo{hinst[k].p.c, (uint32_t)(off + graphs[k]->n)});
+        }
         off += tiles * kTile;
     }
     if (st == VGA_OK && off >= ((int64_t)1 << 31)) st = fail(VGA_ERR_UNSUPPORTED, "a batch holds fewer than 2^31 nodes");
@@ -494,6 +501,7 @@ vga_status vga_batch_create(const vga_graph *const *graphs, const vga_params *pa
     }
     if (st == VGA_OK) st = dmalloc((void **)&b->table, sizeof(uint32_t) * 3 * (size_t)b->npad, "batch table");
     if (st == VGA_OK) st = dmalloc((void **)&b->tile_inst, sizeof(int32_t) * std::max<size_t>(tinst.size(), 1), "tile map");
+    if (st == VGA_OK) st = dmalloc((void **)&b->tile_info, sizeof(ChunkInfo) * std::max<size_t>(tinfo.size(), 1), "tile map");
     if (st == VGA_OK) st = dmalloc((void **)&b->inst, sizeof(BInst) * (size_t)count, "instances");
     if (st == VGA_OK) st = dmalloc((void **)&b->bar, sizeof(unsigned) * 2, "barrier");
     if (st == VGA_OK) st = dmalloc((void **)&b->err, sizeof(int32_t), "error flag");
@@ -506,6 +514,9 @@ vga_status vga_batch_create(const vga_graph *const *graphs, const vga_params *pa
         if (e == cudaSuccess) e = cudaMemsetAsync(b->table, 0, sizeof(uint32_t) * 3 * (size_t)b->npad, b->stream);
         if (e == cudaSuccess && !tinst.empty())
             e = cudaMemcpyAsync(b->tile_inst, tinst.data(), sizeof(int32_t) * tinst.size(), cudaMemcpyHostToDevice,
+                                b->stream);
+        if (e == cudaSuccess && !tinfo.empty())
+            e = cudaMemcpyAsync(b->tile_info, tinfo.data(), sizeof(ChunkInfo) * tinfo.size(), cudaMemcpyHostToDevice,
                                 b->stream);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(b->inst, hinst.data(), sizeof(BInst) * (size_t)count, cudaMemcpyHostToDevice, b->stream);

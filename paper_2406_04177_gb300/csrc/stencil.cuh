@@ -462,68 +462,6 @@ __device__ __forceinline__ void group_finish(uint32_t i0, uint32_t n, const Step
     }
 }
 
-// First half of the sparse fused pass (MODE 4, unit conductances, compensated state) for a full
-// group of four nodes, in packed pairs (0, 1) and (2, 3): the flux sum in slot order -x, +x, -y, +y,
-// -z, +z (an absent neighbour carries the node's own value, adding +0), Scheme 1's increment by
-// TwoSum, the rounding of vround, and the store of MODE 4 (a marked node's rounded pair itself, the
-// others renormalised as vstore).  Every lane does the scalar path's operations in its order, so the
-// results are the same bits.  REC: also writes h + l of the rounded pairs to rec_y2 (the adjoint's
-// record of the diffused DOM; at an unmarked node it is also the transformed DOM).
-template <bool REC = false>
-__device__ __forceinline__ void dom4_packed(uint32_t i0, const uint32_t (&ty)[4], const float (&y)[4], float yl,
-                                            float yr, const float (&ym)[4], const float (&yp)[4], const float (&zv)[4],
-                                            const float (&zw)[4], const V (&x2)[4], uint32_t act_bits,
-                                            const StepParams &p, const StateIO &io, float *rec_y2 = nullptr) {
-    float xm[4], xp[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        xm[k] = ((ty[k] >> 15) & 1u) ? (k == 0 ? yl : y[k > 0 ? k - 1 : 0]) : y[k];
-        xp[k] = (ty[k] >> 31) ? (k == 3 ? yr : y[k < 3 ? k + 1 : 0]) : y[k];
-    }
-    float hw[4], hr[4];
-    uint32_t qw[2];
-#pragma unroll
-    for (int h2 = 0; h2 < 2; ++h2) {
-        const int a = 2 * h2, b = a + 1;
-        const float2 Y = make_float2(y[a], y[b]);
-        float2 acc = make_float2(0.0f, 0.0f);
-        acc = add2_rn(acc, sub2_rn(Y, make_float2(xm[a], xm[b])));
-        acc = add2_rn(acc, sub2_rn(Y, make_float2(xp[a], xp[b])));
-        acc = add2_rn(acc, sub2_rn(Y, make_float2(ym[a], ym[b])));
-        acc = add2_rn(acc, sub2_rn(Y, make_float2(yp[a], yp[b])));
-        acc = add2_rn(acc, sub2_rn(Y, make_float2(zv[a], zv[b])));
-        acc = add2_rn(acc, sub2_rn(Y, make_float2(zw[a], zw[b])));
-        // Scheme 1: -D dt sum_j (y_i - y_j), in scalar (see add2_rn: a packed product would be fused)
-        const float2 d = make_float2(__fmul_rn(-p.c, acc.x), __fmul_rn(-p.c, acc.y));
-        float2 H = Y, L = make_float2(x2[a].l, x2[b].l);
-        // vadd: TwoSum, the rounding error into the residual
-        float2 s = add2_rn(H, d);
-        const float2 bp = sub2_rn(s, H);
-        const float2 e = add2_rn(sub2_rn(H, sub2_rn(s, bp)), sub2_rn(d, bp));
-        L = add2_rn(L, e);
-        H = s;
-        // vround: as if stored and loaded
-        s = add2_rn(H, L);
-        const float2 r = add2_rn(sub2_rn(H, s), L);
-        const uint32_t rq = bf16x2_bits(r.x, r.y);
-        L = make_float2(__uint_as_float(rq << 16), __uint_as_float(rq & 0xffff0000u));
-        H = s;
-        // store: renormalised (unmarked) or the rounded pair itself (marked)
-        const float2 hn = add2_rn(H, L);
-        const float2 rn = add2_rn(sub2_rn(H, hn), L);
-        const uint32_t qn = bf16x2_bits(rn.x, rn.y);
-        const bool ma = (act_bits >> a) & 1u, mb = (act_bits >> b) & 1u;
-        hw[a] = ma ? H.x : hn.x;
-        hw[b] = mb ? H.y : hn.y;
-        hr[a] = hn.x;
-        hr[b] = hn.y;
-        qw[h2] = ((ma ? rq : qn) & 0xffffu) | ((mb ? rq : qn) & 0xffff0000u);
-    }
-    st_floats<4>(io.out[1] + i0, hw);
-    *reinterpret_cast<uint2 *>(io.lout[1] + i0) = make_uint2(qw[0], qw[1]);
-    if (REC) st_floats<4>(rec_y2 + i0, hr);
-}
-
 // K consecutive nodes per thread (i0 a multiple of K, K = 2 or 4): table_node for nodes i0 ..
 // i0 + K - 1, the per-node streams (offset table, block ids, the five compartments) read and
 // written as 8- or 16-byte FP32 / table vectors and 4- or 8-byte residual vectors, so a warp moves
@@ -532,26 +470,18 @@ __device__ __forceinline__ void dom4_packed(uint32_t i0, const uint32_t (&ty)[4]
 // previous lane's last node and the +x neighbour of the last node the next lane's first node.
 // Arithmetic and slot order per node are those of table_node, so the results are the same bits.
 // Rows and tables start on 16-byte boundaries (row strides are multiples of 64 values).  REC: also
-// writes the pass record of the discrete adjoint (MODE 1: X and the transformed DOM; MODE 4: h + l of
-// every node's rounded DOM pair into rec.y2, which the second half overwrites at the marked nodes
-// with their transformed DOM).  MODE 4 is the first half of
-// the sparse fused pass: the DOM of every node is diffused and rounded as in MODE 1; a node whose
-// bit in the activity mask is clear has its DOM stored as MODE 1 stores a DOM that the (identity)
-// transformation left unchanged, a marked node the rounded pair itself (the second half, over the
-// marked nodes in rank order, reads it back exactly as MODE 1 holds it in registers).  Must be
-// called by all 32 lanes of a warp.
+// writes the pass record of the discrete adjoint (MODE 1: X and the transformed DOM).  Must be called
+// by all 32 lanes of a warp.
 template <int MODE, int WM, int TR, int PREC, int TF, int K, bool REC = false>
 __device__ __forceinline__ void table_vec(uint32_t i0, uint32_t n, const NbrTable &tb, const BlockTable &bt,
                                           const StepParams &p, const StateIO &io,
-                                          const PassRecord &rec = PassRecord{}, const SparseState &ss = SparseState{}) {
+                                          const PassRecord &rec = PassRecord{}) {
     const bool full = i0 + K <= n;
     const float *__restrict__ Y2 = io.in[1];
     uint32_t ty[K], zm[K], zp[K], bn[K];
     V x2[K];
     if (full) group_load<WM, PREC, TF, K, true>(i0, n, tb, bt, io, ty, zm, zp, bn, x2);
     else group_load<WM, PREC, TF, K, false>(i0, n, tb, bt, io, ty, zm, zp, bn, x2);
-    uint32_t act_bits = 0u;  // MODE 4: activity bits of the group
-    if (MODE == 4 && i0 < n) act_bits = (__ldg(ss.mask + (i0 >> 5)) >> (i0 & 31)) & ((1u << K) - 1u);
     float y[K];
 #pragma unroll
     for (int k = 0; k < K; ++k) y[k] = x2[k].h;
@@ -560,8 +490,7 @@ __device__ __forceinline__ void table_vec(uint32_t i0, uint32_t n, const NbrTabl
     float yr = __shfl_down_sync(0xffffffffu, y[0], 1);    // node i0 + K
     if (lane == 0 && ((ty[0] >> 15) & 1u)) yl = __ldg(Y2 + (i0 - 1));
     if (lane == 31 && (ty[K - 1] >> 31)) yr = __ldg(Y2 + (i0 + K));
-    // an absent neighbour reads the node's own value: the scalar path below skips it, the packed
-    // path adds y - y = +0, which leaves a sum that starts at +0 unchanged (it is never -0)
+    // an absent neighbour reads the node's own value (skipped below, or adding g * (+0))
     float ym[K], yp[K], zv[K], zw[K];
 #pragma unroll
     for (int k = 0; k < K; ++k) {
@@ -572,12 +501,6 @@ __device__ __forceinline__ void table_vec(uint32_t i0, uint32_t n, const NbrTabl
         zw[k] = zp[k] ? __ldg(Y2 + (i0 + k + zp[k])) : y[k];
     }
     if (i0 >= n) return;
-    if constexpr (MODE == 4 && WM == W_UNIT && PREC == P_COMP && K == 4) {
-        if (full) {
-            dom4_packed<REC>(i0, ty, y, yl, yr, ym, yp, zv, zw, x2, act_bits, p, io, rec.y2);
-            return;
-        }
-    }
 #pragma unroll
     for (int k = 0; k < K; ++k) {
         float acc = 0.0f;
@@ -597,38 +520,6 @@ __device__ __forceinline__ void table_vec(uint32_t i0, uint32_t n, const NbrTabl
             if (zp[k]) add(zw[k]);
         }
         vadd<PREC>(x2[k], __fmul_rn(-p.c, acc));  // Scheme 1
-    }
-    if (MODE == 4) {
-        float h[K], hr[K];
-        res_t q[K];
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            vround<PREC>(x2[k]);
-            hr[k] = __fadd_rn(x2[k].h, x2[k].l);  // REC: the adjoint's record of the rounded pair
-            if ((act_bits >> k) & 1u) {  // the rounded pair itself
-                h[k] = x2[k].h;
-                q[k] = PREC == P_COMP ? res_encode(x2[k].l, h[k]) : (res_t)0;
-            } else if (PREC == P_COMP) {  // renormalised as vstore does
-                h[k] = __fadd_rn(x2[k].h, x2[k].l);
-                q[k] = res_encode(__fadd_rn(__fsub_rn(x2[k].h, h[k]), x2[k].l), h[k]);
-            } else {
-                h[k] = x2[k].h;
-            }
-        }
-        if (full) {
-            st_floats<K>(io.out[1] + i0, h);
-            if (PREC == P_COMP) st_res<K>(io.lout[1] + i0, q);
-            if (REC) st_floats<K>(rec.y2 + i0, hr);
-        } else {
-#pragma unroll
-            for (int k = 0; k < K; ++k)
-                if (i0 + k < n) {
-                    io.out[1][i0 + k] = h[k];
-                    if (PREC == P_COMP) io.lout[1][i0 + k] = q[k];
-                    if (REC) rec.y2[i0 + k] = hr[k];
-                }
-        }
-        return;
     }
     if (full) group_finish<MODE, TR, PREC, K, true, REC>(i0, n, p, io, x2, rec);
     else group_finish<MODE, TR, PREC, K, false, REC>(i0, n, p, io, x2, rec);

@@ -20,7 +20,9 @@
 #include <cmath>
 #include <cstring>
 
+#include "pdl.cuh"
 #include "physics.cuh"
+#include "sparse_pass.cuh"
 #include "stencil.cuh"
 #include "tma.cuh"
 #include "vga_internal.cuh"
@@ -282,58 +284,30 @@ __global__ void __launch_bounds__(kThreads) k_stencil_table(int64_t n, NbrTable 
     table_node<MODE, WM, TR, PREC, LD_NC, TF>(i, i < (uint64_t)n, tb, bt, p, io);
 }
 
-// Programmatic dependent launch (PTX griddepcontrol, sm_90 and later). A grid launched with
-// programmatic stream serialisation may be scheduled while the kernel before it on the stream is
-// still running; pdl_wait, before the grid's first global access, holds it until that kernel has
-// completed and its writes are visible. For a grid launched without the attribute it returns at
-// once. pdl_trigger lets the next grid on the stream be scheduled once every block of this one has
-// issued it (its blocks then sit in their own pdl_wait).
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
-// Resident blocks per SM the compiler must fit: the DOM half of the sparse pass (MODE 4) is bound
-// by the latency of its gathers and fits 40 registers (6 blocks) without spills, except with block
-// conductances (5).
-template <int MODE, int WM>
-constexpr int tablev_min_blocks() {
-    return MODE == 4 ? (WM == W_UNIT ? 6 : 5) : 4;
-}
-
 // K consecutive nodes per thread (table_vec); n < 2^31, so K * thread index fits 32 bits.
 template <int MODE, int WM, int TR, int PREC, int TF, int K>
-__global__ void __launch_bounds__(kThreads, tablev_min_blocks<MODE, WM>()) k_stencil_tablev(int64_t n, NbrTable tb, BlockTable bt, StepParams p,
-                                                             StateIO io, SparseState ss) {
-    if constexpr (MODE == 1 || MODE == 4) {
+__global__ void __launch_bounds__(kThreads, 4) k_stencil_tablev(int64_t n, NbrTable tb, BlockTable bt, StepParams p,
+                                                             StateIO io) {
+    if constexpr (MODE == 1) {
         pdl_wait();
         pdl_trigger();
     }
     const uint32_t i0 = (uint32_t)K * ((uint32_t)blockIdx.x * blockDim.x + threadIdx.x);
-    table_vec<MODE, WM, TR, PREC, TF, K>(i0, (uint32_t)n, tb, bt, p, io, PassRecord{}, ss);
+    table_vec<MODE, WM, TR, PREC, TF, K>(i0, (uint32_t)n, tb, bt, p, io);
 }
 
-// Second half of the two-kernel sparse pass: one thread per marked node, in rank order, with its
-// MB, SOM, FOM, CO2 from the compact state (updated in place) and its DOM as the first half stored it
-// (the rounded pair); stores the DOM as MODE 1 does.
-template <int TR, int PREC>
-__global__ void __launch_bounds__(kThreads) k_transform_compact(int64_t m, SparseState ss, StepParams p, StateIO io) {
+// One sparse fused pass (sparse_pass.cuh).  40 registers, so that 6 blocks are resident per SM, fit
+// without spills, except with block conductances (48, 5 blocks).
+template <int WM, int TR, int PREC, int TF, bool AHEAD>
+__global__ void __launch_bounds__(kSparseThreads, WM == W_UNIT ? 6 : 5)
+    k_sparse_pass(int64_t n, NbrTable tb, BlockTable bt, StepParams p, StateIO io, SparseState ss, int ahead) {
+    __shared__ SparseShared sm;
     pdl_wait();
     pdl_trigger();
-    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= m) return;
-    const uint32_t i = __ldg(ss.list + r);
-    V x2;
-    x2.h = io.out[1][i];
-    x2.l = PREC == P_COMP ? res_decode(io.lout[1][i], x2.h) : 0.0f;
-    V v[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        v[q].h = ss.h[q][r];
-        v[q].l = PREC == P_COMP ? res_decode(ss.l[q][r], v[q].h) : 0.0f;
-    }
-    transform_n<TR, PREC>(v[0], x2, v[1], v[2], v[3], p);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) vstore<PREC>(ss.h[q], ss.l[q], r, v[q]);
-    vstore<PREC>(io.out[1], io.lout[1], i, x2);
+    const uint32_t blk = AHEAD && ahead < 0 ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
+    sparse_pass_block<WM, TR, PREC, TF, false, AHEAD>(sm, blk * kSparseNodes, (uint32_t)n, (n + 31) >> 5, p.c, tb, bt, io,
+                                                      ss, SparseRecord{}, ahead,
+                                                      [&](uint32_t) -> const StepParams & { return p; });
 }
 
 // Node of each rank (once per state upload, after the prefix).
@@ -639,63 +613,36 @@ void launch_staged_any(vga_sim *s, const StateIO &io) {
 // The compact state of the running step call.
 SparseState sparse_state(vga_sim *s) { return activity_state(s->act); }
 
-// Launch with programmatic stream serialisation: the grid may be scheduled during the tail of the
-// kernel before it on the stream and waits for it in pdl_wait (the kernel must call it first).
-template <typename... KArgs, typename... Args>
-void launch_pdl(void (*kernel)(KArgs...), unsigned grid, cudaStream_t stream, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, kernel, args...);
-}
-
-template <int MODE, int WM, int PREC, int K>
-void launch_tablev_m(vga_sim *s, const StateIO &io, const NbrTable &tb, const BlockTable &bt) {
+template <int MODE, int WM, int TR, int PREC, int TF, int K>
+void launch_tablev_k(vga_sim *s, const StateIO &io, const NbrTable &tb, const BlockTable &bt) {
     const unsigned grid = grid_for((s->n + K - 1) / K, kThreads);
-    const SparseState act = sparse_state(s);
-    if constexpr (MODE == 1 || MODE == 4) {
-        if (tb.tz) {
-            if (s->sp.transform == 0) launch_pdl(k_stencil_tablev<MODE, WM, 0, PREC, 1, K>, grid, s->stream, s->n, tb, bt, s->sp, io, act);
-            else launch_pdl(k_stencil_tablev<MODE, WM, 1, PREC, 1, K>, grid, s->stream, s->n, tb, bt, s->sp, io, act);
-        } else {
-            if (s->sp.transform == 0) launch_pdl(k_stencil_tablev<MODE, WM, 0, PREC, 0, K>, grid, s->stream, s->n, tb, bt, s->sp, io, act);
-            else launch_pdl(k_stencil_tablev<MODE, WM, 1, PREC, 0, K>, grid, s->stream, s->n, tb, bt, s->sp, io, act);
-        }
-        return;
-    }
-    if (tb.tz) {
-        if (s->sp.transform == 0) k_stencil_tablev<MODE, WM, 0, PREC, 1, K><<<grid, kThreads, 0, s->stream>>>(s->n, tb, bt, s->sp, io, act);
-        else k_stencil_tablev<MODE, WM, 1, PREC, 1, K><<<grid, kThreads, 0, s->stream>>>(s->n, tb, bt, s->sp, io, act);
-    } else {
-        if (s->sp.transform == 0) k_stencil_tablev<MODE, WM, 0, PREC, 0, K><<<grid, kThreads, 0, s->stream>>>(s->n, tb, bt, s->sp, io, act);
-        else k_stencil_tablev<MODE, WM, 1, PREC, 0, K><<<grid, kThreads, 0, s->stream>>>(s->n, tb, bt, s->sp, io, act);
-    }
+    if (MODE == 1) launch_pdl(k_stencil_tablev<MODE, WM, TR, PREC, TF, K>, grid, kThreads, s->stream, s->n, tb, bt, s->sp, io);
+    else k_stencil_tablev<MODE, WM, TR, PREC, TF, K><<<grid, kThreads, 0, s->stream>>>(s->n, tb, bt, s->sp, io);
 }
 
-// Fused passes of the four-node kernel run sparse inside a sparse step call: the DOM of every node
-// (MODE 4), then the transformation of the marked nodes in rank order.
+// Fused passes of the four-node kernel run sparse inside a sparse step call.
+template <int MODE, int WM, int TR, int PREC, int TF, int K>
+void launch_tablev_t(vga_sim *s, const StateIO &io, const NbrTable &tb, const BlockTable &bt) {
+    if constexpr (MODE == 1 && K == 4) {
+        if (s->sparse_call) {
+            launch_pdl(sparse_streams(s->n) ? k_sparse_pass<WM, TR, PREC, TF, true> : k_sparse_pass<WM, TR, PREC, TF, false>,
+                       grid_for(s->n, kSparseNodes), kSparseThreads, s->stream, s->n, tb, bt, s->sp, io, sparse_state(s),
+                       sparse_ahead(s->cur[1]));
+            return;
+        }
+    }
+    launch_tablev_k<MODE, WM, TR, PREC, TF, K>(s, io, tb, bt);
+}
+
 template <int MODE, int WM, int PREC, int K>
 void launch_tablev(vga_sim *s, const StateIO &io, const NbrTable &tb, const BlockTable &bt) {
-    if (MODE == 1 && K == 4 && s->sparse_call) {
-        launch_tablev_m<4, WM, PREC, K>(s, io, tb, bt);
-        const int64_t m = s->act.n_active;
-        if (m > 0) {
-            const unsigned g = grid_for(m, kThreads);
-            const SparseState ss = activity_state(s->act);
-            if (s->sp.transform == 0) launch_pdl(k_transform_compact<0, PREC>, g, s->stream, m, ss, s->sp, io);
-            else launch_pdl(k_transform_compact<1, PREC>, g, s->stream, m, ss, s->sp, io);
-            ++s->launches;
-        }
-        return;
+    if (tb.tz) {
+        if (s->sp.transform == 0) launch_tablev_t<MODE, WM, 0, PREC, 1, K>(s, io, tb, bt);
+        else launch_tablev_t<MODE, WM, 1, PREC, 1, K>(s, io, tb, bt);
+    } else {
+        if (s->sp.transform == 0) launch_tablev_t<MODE, WM, 0, PREC, 0, K>(s, io, tb, bt);
+        else launch_tablev_t<MODE, WM, 1, PREC, 0, K>(s, io, tb, bt);
     }
-    launch_tablev_m<MODE, WM, PREC, K>(s, io, tb, bt);
 }
 
 template <int MODE, int WM, int PREC>
