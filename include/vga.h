@@ -355,9 +355,9 @@ vga_status vga_sim_autotune(vga_sim *s, int32_t trial_steps, vga_tune_result *ou
 
 /* ============================================================================================
  * Batched simulation: many independent graphs (uneven node counts, per-instance parameters)
- * advanced together by one persistent cooperative kernel per launch, several time steps per
- * launch with a bounded grid-wide barrier between passes, the launches of one call captured in a
- * CUDA graph and replayed.  Explicit scheme only; all instances share transform and
+ * advanced together, by default one launch per time step (64 of them replayed as a CUDA graph), or by
+ * persistent cooperative launches of several time steps with a bounded grid-wide barrier between
+ * passes, the launches of one call captured in a CUDA graph and replayed (vga_batch_set_launch).  Explicit scheme only; all instances share transform and
  * state_precision.  Results are bit-identical to vga_sim on each graph.
  * ============================================================================================ */
 typedef struct vga_batch vga_batch;
@@ -375,7 +375,8 @@ vga_status vga_batch_get_masses(vga_batch *b, int32_t instance, double *x);
 /* Advances every instance n_steps; returns when done.  VGA_ERR_TIMEOUT if a barrier gave up. */
 vga_status vga_batch_step(vga_batch *b, int64_t n_steps);
 /* Launch shape: time steps per persistent launch, resident blocks per SM (0 = occupancy maximum),
- * CUDA-graph capture on or off. */
+ * CUDA-graph capture on or off.  (1, 0), the initial shape: every sparse fused pass is a launch of its
+ * own, without barriers; dense passes then take persistent launches of 100. */
 vga_status vga_batch_set_launch(vga_batch *b, int32_t steps_per_launch, int32_t blocks_per_sm, int32_t use_graph);
 
 /* Sparse fused passes for the batch, as vga_sim_set_activity_skip (on by default): the first step

@@ -1,16 +1,17 @@
-// Batched simulation of many independent subvolumes (uneven node counts, per-instance parameters)
-// in one persistent kernel per launch.
+// Batched simulation of many independent subvolumes (uneven node counts, per-instance parameters),
+// all advanced by the same launches.
 //
 // Layout: the instances' nodes are concatenated, each instance starting at a multiple of 256 nodes
 // (kTile), so a 256-node tile never straddles two instances and carries one instance id.  Every
 // instance keeps its own neighbour-offset table (offsets are relative, so they remain valid in the
 // concatenated index space) and its own StepParams.
 //
-// A launch runs passes [pass0, pass1) of a step() call of N time steps (N + 1 passes: one
-// transformation-only pass, N - 1 fused passes, one diffusion-only pass; see step.cu).  Passes are
-// separated by a grid-wide barrier; the launch is cooperative, so every block is resident, and
-// every wait in the barrier is bounded (VGA_ERR_TIMEOUT instead of a hang).  The launches of a
-// step() call are captured once into a CUDA graph and replayed.
+// A step() call of N time steps is N + 1 passes: one transformation-only pass, N - 1 fused passes, one
+// diffusion-only pass (see step.cu).  By default a sparse fused pass is a launch of its own, 64 of them
+// a CUDA graph.  In the persistent form (vga_batch_set_launch, dense passes) a launch runs passes
+// [pass0, pass1): passes are separated by a grid-wide barrier; the launch is cooperative, so every
+// block is resident, and every wait in the barrier is bounded (VGA_ERR_TIMEOUT instead of a hang).
+// Its launches of a step() call are captured once into a CUDA graph and replayed.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -19,6 +20,7 @@
 #include <vector>
 
 #include "grid_sync.cuh"
+#include "pdl.cuh"
 #include "physics.cuh"
 #include "sparse_pass.cuh"
 #include "stencil.cuh"
@@ -93,20 +95,40 @@ __device__ __forceinline__ void batch_fused_pass(const BatchArgs &a, const State
     }
 }
 
-// The sparse fused pass (sparse_pass.cuh) over the whole batch: the 128 nodes of a warp lie in one tile,
-// hence in one instance.
+// The sparse fused pass (sparse_pass.cuh) of the batch over the nodes v0 .. v0 + 1023: the 128 nodes of a
+// warp lie in one tile, hence in one instance.
+template <int TR, int PREC, int TF, bool AHEAD>
+__device__ __forceinline__ void batch_sparse_block(SparseShared &sm, const BatchArgs &a, const StateIO &io, int64_t v0,
+                                                   int ahead) {
+    const int64_t tile = (v0 + 4 * threadIdx.x) / kTile;
+    const ChunkInfo ci = tile < a.ntiles ? __ldg_chunk(a.tile_info + tile) : ChunkInfo{0.0f, 0u};
+    sparse_pass_block<W_UNIT, TR, PREC, TF, false, AHEAD>(
+        sm, (uint32_t)v0, ci.end, a.ntiles * (kTile / 32), ci.c, a.tb, BlockTable{}, io, a.ss, SparseRecord{}, ahead,
+        [&](uint32_t i) -> const StepParams & { return a.inst[__ldg(a.tile_inst + i / kTile)].p; });
+}
+
 template <int TR, int PREC, int TF>
 __device__ __forceinline__ void batch_sparse_pass(const BatchArgs &a, const StateIO &io) {
     __shared__ SparseShared sm;
-    const int64_t nsuper = (a.ntiles + 3) / 4, words = a.ntiles * (kTile / 32);
+    const int64_t nsuper = (a.ntiles * kTile + kSparseNodes - 1) / kSparseNodes;
     for (int64_t s = blockIdx.x; s < nsuper; s += gridDim.x) {
-        const int64_t v0 = s * kSparseNodes, tile = (v0 + 4 * threadIdx.x) / kTile;
-        const ChunkInfo ci = tile < a.ntiles ? __ldg_chunk(a.tile_info + tile) : ChunkInfo{0.0f, 0u};
-        sparse_pass_block<W_UNIT, TR, PREC, TF, false, false>(
-            sm, (uint32_t)v0, ci.end, words, ci.c, a.tb, BlockTable{}, io, a.ss, SparseRecord{}, 0,
-            [&](uint32_t i) -> const StepParams & { return a.inst[__ldg(a.tile_inst + i / kTile)].p; });
+        batch_sparse_block<TR, PREC, TF, false>(sm, a, io, s * kSparseNodes, 0);
         __syncthreads();  // the next turn reuses the shared pairs
     }
+}
+
+// One sparse fused pass as a launch of its own (the default launch shape): 1024 nodes per block, no
+// grid barrier, scheduled in the tail of the pass before it (programmatic dependent launch).  The
+// persistent form below keeps every block for the whole launch and makes it wait at a grid barrier
+// after every pass.  Per pass: 12 subvolumes, 8.2 M nodes: 33.7 us (persistent 46.4); 40
+// subvolumes, 24.5 M nodes: 97 us (126); 6 subvolumes, 0.53 M nodes: 4.7 us (6.5).
+template <int TR, int PREC, int TF, bool AHEAD>
+__global__ void __launch_bounds__(kSparseThreads, 6) k_batch_sparse_pass(BatchArgs a, int bi, int ahead) {
+    __shared__ SparseShared sm;
+    pdl_wait();
+    pdl_trigger();
+    const int64_t blk = AHEAD && ahead < 0 ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
+    batch_sparse_block<TR, PREC, TF, AHEAD>(sm, a, a.io[bi], blk * kSparseNodes, ahead);
 }
 
 // FUSED_ONLY: an instantiation for launches whose passes are all fused ones (every launch but the
@@ -257,7 +279,7 @@ struct vga_batch {
     int grid_edge = 0;     // blocks of a launch of the first or the last pass
     int grid_sparse = 0;   // blocks of a sparse fused-only launch
     int blocks_per_sm = 0;  // tuning knob (0: the occupancy maximum)
-    int steps_per_launch = 100;
+    int steps_per_launch = 1;
     bool use_graph = true;
     bool capture_failed = false;
     std::map<std::tuple<int64_t, int, int, int>, cudaGraphExec_t> graphs;
@@ -308,7 +330,7 @@ vga_status batch_grid(vga_batch *b) {
     return batch_grid_of(b, b->tz ? batch_kernel<1, true, false>(b) : batch_kernel<0, true, false>(b), &b->grid);
 }
 
-vga_status launch_batch(vga_batch *b, int32_t pass0, int32_t pass1, int32_t npass, int32_t cur0, bool sparse) {
+BatchArgs batch_args(const vga_batch *b) {
     BatchArgs a;
     a.ntiles = b->ntiles;
     a.npad = b->npad;
@@ -336,6 +358,11 @@ vga_status launch_batch(vga_batch *b, int32_t pass0, int32_t pass1, int32_t npas
             a.io[k].lout[c] = b->l[1 - k] + c * b->npad;
         }
     }
+    return a;
+}
+
+vga_status launch_batch(vga_batch *b, int32_t pass0, int32_t pass1, int32_t npass, int32_t cur0, bool sparse) {
+    const BatchArgs a = batch_args(b);
     // the first and the last pass of a call need the full kernel; the others run the fused-only one
     const bool fused_only = pass0 > 0 && pass1 < npass;
     cudaLaunchConfig_t cfg = {};
@@ -362,10 +389,52 @@ vga_status launch_batch(vga_batch *b, int32_t pass0, int32_t pass1, int32_t npas
     return VGA_OK;
 }
 
+// One sparse fused pass, reading state buffer bi.
+template <int TR, int PREC>
+void launch_sparse_pass_t(const vga_batch *b, const BatchArgs &a, int bi, cudaStream_t st) {
+    const bool str = sparse_streams(b->total);
+    auto kern = b->tz ? (str ? k_batch_sparse_pass<TR, PREC, 1, true> : k_batch_sparse_pass<TR, PREC, 1, false>)
+                      : (str ? k_batch_sparse_pass<TR, PREC, 0, true> : k_batch_sparse_pass<TR, PREC, 0, false>);
+    launch_pdl(kern, (unsigned)((b->total + kSparseNodes - 1) / kSparseNodes), kSparseThreads, st, a, bi, sparse_ahead(bi));
+}
+
+vga_status launch_sparse_passes(const vga_batch *b, int64_t passes, int bi, cudaStream_t st) {
+    const BatchArgs a = batch_args(b);
+    for (int64_t k = 0; k < passes; ++k, bi ^= 1) {
+        if (b->transform == 0) {
+            if (b->precision == P_COMP) launch_sparse_pass_t<0, P_COMP>(b, a, bi, st);
+            else launch_sparse_pass_t<0, P_F32>(b, a, bi, st);
+        } else {
+            if (b->precision == P_COMP) launch_sparse_pass_t<1, P_COMP>(b, a, bi, st);
+            else launch_sparse_pass_t<1, P_F32>(b, a, bi, st);
+        }
+    }
+    VGA_CHECK_LAUNCH();
+    return VGA_OK;
+}
+
+// Launch shape "one step per launch on as many blocks as there are": sparse fused passes are launches
+// of their own (k_batch_sparse_pass).  The test of the bounded waits needs the persistent form.
+bool per_pass(const vga_batch *b, bool sparse) {
+    return sparse && b->steps_per_launch == 1 && b->blocks_per_sm == 0 && b->wait_test_block < 0;
+}
+
+// Blocks of a launch of fused passes.
+int step_grid(const vga_batch *b) {
+    if (per_pass(b, b->activity_skip)) return (int)((b->total + kSparseNodes - 1) / kSparseNodes);
+    return b->activity_skip ? b->grid_sparse : b->grid;
+}
+
+// Time steps per persistent launch: the shape that asks for a launch per pass (1, 0) gets launches of
+// 100 passes where the persistent form runs (dense passes, the test of the bounded waits).
+int persistent_steps(const vga_batch *b) {
+    return b->steps_per_launch == 1 && b->blocks_per_sm == 0 ? 100 : std::max(1, b->steps_per_launch);
+}
+
 // Launches of one call: the first pass alone, the fused passes in launches of steps_per_launch
 // passes, the last pass alone.
-int64_t launches_of(const vga_batch *b, int64_t n_steps) {
-    const int64_t S = std::max(1, b->steps_per_launch), mid = n_steps - 1;
+int64_t launches_of(const vga_batch *b, int64_t n_steps, bool sparse) {
+    const int64_t S = per_pass(b, sparse) ? 1 : persistent_steps(b), mid = n_steps - 1;
     return 2 + (mid > 0 ? (mid + S - 1) / S : 0);
 }
 
@@ -385,7 +454,7 @@ StateIO batch_io(const vga_batch *b, int k) {
 // after the first pass and back before the last.
 vga_status enqueue_steps(vga_batch *b, int64_t n_steps, int cur0, bool sparse) {
     const int64_t npass = n_steps + 1;
-    const int S = std::max(1, b->steps_per_launch);
+    const int S = persistent_steps(b);
     const bool comp = b->precision == P_COMP;
     VGA_TRY(launch_batch(b, 0, 1, (int32_t)npass, cur0, false));
     if (sparse) VGA_TRY(activity_copy(b->act, b->total, batch_io(b, (cur0 + 1) & 1), true, comp, b->stream));
@@ -397,6 +466,51 @@ vga_status enqueue_steps(vga_batch *b, int64_t n_steps, int cur0, bool sparse) {
     if (sparse)
         VGA_TRY(activity_copy(b->act, b->total, batch_io(b, 1 - (int)((cur0 + npass - 1) & 1)), false, comp, b->stream));
     return launch_batch(b, (int32_t)(npass - 1), (int32_t)npass, (int32_t)npass, cur0, false);
+}
+
+// A call in per-pass launches: the fused passes as replays of one graph of kPassGraph passes (an even
+// number, so every replay reads the same buffer), the others launched directly.  A graph of the whole
+// call would have to be captured again for every number of steps.
+constexpr int64_t kPassGraph = 64;
+
+vga_status step_per_pass(vga_batch *b, int64_t n_steps, int cur0) {
+    const bool comp = b->precision == P_COMP;
+    const int32_t npass = (int32_t)(n_steps + 1);
+    VGA_TRY(launch_batch(b, 0, 1, npass, cur0, false));
+    int bi = (cur0 + 1) & 1;
+    VGA_TRY(activity_copy(b->act, b->total, batch_io(b, bi), true, comp, b->stream));
+    int64_t left = n_steps - 1;
+    if (b->use_graph && left >= 2 * kPassGraph) {
+        const auto key = std::make_tuple((int64_t)-1, 1, 0, bi);
+        auto it = b->graphs.find(key);
+        if (it == b->graphs.end()) {
+            cudaGraph_t graph = nullptr;
+            cudaGraphExec_t exec = nullptr;
+            VGA_CUDA(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
+            const vga_status st = launch_sparse_passes(b, kPassGraph, bi, b->stream);
+            const cudaError_t ec = cudaStreamEndCapture(b->stream, &graph);
+            cudaError_t ei = cudaErrorUnknown;
+            if (st == VGA_OK && ec == cudaSuccess) ei = cudaGraphInstantiate(&exec, graph, 0);
+            if (graph) cudaGraphDestroy(graph);
+            if (st == VGA_OK && ec == cudaSuccess && ei == cudaSuccess) {
+                it = b->graphs.emplace(key, exec).first;
+            } else {  // the passes are launched directly from now on
+                cudaGetLastError();
+                b->use_graph = false;
+                b->capture_failed = true;
+            }
+        }
+        if (it != b->graphs.end()) {
+            for (; left >= kPassGraph; left -= kPassGraph) {
+                VGA_CUDA(cudaGraphLaunch(it->second, b->stream));
+                ++b->graph_replays;
+            }
+        }
+    }
+    VGA_TRY(launch_sparse_passes(b, left, bi, b->stream));
+    // the state after pass npass - 2 is buffer (cur0 + npass - 1) & 1: the out side of the other
+    VGA_TRY(activity_copy(b->act, b->total, batch_io(b, 1 - (int)((cur0 + npass - 1) & 1)), false, comp, b->stream));
+    return launch_batch(b, npass - 1, npass, npass, cur0, false);
 }
 
 vga_status check_err(vga_batch *b) {
@@ -633,7 +747,9 @@ vga_status vga_batch_step(vga_batch *b, int64_t n_steps) {
                                b->stream));
         drop_graphs(b);
     }
-    if (b->use_graph) {
+    if (per_pass(b, sparse)) {
+        VGA_TRY(step_per_pass(b, n_steps, cur0));
+    } else if (b->use_graph) {
         const auto key = std::make_tuple(n_steps, b->steps_per_launch, b->grid, cur0 + (sparse ? 2 : 0));
         auto it = b->graphs.find(key);
         if (it == b->graphs.end()) {
@@ -663,7 +779,7 @@ vga_status vga_batch_step(vga_batch *b, int64_t n_steps) {
     } else {
         VGA_TRY(enqueue_steps(b, n_steps, cur0, sparse));
     }
-    b->launches += launches_of(b, n_steps);
+    b->launches += launches_of(b, n_steps, sparse);
     b->cur = (int)((cur0 + n_steps + 1) & 1);
     b->steps_done += n_steps;
     return check_err(b);
@@ -674,7 +790,7 @@ vga_status vga_batch_get_stats(const vga_batch *b, vga_batch_stats *out) {
     out->instances = b->count;
     out->total_nodes = 0;
     for (int64_t v : b->nodes) out->total_nodes += v;
-    out->grid_blocks = b->activity_skip ? b->grid_sparse : b->grid;
+    out->grid_blocks = step_grid(b);
     out->steps_per_launch = b->steps_per_launch;
     out->kernel_launches = b->launches;
     out->graph_replays = b->graph_replays;
@@ -685,8 +801,8 @@ vga_status vga_batch_get_stats(const vga_batch *b, vga_batch_stats *out) {
 
 vga_status vga_batch_autotune(vga_batch *b, int32_t trial_steps, vga_batch_tune *out) {
     if (!b || !out || trial_steps < 2) return fail(VGA_ERR_INVALID_ARG, "bad batch, out or trial_steps");
-    static const int kSteps[] = {25, 100, 400};
-    static const int kBlocks[] = {0, 4, 2};
+    // one launch per pass, then persistent launches
+    static const int kShapes[][2] = {{1, 0}, {25, 0}, {25, 4}, {100, 0}, {100, 4}, {100, 2}, {400, 0}, {400, 4}, {400, 2}};
     const int keep_s = b->steps_per_launch, keep_b = b->blocks_per_sm;
     // save the state (both buffers' current side) so the trials leave it untouched
     float *h = nullptr;
@@ -705,29 +821,27 @@ vga_status vga_batch_autotune(vga_batch *b, int32_t trial_steps, vga_batch_tune 
     out->count = 0;
     out->best = -1;
     double best = 1e300;
-    for (int si = 0; si < 3 && st == VGA_OK; ++si) {
-        for (int bi = 0; bi < 3 && st == VGA_OK; ++bi) {
-            if (out->count >= VGA_TUNE_MAX) break;
-            st = vga_batch_set_launch(b, kSteps[si], kBlocks[bi], 1);
-            if (st == VGA_OK) st = vga_batch_step(b, trial_steps);  // capture + warm-up
-            cudaEventRecord(e0, b->stream);
-            if (st == VGA_OK) st = vga_batch_step(b, trial_steps);
-            cudaEventRecord(e1, b->stream);
-            cudaEventSynchronize(e1);
-            float ms = 0.0f;
-            cudaEventElapsedTime(&ms, e0, e1);
-            if (st != VGA_OK) break;
-            vga_batch_tune_entry &en = out->entries[out->count];
-            en.steps_per_launch = kSteps[si];
-            en.blocks_per_sm = kBlocks[bi];
-            en.grid_blocks = b->activity_skip ? b->grid_sparse : b->grid;
-            en.ms_per_step = ms / trial_steps;
-            if (ms < best) {
-                best = ms;
-                out->best = out->count;
-            }
-            ++out->count;
+    for (const auto &sh : kShapes) {
+        if (st != VGA_OK) break;
+        st = vga_batch_set_launch(b, sh[0], sh[1], 1);
+        if (st == VGA_OK) st = vga_batch_step(b, trial_steps);  // capture + warm-up
+        cudaEventRecord(e0, b->stream);
+        if (st == VGA_OK) st = vga_batch_step(b, trial_steps);
+        cudaEventRecord(e1, b->stream);
+        cudaEventSynchronize(e1);
+        float ms = 0.0f;
+        cudaEventElapsedTime(&ms, e0, e1);
+        if (st != VGA_OK) break;
+        vga_batch_tune_entry &en = out->entries[out->count];
+        en.steps_per_launch = sh[0];
+        en.blocks_per_sm = sh[1];
+        en.grid_blocks = step_grid(b);
+        en.ms_per_step = ms / trial_steps;
+        if (ms < best) {
+            best = ms;
+            out->best = out->count;
         }
+        ++out->count;
     }
     if (st == VGA_OK && out->best >= 0)
         st = vga_batch_set_launch(b, out->entries[out->best].steps_per_launch, out->entries[out->best].blocks_per_sm, 1);
