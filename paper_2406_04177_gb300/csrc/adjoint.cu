@@ -22,8 +22,10 @@
 #include <cmath>
 #include <vector>
 
+#include "adjoint_sums.cuh"
 #include "pdl.cuh"
 #include "physics.cuh"
+#include "small_graph.cuh"
 #include "sparse_pass.cuh"
 #include "stencil.cuh"
 #include "vga_internal.cuh"
@@ -199,44 +201,6 @@ __global__ void __launch_bounds__(kSparseThreads, 5)
                                                     ss, rec, ahead, [&](uint32_t) -> const StepParams & { return p; });
 }
 
-// Compensated FP32 accumulator (TwoSum into a second float): GB300 issues FP64 at a small fraction of
-// its FP32 rate, and a per-thread sum of ~100 terms carried this way keeps ~45 significant bits.
-struct CAcc {
-    float s = 0.0f, c = 0.0f;
-};
-
-__device__ __forceinline__ void cacc_add(CAcc &a, float x) {
-    const float t = __fadd_rn(a.s, x);
-    const float bp = __fsub_rn(t, a.s);
-    const float err = __fadd_rn(__fsub_rn(a.s, __fsub_rn(t, bp)), __fsub_rn(x, bp));
-    a.s = t;
-    a.c = __fadd_rn(a.c, err);
-}
-
-// x * y added exactly (TwoProd by FMA: the product's rounding error is a second float).
-__device__ __forceinline__ void cacc_add_prod(CAcc &a, float x, float y) {
-    const float p = __fmul_rn(x, y);
-    const float e = __fmaf_rn(x, y, -p);
-    cacc_add(a, p);
-    a.c = __fadd_rn(a.c, e);
-}
-
-// FP32 value as FP64, built with integer operations: exact for normal values, infinities and NaN;
-// subnormal values (below 2^-126 in magnitude) become zeros of their sign.  The conversion
-// instruction would issue on the FP64 pipe, which GB300 runs at a small fraction of its FP32 rate.
-__device__ __forceinline__ double f32_to_f64_alu(float f) {
-    const uint32_t u = __float_as_uint(f);
-    const uint32_t e = (u >> 23) & 0xffu;
-    const uint32_t sign = u & 0x80000000u;
-    uint32_t hi = sign, lo = 0u;
-    if (e != 0u) {
-        const uint32_t ed = e == 0xffu ? 0x7ffu : e + 896u;  // rebias 127 -> 1023
-        hi = sign | (ed << 20) | ((u & 0x7fffffu) >> 3);
-        lo = u << 29;
-    }
-    return __hiloint2double((int)hi, (int)lo);
-}
-
 // Block sums of K compensated per-thread accumulators into out[0..K) (FP64, by thread 0 .. K-1): a
 // warp butterfly of the (sum, error) pairs in FP32, merged by TwoSum at each level, then one FP64
 // conversion per value and warp and the warps' sums in FP64.  The FP64 work is a few instructions
@@ -270,39 +234,6 @@ __device__ __forceinline__ void block_sum_cacc(const CAcc (&a)[K], double *out) 
         out[threadIdx.x] = b;
     }
     __syncthreads();
-}
-
-// Adds v to gtheta[f] when f >= 0: one FP64 atomic per crossing edge.  At the porosities of the
-// workloads a block face carries a few edges per step, spread over rows far apart in node order, so
-// lanes of one warp rarely share a face and a warp-level pre-reduction would cost more instructions
-// than it saves atomics.  The FP64 sums of FP32 terms are exact while the terms of a face span fewer
-// than 29 binary orders, so the result does not depend on the atomics' order there.
-__device__ __forceinline__ void face_atomic_add_f(double *gtheta, int32_t f, float v) {
-    if (f >= 0) atomicAdd(gtheta + f, f32_to_f64_alu(v));
-}
-
-// transform_sync_reverse at an unmarked node, x = (0, y, 0, 0, .) with +0, without the operations whose
-// results are known there: every flux is zero, the mortality and turnover branches are the free ones, and
-// dL/dx2 gets a term only when the uptake is clamped (y < 0).  A sum that starts at +0 and gets one
-// product keeps the product's value (0 + t), as there.  The same bits for finite values.
-template <int PREC>
-__device__ __forceinline__ void reverse_unmarked(float y, const V (&mu)[5], V (&lam)[5], const StepParams &p) {
-    const float sat = __fdividef(y, __fadd_rn(p.K, y));
-    const float w_upt = __fsub_rn(mu[0].h, mu[1].h);
-    const float w_mor = __fadd_rn(__fadd_rn(-mu[0].h, __fmul_rn(p.beta, mu[1].h)), __fmul_rn(p.omb, mu[2].h));
-    const float w_resp = __fsub_rn(mu[4].h, mu[0].h);
-    const bool clamped = 0.0f > y;
-    const float du = clamped ? 0.0f : __fadd_rn(0.0f, __fmul_rn(w_upt, __fmul_rn(p.a, sat)));
-    const float d1 = clamped ? __fadd_rn(0.0f, w_upt) : 0.0f;
-    const float d0 = __fadd_rn(du, __fadd_rn(__fmul_rn(w_mor, p.m), __fmul_rn(w_resp, p.r)));
-    const float d3 = __fadd_rn(0.0f, __fmul_rn(__fsub_rn(mu[1].h, mu[3].h), p.f));
-    const float d2 = __fadd_rn(0.0f, __fmul_rn(__fsub_rn(mu[1].h, mu[2].h), p.s));
-#pragma unroll
-    for (int c = 0; c < 5; ++c) lam[c] = mu[c];
-    vadd<PREC>(lam[0], d0);
-    vadd<PREC>(lam[1], d1);
-    vadd<PREC>(lam[2], d2);
-    vadd<PREC>(lam[3], d3);
 }
 
 // Reverse step with four consecutive nodes per thread: the per-node streams (offset table, block
@@ -519,7 +450,7 @@ __global__ void __launch_bounds__(kThreads, VGA_ADJ_MIN_BLOCKS) k_adjoint_vec(in
 // Neither the grid nor the node of a thread changes, so the sums are the same bits on every run.
 constexpr int kLeanK = 2;  // consecutive nodes per thread: 2 at 5 blocks per SM 250 us per step, 4 at 3 blocks 285 (512^3)
 
-constexpr int64_t kLeanNodes = (int64_t)1 << 19;  // graphs from this size (measured in sim_adjoint_backward)
+constexpr int64_t kLeanNodes = (int64_t)1 << 19;  // graphs from this size (measured in adjoint_backward_impl)
 
 struct LeanArgs {
     const float *y2k;     // transformed DOM of the step
@@ -900,7 +831,7 @@ struct AdjointBuffers {
     int64_t rec_xc_count = 0, xcap = 1;
     PairBuf work[2];
     PairBuf lam[2];
-    double *gpart = nullptr;  // G x kPar
+    double *gpart = nullptr;  // (G + 4) x kPar
     float *tacc = nullptr;    // per-thread partial sums of the table reverse steps: 2 kPar x (grid threads)
     int64_t tacc_count = 0;
     // Reverse steps without dL/dX^0: the marked nodes' adjoints and the per-thread / per-rank gradient sums.
@@ -908,7 +839,7 @@ struct AdjointBuffers {
     int64_t lean_bytes = 0;
     cudaStream_t cap_stream = nullptr;  // private stream the backward sweep's loops are captured on
     double *gtheta = nullptr; // ntheta
-    double *gsum = nullptr;   // kPar
+    double *gsum = nullptr;   // kPar, then the flag of a sweep without dL/dX^0
     double *lamstage = nullptr;  // 5 n FP64 (host-pointer staging)
 };
 
@@ -959,9 +890,9 @@ static vga_status ensure_adjoint(vga_sim *s, int64_t nseg, int64_t ckpt) {
         VGA_TRY(dmalloc((void **)&a->lam[b].h, sizeof(float) * 5 * (size_t)npad, "adjoint state"));
         VGA_TRY(dmalloc((void **)&a->lam[b].l, sizeof(res_t) * 5 * (size_t)npad, "adjoint state"));
     }
-    VGA_TRY(dmalloc((void **)&a->gpart, sizeof(double) * kPar * (size_t)std::max<int64_t>(G, 1), "gradient partials"));
+    VGA_TRY(dmalloc((void **)&a->gpart, sizeof(double) * kPar * (size_t)(G + 4), "gradient partials"));
     VGA_TRY(dmalloc((void **)&a->gtheta, sizeof(double) * (size_t)ntheta, "theta gradient"));
-    VGA_TRY(dmalloc((void **)&a->gsum, sizeof(double) * kPar, "gradient sums"));
+    VGA_TRY(dmalloc((void **)&a->gsum, sizeof(double) * (kPar + 1), "gradient sums"));
     return VGA_OK;
 }
 
@@ -992,6 +923,25 @@ static PairBuf ck_slot(AdjointBuffers *a, int64_t s) {
     p.h = reinterpret_cast<float *>(a->ck + pairb * (size_t)s);
     p.l = reinterpret_cast<res_t *>(a->ck + pairb * (size_t)s + 5 * (size_t)a->npad * sizeof(float));
     return p;
+}
+
+// The rows of a pair buffer, and of the simulation's current state.
+static StateRows rows_of(PairBuf p, int64_t npad) {
+    StateRows r;
+    for (int c = 0; c < 5; ++c) {
+        r.h[c] = p.h + (size_t)c * npad;
+        r.l[c] = p.l + (size_t)c * npad;
+    }
+    return r;
+}
+
+static StateRows rows_of(vga_sim *s) {
+    StateRows r;
+    for (int c = 0; c < 5; ++c) {
+        r.h[c] = s->comp(c);
+        r.l[c] = s->lcomp(c);
+    }
+    return r;
 }
 
 // Copies the simulation's current state into a pair buffer (or back).
@@ -1108,9 +1058,19 @@ vga_status sim_adjoint_forward(vga_sim *s, int64_t N, int64_t ckpt) {
             a->xcap = std::max<int64_t>(a->act.n_active, 1);
         }
     }
+    const bool small = a->sparse && small_ok(s, a->act);
     for (int64_t sg = 0; sg < nseg; ++sg) {
-        VGA_TRY(copy_state(s, ck_slot(a, sg), false));
         const int64_t len = std::min(ckpt, N - sg * ckpt);
+        if (small) {  // the checkpoint and the segment as one launch
+            const bool rec = sg == nseg - 1;
+            if (rec) VGA_TRY(ensure_records(a));
+            VGA_TRY(small_forward(s, a->act, rows_of(s), rows_of(s), rows_of(ck_slot(a, sg), s->npad), len - 1, true,
+                                  rec ? a->rec_y2 : nullptr, rec ? a->rec_xc : nullptr, a->xcap));
+            s->steps_done += len;
+            a->last_recorded = rec;
+            continue;
+        }
+        VGA_TRY(copy_state(s, ck_slot(a, sg), false));
         if (sg == nseg - 1 && s->g->nx <= 32767) {
             const vga_status r = s->wmode == W_BLOCK ? forward_recording<W_BLOCK>(s, a, len)
                                                      : forward_recording<W_UNIT>(s, a, len);
@@ -1170,19 +1130,18 @@ struct SweepGraphs {
     }
 };
 
-// Work buffers of a lean sweep (k_lean_dom, k_lean_marked): dL/dD slots, the marked nodes' adjoints, the flag.
+// Work buffers of a lean sweep (k_lean_dom, k_lean_marked): dL/dD slots and the marked nodes' adjoints.
 struct LeanWork {
     LeanArgs args;
     SparseState ss;
     int64_t T = 0;
-    int32_t *flag = nullptr;
 };
 
 static vga_status lean_work(vga_sim *s, AdjointBuffers *a, LeanWork *w) {
     const int64_t xcap = a->xcap;
     w->T = (int64_t)grid_for(s->n, kLeanK * kThreads) * kThreads;
     const size_t slots = sizeof(float2) * (size_t)w->T;
-    const size_t total = slots + (sizeof(float2) + (sizeof(float) + sizeof(res_t)) * 4) * (size_t)xcap + 16;
+    const size_t total = slots + (sizeof(float2) + (sizeof(float) + sizeof(res_t)) * 4) * (size_t)xcap;
     if (a->lean_bytes < (int64_t)total) {
         dfree(a->lean);
         a->lean = nullptr;
@@ -1203,15 +1162,13 @@ static vga_status lean_work(vga_sim *s, AdjointBuffers *a, LeanWork *w) {
         w->ss.h[q] = h + q * xcap;
         w->ss.l[q] = l + q * xcap;
     }
-    w->flag = reinterpret_cast<int32_t *>(l + 4 * xcap);
-    w->args.flag = w->flag;
+    w->args.flag = reinterpret_cast<int32_t *>(a->gsum + kPar);
     VGA_CUDA(cudaMemsetAsync(a->lean, 0, slots, s->stream));
-    VGA_CUDA(cudaMemsetAsync(w->flag, 0, sizeof(int32_t), s->stream));
     return VGA_OK;
 }
 
-// lean: without dL/dX^0 (k_lean_dom); *redo is set when its premise did not hold (call again with
-// lean = false).
+// lean: without dL/dX^0 where that pays (k_lean_dom, k_small_reverse); *redo is set when its premise did not
+// hold (call again with lean = false).
 template <int WM>
 static vga_status adjoint_backward_impl(vga_sim *s, const double *d_lamN, double *d_lam0, double *grad8,
                                         double *h_gtheta, bool lean, bool *redo) {
@@ -1266,10 +1223,21 @@ static vga_status adjoint_backward_impl(vga_sim *s, const double *d_lamN, double
         a->last_recorded = false;
     }
     VGA_TRY(ensure_records(a));
-    lean = lean && sparse && !d_lam0;
+    // small graphs: a segment's recomputation and its reverse steps are one launch each
+    const bool may_lean = lean && sparse && !d_lam0;
+    // (with dL/dX^0 its sums are one per pair of nodes: k_adjoint_vec's, when each of its threads takes one pair)
+    const bool small = sparse && small_ok(s, a->act) && small_reverse_ok(s, !may_lean) &&
+                       (may_lean || (kAdjK == 2 && (int64_t)Gt * kThreads * 2 >= s->n));
+    // Above a quarter of the nodes marked a lean step moves as much as a full one (36 B per node and about
+    // 120 B per marked node against 66 B per node); on small graphs its second launch costs more than it
+    // saves.  Backward sweep per step, recomputation included, 6% marked, 8^3 blocks: 0.57 M nodes 19.9 us
+    // lean, 21.9 full; 1.0 M 26.8 / 32.5; 4.7 M 96 / 147; 20.8 M 349 / 581.
+    lean = may_lean && !small && s->n >= kLeanNodes && m * 4 < s->n;
+    int32_t *flag_dev = lean || (small && may_lean) ? reinterpret_cast<int32_t *>(a->gsum + kPar) : nullptr;
+    if (flag_dev) VGA_CUDA(cudaMemsetAsync(flag_dev, 0, sizeof(int32_t), st));
     LeanWork lw;
     if (lean) VGA_TRY(lean_work(s, a, &lw));
-    k_lam_in<<<grid_for(s->n, kThreads), kThreads, 0, st>>>(s->n, d_lamN, io_from(a->lam[0], a->lam[0], npad), lw.flag);
+    k_lam_in<<<grid_for(s->n, kThreads), kThreads, 0, st>>>(s->n, d_lamN, io_from(a->lam[0], a->lam[0], npad), flag_dev);
     if (lean && m > 0) k_lean_gather<<<grid_for(m, kThreads), kThreads, 0, st>>>(m, lw.ss, io_from(a->lam[0], a->lam[0], npad));
     VGA_CHECK_LAUNCH();
     // k_lean_marked: the gradient partials bound its grid; a thread takes a few nodes, so that the block sums
@@ -1289,8 +1257,9 @@ static vga_status adjoint_backward_impl(vga_sim *s, const double *d_lamN, double
     // per-thread slots when a thread takes at most kSlotGroups groups of nodes per reverse launch
     const int64_t groups_per_thread = table ? ((s->n + kAdjK * kThreads - 1) / (kAdjK * kThreads) + Gt - 1) / Gt : 0;
     float *tacc = nullptr;
-    if (table && !lean && groups_per_thread <= kSlotGroups) {  // zeroed for this sweep
-        const int64_t count = 2 * kPar * (int64_t)Gt * kThreads;
+    const int64_t Ts = small && may_lean ? small_threads(s) : (int64_t)Gt * kThreads;  // threads that keep slots
+    if (small || (table && !lean && groups_per_thread <= kSlotGroups)) {  // zeroed for this sweep
+        const int64_t count = 2 * kPar * Ts;
         if (a->tacc_count < count) {
             dfree(a->tacc);
             a->tacc = nullptr;
@@ -1310,6 +1279,14 @@ static vga_status adjoint_backward_impl(vga_sim *s, const double *d_lamN, double
         PairBuf cks = ck_slot(a, sg);
         Rec rec;
         const bool recorded = sg == nseg - 1 && a->last_recorded;
+        if (small) {
+            if (!recorded)
+                VGA_TRY(small_forward(s, a->act, rows_of(cks, npad), StateRows{}, StateRows{}, len - 1, false, a->rec_y2,
+                                      a->rec_xc, a->xcap));
+            VGA_TRY(small_reverse(s, a->act, rows_of(a->lam[0], npad), cks.h, a->rec_y2, a->rec_xc, a->xcap, len, !may_lean,
+                                  tacc, Ts, a->gtheta, flag_dev));
+            continue;
+        }
         if (!recorded) {
             timing_begin(s, VGA_KERNEL_TRANSFORM);
             k_transform_rec<PREC><<<grid_for(s->n, kThreads), kThreads, 0, st>>>(s->n, s->sp, io_from(cks, a->work[0], npad),
@@ -1419,10 +1396,12 @@ static vga_status adjoint_backward_impl(vga_sim *s, const double *d_lamN, double
         VGA_CHECK_LAUNCH();
     }
     if (tacc) {
-        k_reduce_tacc<<<Gt, kThreads, 0, st>>>(tacc, a->gpart);
+        k_reduce_tacc<<<(unsigned)(Ts / kThreads), kThreads, 0, st>>>(tacc, a->gpart);
         ++s->launches;
     }
-    const int Gr = lean ? (int)std::max<int64_t>(Gm, std::min<int64_t>(G, 304)) : G;
+    const int Gr = lean    ? (int)std::max<int64_t>(Gm, std::min<int64_t>(G, 304))
+                   : tacc ? (int)(Ts / kThreads)
+                           : G;
     if (lean) {
         k_reduce_lean<<<Gr, kThreads, 0, st>>>(lw.T, lw.args.dslot, a->gpart);
         ++s->launches;
@@ -1431,13 +1410,20 @@ static vga_status adjoint_backward_impl(vga_sim *s, const double *d_lamN, double
     VGA_CHECK_LAUNCH();
     s->launches += 2;
     double h[kPar];
-    int32_t flag = 0;
-    if (lean) VGA_CUDA(cudaMemcpyAsync(&flag, lw.flag, sizeof(flag), cudaMemcpyDeviceToHost, st));
+    int32_t flag = 0, gave_up = 0;
+    if (flag_dev) VGA_CUDA(cudaMemcpyAsync(&flag, flag_dev, sizeof(flag), cudaMemcpyDeviceToHost, st));
+    if (small) VGA_CUDA(cudaMemcpyAsync(&gave_up, s->d_err, sizeof(gave_up), cudaMemcpyDeviceToHost, st));
     VGA_CUDA(cudaMemcpyAsync(h, a->gsum, sizeof(double) * kPar, cudaMemcpyDeviceToHost, st));
     if (s->face_mode) VGA_TRY(sim_face_mirror(s, a->gtheta));  // both slots of every edge
     if (h_gtheta && s->n_theta > 0 && s->wmode == W_BLOCK)
         VGA_CUDA(cudaMemcpyAsync(h_gtheta, a->gtheta, sizeof(double) * (size_t)s->n_theta, cudaMemcpyDeviceToHost, st));
     VGA_CUDA(cudaStreamSynchronize(st));
+    if (gave_up) {
+        VGA_CUDA(cudaMemsetAsync(s->d_err, 0, sizeof(int32_t), st));
+        small_reset(s);
+        a->valid = false;
+        return fail(VGA_ERR_TIMEOUT, "a bounded device wait timed out (small-graph launch)");
+    }
     if (flag) {
         *redo = true;
         return VGA_OK;
@@ -1471,11 +1457,7 @@ vga_status sim_adjoint_backward(vga_sim *s, const double *d_lamN, double *d_lam0
     if (!s->adj || !s->adj->valid) return fail(VGA_ERR_INVALID_ARG, "no adjoint forward pass to reverse");
     if (s->adj->param_gen != s->param_gen)
         return fail(VGA_ERR_INVALID_ARG, "parameters or conductances changed since the adjoint forward pass");
-    // Above a quarter of the nodes marked a lean step moves as much as a full one (36 B per node and about
-    // 120 B per marked node against 66 B per node); on small graphs its second launch costs more than it
-    // saves.  Backward sweep per step, recomputation included, 6% marked, 8^3 blocks: 0.30 M nodes 15.4 us
-    // lean, 13.2 full; 0.57 M 19.9 / 21.9; 1.0 M 26.8 / 32.5; 4.7 M 96 / 147; 20.8 M 349 / 581.
-    bool lean = !d_lam0 && s->adj->sparse && s->n >= kLeanNodes && s->adj->act.n_active * 4 < s->n, redo = false;
+    bool lean = !d_lam0, redo = false;
     for (;;) {
         VGA_TRY(s->wmode == W_BLOCK ? adjoint_backward_impl<W_BLOCK>(s, d_lamN, d_lam0, grad8, h_gtheta, lean, &redo)
                                     : adjoint_backward_impl<W_UNIT>(s, d_lamN, d_lam0, grad8, h_gtheta, lean, &redo));

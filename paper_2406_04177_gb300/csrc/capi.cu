@@ -8,6 +8,7 @@
 #include <cstring>
 #include <string>
 
+#include "small_graph.cuh"
 #include "vga_internal.cuh"
 
 namespace vga {
@@ -117,8 +118,10 @@ static vga_status check_device_error(vga_sim *s) {
     VGA_CUDA(cudaStreamSynchronize(s->stream));
     if (h != 0) {
         cudaMemsetAsync(s->d_err, 0, sizeof(int32_t), s->stream);
-        return fail(VGA_ERR_TIMEOUT, h == 2 ? "a bounded device wait timed out (wavefront dependency)"
-                                            : "a bounded device wait timed out (bulk copy did not complete)");
+        small_reset(s);
+        return fail(VGA_ERR_TIMEOUT, h == 3   ? "a bounded device wait timed out (small-graph launch)"
+                                     : h == 2 ? "a bounded device wait timed out (wavefront dependency)"
+                                              : "a bounded device wait timed out (bulk copy did not complete)");
     }
     return VGA_OK;
 }
@@ -775,6 +778,7 @@ vga_status vga_sim_free(vga_sim *s) {
     dfree(s->d_err);
     dfree(s->nbr_table);
     step_graphs_free(s);
+    small_free(s);
     dfree(s->nbr_tz);
     activity_free(&s->act);
     dfree(s->bnode);

@@ -22,6 +22,7 @@
 
 #include "pdl.cuh"
 #include "physics.cuh"
+#include "small_graph.cuh"
 #include "sparse_pass.cuh"
 #include "stencil.cuh"
 #include "tma.cuh"
@@ -405,6 +406,16 @@ __global__ void __launch_bounds__(kThreads) k_mask_prefix(int64_t words, const u
     }
 }
 
+// Most marked nodes among any `per_words` consecutive mask words that start at a multiple of them (one block).
+__global__ void __launch_bounds__(kThreads) k_mask_block_max(int64_t words, int64_t per_words, const uint32_t *__restrict__ prefix,
+                                                             uint32_t *__restrict__ out) {
+    uint32_t m = 0;
+    for (int64_t w = threadIdx.x * per_words; w < words; w += (int64_t)blockDim.x * per_words)
+        m = max(m, __ldg(prefix + (w + per_words < words ? w + per_words : words)) - __ldg(prefix + w));
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0) atomicMax(out, m);
+}
+
 // Marked nodes' MB, SOM, FOM, CO2 between the state arrays (io.in read, io.out written) and the
 // compact state: to_compact copies state -> compact, otherwise compact -> state.
 __global__ void k_active_copy(int64_t m, SparseState ss, StateIO io, int to_compact, int comp) {
@@ -432,9 +443,9 @@ __global__ void k_active_copy(int64_t m, SparseState ss, StateIO io, int to_comp
 // of MB, SOM, FOM and CO2 (their current values are zero), so that a pass may skip them.
 template <int PREC>
 __global__ void k_build_active(int64_t n, StateIO cur, StateIO spare, uint32_t *__restrict__ mask,
-                               unsigned long long *__restrict__ count) {
+                               unsigned long long *__restrict__ count, uint32_t *__restrict__ negative) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    bool act = false;
+    bool act = false, neg = false;
     if (i < n) {
         const int cs[4] = {0, 2, 3, 4};
 #pragma unroll
@@ -443,6 +454,7 @@ __global__ void k_build_active(int64_t n, StateIO cur, StateIO spare, uint32_t *
             if (PREC == P_COMP) act |= cur.lin[cs[q]][i] != 0;
         }
         act |= __float_as_uint(cur.in[1][i]) == 0x80000000u;
+        neg = cur.in[1][i] < 0.0f;
         if (PREC == P_COMP) act |= cur.lin[1][i] == (res_t)0x8000u;
         if (!act) {
 #pragma unroll
@@ -453,6 +465,7 @@ __global__ void k_build_active(int64_t n, StateIO cur, StateIO spare, uint32_t *
         }
     }
     const unsigned b = __ballot_sync(0xffffffffu, act);
+    if (__any_sync(0xffffffffu, neg) && (threadIdx.x & 31) == 0) atomicOr(negative, 1u);
     if ((threadIdx.x & 31) == 0 && i < n) {
         mask[i >> 5] = b;
         if (b) atomicAdd(count, (unsigned long long)__popc(b));
@@ -821,34 +834,42 @@ SparseState activity_state(const Activity &a) {
 vga_status activity_build(Activity *a, int64_t n, int64_t npad, const StateIO &cur, const StateIO &spare, bool comp,
                           cudaStream_t st) {
     const int64_t nw = (std::max<int64_t>(npad, 64) + 31) / 32 + 8;
-    if (!a->words || a->nw < nw) {  // mask words, their prefix, a counter, the tile sums of the prefix
+    if (!a->words || a->nw < nw) {  // mask words, their prefix, four words of counters, the tile sums of the prefix
         dfree(a->words);
         a->words = nullptr;
-        VGA_TRY(dmalloc((void **)&a->words,
-                        sizeof(uint32_t) * (2 * (size_t)nw + (size_t)mask_tiles(nw)) + sizeof(unsigned long long),
-                        "activity mask"));
+        VGA_TRY(dmalloc((void **)&a->words, sizeof(uint32_t) * (2 * (size_t)nw + 4 + (size_t)mask_tiles(nw)), "activity mask"));
         a->nw = nw;
         VGA_CUDA(cudaMemsetAsync(a->words, 0, sizeof(uint32_t) * 2 * (size_t)nw, st));
     }
-    unsigned long long *count = reinterpret_cast<unsigned long long *>(a->words + 2 * a->nw);
-    VGA_CUDA(cudaMemsetAsync(count, 0, sizeof(unsigned long long), st));
+    // the number of marked nodes (64 bits), the most in a block of a small-graph launch, whether a DOM is negative
+    uint32_t *info = a->words + 2 * a->nw;
+    unsigned long long *count = reinterpret_cast<unsigned long long *>(info);
+    VGA_CUDA(cudaMemsetAsync(info, 0, 4 * sizeof(uint32_t), st));
     if (n > 0) {
-        if (comp) k_build_active<P_COMP><<<grid_for(n, kThreads), kThreads, 0, st>>>(n, cur, spare, a->words, count);
-        else k_build_active<P_F32><<<grid_for(n, kThreads), kThreads, 0, st>>>(n, cur, spare, a->words, count);
+        if (comp) k_build_active<P_COMP><<<grid_for(n, kThreads), kThreads, 0, st>>>(n, cur, spare, a->words, count, info + 3);
+        else k_build_active<P_F32><<<grid_for(n, kThreads), kThreads, 0, st>>>(n, cur, spare, a->words, count, info + 3);
         VGA_CHECK_LAUNCH();
     }
     {
         const int64_t tiles = mask_tiles(a->nw);
-        uint32_t *tile_sum = a->words + 2 * a->nw + 2;  // after the 64-bit counter
+        uint32_t *tile_sum = info + 4;
         k_mask_tile_count<<<(unsigned)tiles, kThreads, 0, st>>>(a->nw, a->words, tile_sum);
         k_mask_tile_scan<<<1, kThreads, 0, st>>>(tiles, tile_sum);
         k_mask_prefix<<<(unsigned)tiles, kThreads, 0, st>>>(a->nw, a->words, tile_sum, a->words + a->nw);
         VGA_CHECK_LAUNCH();
     }
-    unsigned long long h = 0;
-    VGA_CUDA(cudaMemcpyAsync(&h, count, sizeof(h), cudaMemcpyDeviceToHost, st));
+    int K = 0, G = 0;
+    const bool small = small_shape(n, &K, &G);
+    if (small) {
+        k_mask_block_max<<<1, kThreads, 0, st>>>((n + 31) / 32, kSmallWords * K, a->words + a->nw, info + 2);
+        VGA_CHECK_LAUNCH();
+    }
+    uint32_t h[4] = {0, 0, 0, 0};
+    VGA_CUDA(cudaMemcpyAsync(h, info, sizeof(h), cudaMemcpyDeviceToHost, st));
     VGA_CUDA(cudaStreamSynchronize(st));
-    a->n_active = (int64_t)h;
+    a->n_active = (int64_t)(((uint64_t)h[1] << 32) | h[0]);
+    a->max_block = small ? (int32_t)h[2] : -1;
+    a->negative_dom = h[3] != 0;
     if (a->cap < a->n_active) {  // compact MB, SOM, FOM, CO2 (values and residuals)
         dfree(a->state);
         a->state = nullptr;
@@ -1015,6 +1036,16 @@ vga_status sim_step_explicit(vga_sim *s, int64_t n_steps) {
     // pass, 256^3 at 20% / 320^3 at 17%: 76% marked 35.8 / 55.0 us sparse, 32.9 / 48.3 dense; 48% marked
     // 24.4 / 42.5 sparse, 32.8 / 48.3 dense.  The line lies between, at five eighths.
     if (sparse && s->act.n_active * 8 >= s->n * 5) sparse = false;
+    if (sparse && n_steps <= (int64_t)1 << 30 && small_ok(s, s->act)) {  // the whole call as one launch
+        StateRows rows;
+        for (int c = 0; c < 5; ++c) {
+            rows.h[c] = s->comp(c);
+            rows.l[c] = s->lcomp(c);
+        }
+        VGA_TRY(small_forward(s, s->act, rows, rows, StateRows{}, n_steps - 1, true, nullptr, nullptr, 0));
+        s->steps_done += n_steps;
+        return VGA_OK;
+    }
     if (step_graph_eligible(s, n_steps)) return step_graphed(s, n_steps, sparse);
     return step_body(s, n_steps, sparse);
 }

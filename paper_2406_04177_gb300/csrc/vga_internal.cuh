@@ -133,6 +133,8 @@ struct Activity {
     char *state = nullptr;      // compact MB, SOM, FOM, CO2: 4 x cap values, 4 x cap residuals, cap nodes
     int64_t cap = 0;
     int64_t n_active = -1;      // marked nodes (-1: not built)
+    int32_t max_block = -1;     // most marked nodes in a block of a small-graph launch (-1: too many nodes for one)
+    bool negative_dom = false;  // a DOM value below zero was found by the build
     bool valid = false;         // built for the current state
     int64_t builds = 0;         // id of the last build, unique in the process (consumers cache per build)
 };
@@ -300,6 +302,7 @@ struct vga_sim {
     float *btheta6 = nullptr;       // BlockTable.theta6 (6 x blocks), rebuilt when param_gen moves
     int64_t btheta6_gen = -1;       // param_gen btheta6 was built for
     int32_t btable_bs = 0;          // block side the block table was built for (0: none)
+    void *small = nullptr;          // small-graph launches (small_graph.cu)
     double *loss_work = nullptr;  // block-mass objective scratch
     int64_t loss_cap = 0;
     int64_t param_gen = 0;  // bumped by every change of parameters or conductances
