@@ -14,8 +14,8 @@
 //             as CSR.  Every quantity is an integer sum, so the graph is bit-exact.
 //   restrict  primitive masses = sums of node masses (warp-aggregated FP64 atomics).
 //   scheme 3  one explicit step per launch, one row per thread, FP64, rounding as in the formula.
-//   scheme 4  (V + c L) u = m^k, m^{k+1} = V u, by Jacobi-PCG inside one CTA per solve (the coarse
-//             graph is small; the whole iteration runs without a host round trip).
+//   scheme 4  (V + c L) u = m^k, m^{k+1} = V u, by Jacobi-PCG, all steps of a call in one cooperative launch
+//             whose blocks exchange tagged words.
 //   objective Objective 1 or 2 over l data pairs and its gradient per slot; one row per thread
 //             owns its slots, so the gradient needs no atomics; the loss is reduced in FP64.
 //   sgd       theta <- theta - lr sign(g) per slot (sign(0) = 0).
@@ -26,6 +26,7 @@
 #include <vector>
 
 #include "stencil.cuh"
+#include "tagged_words.cuh"
 #include "vga_internal.cuh"
 
 using namespace vga;
@@ -44,7 +45,7 @@ struct vga_pngm {
     int32_t *rev = nullptr;      // device, nslots
     double *theta = nullptr;     // device, nslots
     double *grad = nullptr;      // device, 2 * nslots (raw, tied)
-    double *work = nullptr;      // device: PCG vectors (6 q) + loss partials + scalars
+    double *work = nullptr;      // device: PCG vectors (5 q), words (2 q and a few thousand) or loss partials, scalars
     int64_t work_count = 0;
     int32_t *d_pairs = nullptr;  // device pair indices
     int32_t *h_pairs = nullptr;  // pinned staging
@@ -64,7 +65,6 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kCap = 1024;        // nodes per decoded chunk
 constexpr int kObjBlocks = 1024;  // grid of the objective kernel (grid-stride over rows)
-constexpr int kPcgThreads = 1024;
 constexpr unsigned long long kEmpty = ~0ull;
 
 inline unsigned grid_for(int64_t count, int threads) { return (unsigned)((count + threads - 1) / threads); }
@@ -387,98 +387,199 @@ __global__ void __launch_bounds__(kThreads) k_scheme3(int32_t q, const int32_t *
     out[i] = __dsub_rn(m[i], __dmul_rn(c, s));
 }
 
-__device__ __forceinline__ double cta_sum(double v, double *sh) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    v = warp_sum_d(v);
-    if (lane == 0) sh[wid] = v;
-    __syncthreads();
-    if (wid == 0) {
-        double t = lane < (int)(blockDim.x >> 5) ? sh[lane] : 0.0;
-        t = warp_sum_d(t);
-        if (lane == 0) sh[32] = t;
-    }
-    __syncthreads();
-    const double r = sh[32];
-    __syncthreads();
-    return r;
+// ---- Scheme 4: whole solves in one cooperative launch -------------------------------------------------
+//
+// (V + c L) u = b by Jacobi-PCG, m = V u, for n_steps steps.  FP64 runs at a 64th of the FP32 rate, so the rows
+// are spread over every SM (in one block a solve at q = 32,632 took 4.9 ms, nearly all of it FP64 issue on
+// one SM).  A block owns contiguous rows; u, r, p and the inverse diagonal stay in the global work vectors,
+// read and written by the row's own thread.  What crosses blocks, the entries of u or p that rows
+// multiply and the partial sums of the dot products, is exchanged as tagged words (double_words): the
+// reader polls the word itself, so an iteration costs three trips through L2 (p, p.Ap, r.z with r.r) and
+// no barrier.  Every block adds the blocks' partial sums in block order, so all hold the same bits and
+// decide alike, and a run is deterministic.  Waits are bounded: one that gives up sets *err and the blocks
+// leave.
+constexpr int kPcgThreads = 256;
+constexpr uint32_t kPcgSpin = 1u << 21;
+
+struct PcgArgs {
+    int32_t q;
+    const int32_t *rp, *col;
+    const double *th, *vol;
+    double c, rtol;
+    double *m, *w;               // masses; 4 q doubles: u, r, p, inverse diagonal
+    unsigned long long *xw;      // 2 q words: the vector rows multiply
+    unsigned long long *sw;      // 2 x grid x 4 words: partial sums of two reductions in flight
+    int32_t maxit;
+    int64_t n_steps;
+    double *stats;               // iterations, relative residual, converged
+    int32_t *err;
+};
+
+// A double as two words of 32 bits of it and a 32-bit tag each; either may arrive first.
+__device__ __forceinline__ void st_double(unsigned long long *w, double v, uint32_t tag) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v), t = (unsigned long long)tag << 32;
+    st_word_raw(w, t | (b & 0xffffffffull));
+    st_word_raw(w + 1, t | (b >> 32));
 }
 
-// (A x)_i = v_i x_i + c sum_s theta_s (x_i - x_j)
-__device__ __forceinline__ double apply_row(int32_t i, const int32_t *rp, const int32_t *col, const double *th,
-                                            const double *vol, double c, const double *x) {
-    const double xi = x[i];
-    double s = 0.0;
-    for (int32_t k = rp[i]; k < rp[i + 1]; ++k) s += th[k] * (xi - x[col[k]]);
-    return vol[i] * xi + c * s;
-}
-
-// Scheme 4 for one step: solve (V + c L) u = b by Jacobi-PCG in one CTA, then m = V u.
-// w holds 5 q doubles (u, r, z, p, ap) + q (inverse diagonal).  stats: iterations, relres, converged.
-__global__ void __launch_bounds__(kPcgThreads, 1) k_scheme4_pcg(int32_t q, const int32_t *__restrict__ rp,
-                                                              const int32_t *__restrict__ col,
-                                                              const double *__restrict__ th,
-                                                              const double *__restrict__ vol, double c, double *m,
-                                                              double *w, double rtol, int32_t maxit, double *stats) {
-    __shared__ double sh[33];
-    double *u = w, *r = w + q, *z = w + 2 * (int64_t)q, *p = w + 3 * (int64_t)q, *ap = w + 4 * (int64_t)q,
-           *dinv = w + 5 * (int64_t)q;
-    double bb = 0.0;
-    for (int32_t i = threadIdx.x; i < q; i += blockDim.x) {
-        double s = 0.0;
-        for (int32_t k = rp[i]; k < rp[i + 1]; ++k) s += th[k];
-        dinv[i] = 1.0 / (vol[i] + c * s);
-        u[i] = m[i] / vol[i];
-        bb += m[i] * m[i];
-    }
-    bb = cta_sum(bb, sh);
-    double rz = 0.0, rr = 0.0;
-    for (int32_t i = threadIdx.x; i < q; i += blockDim.x) {
-        const double ri = m[i] - apply_row(i, rp, col, th, vol, c, u);
-        r[i] = ri;
-        const double zi = ri * dinv[i];
-        z[i] = zi;
-        p[i] = zi;
-        rz += ri * zi;
-        rr += ri * ri;
-    }
-    rz = cta_sum(rz, sh);
-    rr = cta_sum(rr, sh);
-    const double tol2 = rtol * rtol * bb;
-    int32_t it = 0;
-    while (rr > tol2 && it < maxit) {
-        double pap = 0.0;
-        for (int32_t i = threadIdx.x; i < q; i += blockDim.x) {
-            const double a = apply_row(i, rp, col, th, vol, c, p);
-            ap[i] = a;
-            pap += p[i] * a;
+__device__ __forceinline__ bool ld_double(const unsigned long long *w, uint32_t tag, double &v, const int32_t *err) {
+    for (uint32_t it = 0; it < kPcgSpin; ++it) {
+        const unsigned long long a = ld_word(w), b = ld_word(w + 1);
+        if ((uint32_t)(a >> 32) == tag && (uint32_t)(b >> 32) == tag) {
+            v = __longlong_as_double((long long)((b << 32) | (a & 0xffffffffull)));
+            return true;
         }
-        pap = cta_sum(pap, sh);
-        if (!(pap > 0.0)) break;  // not positive definite (or breakdown): stop, reported as not converged
-        const double alpha = rz / pap;
-        double rzn = 0.0, rrn = 0.0;
-        for (int32_t i = threadIdx.x; i < q; i += blockDim.x) {
-            u[i] += alpha * p[i];
-            const double ri = r[i] - alpha * ap[i];
+        if ((it & 1023u) == 1023u && *(volatile const int32_t *)err) break;
+    }
+    v = 0.0;
+    return false;
+}
+
+// Sums of two values over the whole grid, the same bits in every thread.  tag: 1, 2, ... per reduction (two
+// slots by parity: a block that publishes reduction k + 2 has seen every block's k + 1, hence every block
+// has read k).  False: a wait gave up (in any thread of the block).
+__device__ __forceinline__ bool grid_sum2(const PcgArgs &a, uint32_t tag, double &x, double &y, double *sh, bool ok) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const double wx = warp_sum_d(x), wy = warp_sum_d(y);
+    if (lane == 0) {
+        sh[wid] = wx;
+        sh[32 + wid] = wy;
+    }
+    __syncthreads();
+    unsigned long long *slots = a.sw + (size_t)(tag & 1u) * gridDim.x * 4;
+    if (threadIdx.x < 2) {
+        double s = 0.0;
+        for (int w = 0; w < nw; ++w) s += sh[32 * threadIdx.x + w];
+        st_double(slots + 4 * (size_t)blockIdx.x + 2 * threadIdx.x, s, tag);
+    }
+    double px = 0.0, py = 0.0;
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) {  // at most one per thread (grid <= SMs <= 256)
+        double v;
+        ok &= ld_double(slots + 4 * (size_t)b, tag, v, a.err);
+        px += v;
+        ok &= ld_double(slots + 4 * (size_t)b + 2, tag, v, a.err);
+        py += v;
+    }
+    px = warp_sum_d(px);
+    py = warp_sum_d(py);
+    __syncthreads();  // sh is read above
+    if (lane == 0) {
+        sh[wid] = px;
+        sh[32 + wid] = py;
+    }
+    if (!ok) atomicExch(a.err, 1);
+    ok = __syncthreads_and(ok) != 0;
+    x = 0.0;
+    y = 0.0;
+    for (int w = 0; w < nw; ++w) {
+        x += sh[w];
+        y += sh[32 + w];
+    }
+    __syncthreads();  // sh is written again by the next reduction
+    return ok;
+}
+
+// (A x)_i = v_i x_i + c sum_s theta_s (x_i - x_j), the neighbours' x_j as published words.  A row has about six
+// neighbours: the words of eight are on their way together, and only one that has not arrived is polled.
+__device__ __forceinline__ double apply_row(const PcgArgs &a, int32_t i, double xi, uint32_t tag, bool &ok) {
+    constexpr int B = 8;
+    double s = 0.0;
+    const int32_t k1 = a.rp[i + 1];
+    for (int32_t k0 = a.rp[i]; k0 < k1; k0 += B) {
+        unsigned long long lo[B], hi[B];
+#pragma unroll
+        for (int j = 0; j < B; ++j)
+            if (k0 + j < k1) {
+                const unsigned long long *w = a.xw + 2 * (size_t)__ldg(a.col + k0 + j);
+                lo[j] = ld_word(w);
+                hi[j] = ld_word(w + 1);
+            }
+#pragma unroll
+        for (int j = 0; j < B; ++j)
+            if (k0 + j < k1) {
+                double xj = __longlong_as_double((long long)((hi[j] << 32) | (lo[j] & 0xffffffffull)));
+                if ((uint32_t)(lo[j] >> 32) != tag || (uint32_t)(hi[j] >> 32) != tag)
+                    ok &= ld_double(a.xw + 2 * (size_t)__ldg(a.col + k0 + j), tag, xj, a.err);
+                s += __ldg(a.th + k0 + j) * (xi - xj);
+            }
+    }
+    return a.vol[i] * xi + a.c * s;
+}
+
+__global__ void __launch_bounds__(kPcgThreads, 1) k_scheme4_pcg(PcgArgs a) {
+    __shared__ double sh[64];
+    const int32_t q = a.q, per = (q + (int32_t)gridDim.x - 1) / (int32_t)gridDim.x;
+    const int32_t i0 = (int32_t)blockIdx.x * per + (int32_t)threadIdx.x, i1 = min((int32_t)blockIdx.x * per + per, q);
+    double *u = a.w, *r = a.w + q, *p = a.w + 2 * (int64_t)q, *dinv = a.w + 3 * (int64_t)q;
+    uint32_t xtag = 0, stag = 0;  // words are zero when the launch starts
+    double iters = 0.0, rel = 0.0;
+    bool converged = true, ok = true;
+    for (int32_t i = i0; i < i1; i += blockDim.x) {
+        double s = 0.0;
+        for (int32_t k = a.rp[i]; k < a.rp[i + 1]; ++k) s += a.th[k];
+        dinv[i] = 1.0 / (a.vol[i] + a.c * s);
+    }
+    for (int64_t step = 0; step < a.n_steps; ++step) {
+        double bb = 0.0, zero = 0.0, rz = 0.0, rr = 0.0;
+        ++xtag;
+        for (int32_t i = i0; i < i1; i += blockDim.x) {
+            const double mi = a.m[i], ui = mi / a.vol[i];
+            u[i] = ui;
+            st_double(a.xw + 2 * (size_t)i, ui, xtag);
+            bb += mi * mi;
+        }
+        if (!grid_sum2(a, ++stag, bb, zero, sh, ok)) return;
+        for (int32_t i = i0; i < i1; i += blockDim.x) {
+            const double ri = a.m[i] - apply_row(a, i, u[i], xtag, ok);
             r[i] = ri;
             const double zi = ri * dinv[i];
-            z[i] = zi;
-            rzn += ri * zi;
-            rrn += ri * ri;
+            p[i] = zi;
+            rz += ri * zi;
+            rr += ri * ri;
         }
-        rzn = cta_sum(rzn, sh);
-        rr = cta_sum(rrn, sh);
-        const double beta = rzn / rz;
-        rz = rzn;
-        for (int32_t i = threadIdx.x; i < q; i += blockDim.x) p[i] = z[i] + beta * p[i];
-        __syncthreads();
-        ++it;
+        if (!grid_sum2(a, ++stag, rz, rr, sh, ok)) return;
+        const double tol2 = a.rtol * a.rtol * bb;
+        int32_t it = 0;
+        while (rr > tol2 && it < a.maxit) {
+            // every block has read the words of the last product before any passes the sums after it
+            ++xtag;
+            for (int32_t i = i0; i < i1; i += blockDim.x) st_double(a.xw + 2 * (size_t)i, p[i], xtag);
+            double pap = 0.0;
+            zero = 0.0;
+            double ap1 = 0.0;  // A p of the thread's first row; the others' go to the words' place in u's vector
+            for (int32_t i = i0; i < i1; i += blockDim.x) {
+                const double pi = p[i], x = apply_row(a, i, pi, xtag, ok);
+                if (i == i0) ap1 = x;
+                else a.w[4 * (int64_t)q + i] = x;
+                pap += pi * x;
+            }
+            if (!grid_sum2(a, ++stag, pap, zero, sh, ok)) return;
+            if (!(pap > 0.0)) break;  // not positive definite (or breakdown): stop, reported as not converged
+            const double alpha = rz / pap;
+            double rzn = 0.0, rrn = 0.0;
+            for (int32_t i = i0; i < i1; i += blockDim.x) {
+                u[i] += alpha * p[i];
+                const double ri = r[i] - alpha * (i == i0 ? ap1 : a.w[4 * (int64_t)q + i]);
+                r[i] = ri;
+                rzn += ri * (ri * dinv[i]);
+                rrn += ri * ri;
+            }
+            if (!grid_sum2(a, ++stag, rzn, rrn, sh, ok)) return;
+            rr = rrn;
+            const double beta = rzn / rz;
+            rz = rzn;
+            for (int32_t i = i0; i < i1; i += blockDim.x) p[i] = r[i] * dinv[i] + beta * p[i];
+            ++it;
+        }
+        for (int32_t i = i0; i < i1; i += blockDim.x) a.m[i] = a.vol[i] * u[i];
+        iters += (double)it;
+        rel = bb > 0.0 ? sqrt(rr / bb) : 0.0;
+        if (!(rr <= tol2)) converged = false;
     }
-    for (int32_t i = threadIdx.x; i < q; i += blockDim.x) m[i] = vol[i] * u[i];
-    if (threadIdx.x == 0) {
-        stats[0] += (double)it;
-        const double rel = bb > 0.0 ? sqrt(rr / bb) : 0.0;
-        stats[1] = rel;
-        if (!(rr <= tol2)) stats[2] = 0.0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        a.stats[0] = iters;
+        a.stats[1] = rel;
+        a.stats[2] = converged ? 1.0 : 0.0;
     }
 }
 
@@ -910,16 +1011,47 @@ vga_status vga_pngm_step(vga_pngm *pg, double *d_m, int64_t n_steps, int32_t sch
     }
     if (!pg->symmetric) return fail(VGA_ERR_UNSUPPORTED, "Scheme 4 by PCG needs tied conductances (theta_ij = theta_ji)");
     if (!(std::isfinite(cg_rtol) && cg_rtol > 0.0) || cg_maxit < 1) return fail(VGA_ERR_INVALID_ARG, "need cg_rtol > 0, cg_maxit >= 1");
-    VGA_TRY(ensure_work(pg, 6 * (int64_t)q + kObjBlocks + 8));
-    double *stats = pg->work + 6 * (int64_t)q + kObjBlocks;
-    const double init[3] = {0.0, 0.0, 1.0};
-    VGA_CUDA(cudaMemcpyAsync(stats, init, sizeof(init), cudaMemcpyHostToDevice, st));
-    for (int64_t k = 0; k < n_steps; ++k)
-        k_scheme4_pcg<<<1, kPcgThreads, 0, st>>>(q, pg->row_ptr, pg->col, pg->theta, pg->vol, c, d_m, pg->work, cg_rtol,
-                                                 cg_maxit, stats);
-    VGA_CHECK_LAUNCH();
-    VGA_CUDA(cudaMemcpyAsync(pg->h_scal, stats, sizeof(double) * 3, cudaMemcpyDeviceToHost, st));
+    int dev = 0, sms = 0;
+    VGA_CUDA(cudaGetDevice(&dev));
+    VGA_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const int G = (int)std::max<int64_t>(1, std::min<int64_t>(std::min(sms, kPcgThreads), grid_for(q, kPcgThreads / 4)));
+    // u, r, p, inverse diagonal, A p; then the words, zeroed; then the statistics
+    const int64_t words = 2 * (int64_t)q + 8 * (int64_t)G + 8;
+    VGA_TRY(ensure_work(pg, 5 * (int64_t)q + words + 8));
+    PcgArgs a;
+    a.q = q;
+    a.rp = pg->row_ptr;
+    a.col = pg->col;
+    a.th = pg->theta;
+    a.vol = pg->vol;
+    a.c = c;
+    a.rtol = cg_rtol;
+    a.m = d_m;
+    a.w = pg->work;
+    a.xw = reinterpret_cast<unsigned long long *>(pg->work + 5 * (int64_t)q);
+    a.sw = a.xw + 2 * (size_t)q;
+    a.stats = pg->work + 5 * (int64_t)q + words;
+    a.err = reinterpret_cast<int32_t *>(a.stats + 3);
+    a.maxit = cg_maxit;
+    a.n_steps = n_steps;
+    VGA_CUDA(cudaMemsetAsync(a.xw, 0, sizeof(double) * (size_t)(words + 8), st));
+    if (n_steps > 0) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)G);
+        cfg.blockDim = dim3(kPcgThreads);
+        cfg.stream = st;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeCooperative;
+        attr[0].val.cooperative = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        VGA_CUDA(cudaLaunchKernelEx(&cfg, k_scheme4_pcg, a));
+    }
+    VGA_CUDA(cudaMemcpyAsync(pg->h_scal, a.stats, sizeof(double) * 4, cudaMemcpyDeviceToHost, st));
     VGA_CUDA(cudaStreamSynchronize(st));
+    int32_t gave_up = 0;
+    std::memcpy(&gave_up, pg->h_scal + 3, sizeof(gave_up));
+    if (gave_up) return fail(VGA_ERR_TIMEOUT, "a bounded device wait timed out (Scheme 4 solve)");
     pg->last_iters = (int64_t)pg->h_scal[0];
     pg->last_relres = pg->h_scal[1];
     if (n_steps > 0 && pg->h_scal[2] == 0.0) return fail(VGA_ERR_NOT_CONVERGED, "Scheme 4 solve reached cg_maxit before cg_rtol");

@@ -31,6 +31,7 @@
 #include "physics.cuh"
 #include "small_graph.cuh"
 #include "stencil.cuh"
+#include "tagged_words.cuh"
 
 namespace vga {
 
@@ -58,18 +59,6 @@ struct SmallArgs {
 
 // Node of a block's thread: row k of its 512 K consecutive nodes.
 __device__ __forceinline__ uint32_t node_of(uint32_t i0, int k) { return i0 + (uint32_t)(k * kSmallThreads); }
-
-__device__ __forceinline__ unsigned long long ld_word(const unsigned long long *p) {
-    unsigned long long v;
-    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(__cvta_generic_to_global(p)) : "memory");
-    return v;
-}
-
-__device__ __forceinline__ void st_word(unsigned long long *p, float v, uint32_t tag) {
-    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(__cvta_generic_to_global(p)),
-                 "l"(((unsigned long long)tag << 32) | __float_as_uint(v))
-                 : "memory");
-}
 
 // Offset-table entries of the thread's nodes (zero beyond the last node).
 template <int K>
