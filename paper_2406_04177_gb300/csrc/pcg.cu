@@ -372,9 +372,8 @@ vga_status solve(vga_sim *s, CgVecs v, double *part_chunk, double *part_ew, CgSc
 //
 // Kernels of one inner iteration (three launches; no single-block scalar kernels):
 //   k_mx_spmv   q = B p (four nodes per thread), partial p.q; the last block to finish forms alpha
-//   k_mx_upd    d += alpha p, r -= alpha q, partials r.Tr and r.r; the last block tests the inner
-//               stop and forms beta
-//   k_mx_p      p = T r + beta p
+//   k_mx_upd    r -= alpha q, partials r.Tr and r.r; the last block tests the inner stop and forms beta
+//   k_mx_p      d += alpha p, p = T r + beta p (k_mx_x does the last step's d)
 // The Jacobi scaling T = diag(1 / (1 + c deg_i)) is not stored: each node keeps its degree in one
 // byte and the kernels look t up in a 7-entry table computed by the same expression everywhere.
 // "Last block": each block stores its partials, fences, and takes a ticket from a counter; the
@@ -382,7 +381,12 @@ vga_status solve(vga_sim *s, CgVecs v, double *part_chunk, double *part_ew, CgSc
 // depend on which block that is) and resets the counter.  No block waits for another.
 
 constexpr double kInnerTol = 1e-4;  // reduction asked of one FP32 inner solve
-constexpr int kMxBlocks = 2432;     // grid of the mixed-solver kernels: 152 SMs x 16 (grid-stride)
+// Grid of the mixed-solver kernels (grid-stride): four blocks per SM, and no block without nodes.  Every block
+// ends with a ticket from one counter, which 2432 blocks made the longest part of a kernel (k_mx_upd, 0.30 M
+// nodes: 18.7 us with 1165 blocks): per iteration 2.4 M nodes 68.6 -> 43 us, 20.8 M 247 -> 226.
+constexpr int kMxBlocks = 608;
+constexpr int kMxNodes = 1024;      // nodes of a block's turn
+constexpr int kMxUnroll = 4;        // inner iterations per turn of the device-side loop
 constexpr int kMaxOuter = 64;
 
 struct MxScalars {
@@ -400,6 +404,10 @@ struct MxLoop {
     cudaGraphConditionalHandle outer, inner;
     int cond;
 };
+
+// The kernels of an inner iteration take the nodes in alternating order, so that each starts on what the one
+// before it left in L2.
+__device__ __forceinline__ bool mx_descending(const MxScalars *sc, int stage) { return ((3 * sc->in_iters + stage) & 1) != 0; }
 
 // Deterministic sum of part[k*stride + comp] over k < count by one block, read at L2 (the partials
 // were written by other blocks of the same launch).
@@ -684,7 +692,9 @@ __global__ void __launch_bounds__(kThreads) k_mx_spmv(int64_t n, NbrTable tb, fl
     const uint32_t nn = (uint32_t)n;
     const int lane = threadIdx.x & 31;
     const int64_t nsup = (n + (int64_t)kThreads * K - 1) / ((int64_t)kThreads * K);
-    for (int64_t sup = blockIdx.x; sup < nsup; sup += gridDim.x) {
+    const bool rev = mx_descending(sc, 0);
+    for (int64_t t = blockIdx.x; t < nsup; t += gridDim.x) {
+        const int64_t sup = rev ? nsup - 1 - t : t;
         const uint32_t i0 = (uint32_t)(sup * kThreads * K + (int64_t)threadIdx.x * K);
         const bool full = i0 + K <= nn;
         float pv[K];
@@ -770,30 +780,24 @@ __global__ void __launch_bounds__(kThreads) k_mx_upd(int64_t n, float c, MxVecs 
     float a0 = 0.0f, a1 = 0.0f;
     const int64_t n4 = n >> 2;
     const int64_t g0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, gs = (int64_t)gridDim.x * blockDim.x;
-    float4 *__restrict__ d4 = reinterpret_cast<float4 *>(v.d);
     float4 *__restrict__ r4 = reinterpret_cast<float4 *>(v.r);
-    const float4 *__restrict__ p4 = reinterpret_cast<const float4 *>(v.p);
     const float4 *__restrict__ q4 = reinterpret_cast<const float4 *>(v.q);
     const uchar4 *__restrict__ g4 = reinterpret_cast<const uchar4 *>(v.deg);
-    for (int64_t k = g0; k < n4; k += gs) {
-        float4 d = d4[k], r = r4[k];
-        const float4 p = p4[k], q = q4[k];
+    const bool rev = mx_descending(sc, 1);
+    for (int64_t t = g0; t < n4; t += gs) {
+        const int64_t k = rev ? n4 - 1 - t : t;
+        float4 r = r4[k];
+        const float4 q = q4[k];
         const uchar4 g = g4[k];
-        d.x += alpha * p.x;
-        d.y += alpha * p.y;
-        d.z += alpha * p.z;
-        d.w += alpha * p.w;
         r.x -= alpha * q.x;
         r.y -= alpha * q.y;
         r.z -= alpha * q.z;
         r.w -= alpha * q.w;
-        d4[k] = d;
         r4[k] = r;
         a0 += r.x * (tdeg[g.x] * r.x) + r.y * (tdeg[g.y] * r.y) + r.z * (tdeg[g.z] * r.z) + r.w * (tdeg[g.w] * r.w);
         a1 += r.x * r.x + r.y * r.y + r.z * r.z + r.w * r.w;
     }
     for (int64_t i = 4 * n4 + g0; i < n; i += gs) {
-        v.d[i] += alpha * v.p[i];
         const float ri = v.r[i] - alpha * v.q[i];
         v.r[i] = ri;
         a0 += ri * (tdeg[v.deg[i]] * ri);
@@ -824,7 +828,7 @@ __global__ void __launch_bounds__(kThreads) k_mx_upd(int64_t n, float c, MxVecs 
                 sc->done = 1;
                 sc->notconv = 1;
             }
-            if (loop.cond) cudaGraphSetConditional(loop.inner, sc->inner_done ? 0u : 1u);
+            if (loop.cond && sc->inner_done) cudaGraphSetConditional(loop.inner, 0u);
         }
     }
 }
@@ -834,23 +838,34 @@ __global__ void __launch_bounds__(kThreads) k_mx_p(int64_t n, float c, MxVecs v,
     __shared__ float tdeg[8];
     if (threadIdx.x < 8) tdeg[threadIdx.x] = jacobi_t(c, (int)threadIdx.x);
     __syncthreads();
-    const float beta = (float)sc->beta;
+    const float beta = (float)sc->beta, alpha = (float)sc->alpha;
     const int64_t n4 = n >> 2;
     const int64_t g0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, gs = (int64_t)gridDim.x * blockDim.x;
     float4 *__restrict__ p4 = reinterpret_cast<float4 *>(v.p);
+    float4 *__restrict__ d4 = reinterpret_cast<float4 *>(v.d);
     const float4 *__restrict__ r4 = reinterpret_cast<const float4 *>(v.r);
     const uchar4 *__restrict__ g4 = reinterpret_cast<const uchar4 *>(v.deg);
-    for (int64_t k = g0; k < n4; k += gs) {
-        float4 p = p4[k];
+    const bool rev = !mx_descending(sc, 1);  // in_iters has moved on since k_mx_upd
+    for (int64_t t = g0; t < n4; t += gs) {
+        const int64_t k = rev ? n4 - 1 - t : t;
+        float4 p = p4[k], d = d4[k];
         const float4 r = r4[k];
         const uchar4 g = g4[k];
+        d.x += alpha * p.x;
+        d.y += alpha * p.y;
+        d.z += alpha * p.z;
+        d.w += alpha * p.w;
+        d4[k] = d;
         p.x = tdeg[g.x] * r.x + beta * p.x;
         p.y = tdeg[g.y] * r.y + beta * p.y;
         p.z = tdeg[g.z] * r.z + beta * p.z;
         p.w = tdeg[g.w] * r.w + beta * p.w;
         p4[k] = p;
     }
-    for (int64_t i = 4 * n4 + g0; i < n; i += gs) v.p[i] = tdeg[v.deg[i]] * v.r[i] + beta * v.p[i];
+    for (int64_t i = 4 * n4 + g0; i < n; i += gs) {
+        v.d[i] += alpha * v.p[i];
+        v.p[i] = tdeg[v.deg[i]] * v.r[i] + beta * v.p[i];
+    }
 }
 
 // x += d in float-float (TwoSum of the high part and d, then renormalised).
@@ -868,9 +883,16 @@ __global__ void __launch_bounds__(kThreads) k_mx_x(int64_t n, MxVecs v, const Mx
     float4 *__restrict__ h4 = reinterpret_cast<float4 *>(v.xh);
     float4 *__restrict__ l4 = reinterpret_cast<float4 *>(v.xl);
     const float4 *__restrict__ d4 = reinterpret_cast<const float4 *>(v.d);
+    const float4 *__restrict__ p4 = reinterpret_cast<const float4 *>(v.p);
+    const float alpha = (float)sc->alpha;  // the inner solve's last step (k_mx_p did the others)
     for (int64_t k = g0; k < n4; k += gs) {
         float4 h = h4[k], l = l4[k];
-        const float4 d = d4[k];
+        float4 d = d4[k];
+        const float4 p = p4[k];
+        d.x += alpha * p.x;
+        d.y += alpha * p.y;
+        d.z += alpha * p.z;
+        d.w += alpha * p.w;
         ff_add_f(h.x, l.x, d.x);
         ff_add_f(h.y, l.y, d.y);
         ff_add_f(h.z, l.z, d.z);
@@ -878,7 +900,7 @@ __global__ void __launch_bounds__(kThreads) k_mx_x(int64_t n, MxVecs v, const Mx
         h4[k] = h;
         l4[k] = l;
     }
-    for (int64_t i = 4 * n4 + g0; i < n; i += gs) ff_add_f(v.xh[i], v.xl[i], v.d[i]);
+    for (int64_t i = 4 * n4 + g0; i < n; i += gs) ff_add_f(v.xh[i], v.xl[i], v.d[i] + alpha * v.p[i]);
 }
 
 // The solution as the new stored DOM: h = RN(xh + xl) and the exact remainder as residual.
@@ -896,7 +918,7 @@ __global__ void __launch_bounds__(kThreads) k_mx_out(int64_t n, MxVecs v, float 
 // ---- the mixed solve as one CUDA graph -------------------------------------------------------
 //
 //   k_mx_bmax -> k_mx_bscale -> k_mx_rhs -> k_mx_res<first> -> WHILE(outer) { k_mx_scal_out ->
-//   WHILE(inner) { k_mx_spmv -> k_mx_upd -> k_mx_p } -> k_mx_x -> k_mx_res } -> k_mx_out
+//   WHILE(inner) { kMxUnroll times (k_mx_spmv -> k_mx_upd -> k_mx_p) } -> k_mx_x -> k_mx_res } -> k_mx_out
 //
 // k_mx_scal_out sets both conditions to "not done" at the start of every outer iteration and
 // k_mx_upd clears the inner one when the inner solve stops, so the host launches the graph and
@@ -991,9 +1013,13 @@ cudaError_t mx_graph_build(vga_sim *s, const MxVecs &v, const NbrTable &tb, FF c
     MX_TRY(add_while(&n_inner, body_o, &n_scal, loop.inner, &body_i));
     MX_TRY(add_kernel(&n_x, body_o, &n_inner, k_mx_x, G, s->n, v, sc));
     MX_TRY(add_kernel(&n_res, body_o, &n_x, k_mx_res<false, TF>, G, s->n, tb, cff, v, part_a, sc));
-    MX_TRY(add_kernel(&n_spmv, body_i, nullptr, k_mx_spmv<TF>, G, s->n, tb, ch, v, part_a, sc));
-    MX_TRY(add_kernel(&n_upd, body_i, &n_spmv, k_mx_upd, G, s->n, ch, v, sc, part_b, in_maxit, loop));
-    MX_TRY(add_kernel(&n_p, body_i, &n_upd, k_mx_p, G, s->n, ch, v, sc));
+    // A turn of the loop costs as much as a small kernel, so it holds several iterations; the kernels of those that
+    // come after the last one return at once (per step of 39 iterations, 16 k nodes: 862 -> 795 us).
+    for (int u = 0; u < kMxUnroll; ++u) {
+        MX_TRY(add_kernel(&n_spmv, body_i, u > 0 ? &n_p : nullptr, k_mx_spmv<TF>, G, s->n, tb, ch, v, part_a, sc));
+        MX_TRY(add_kernel(&n_upd, body_i, &n_spmv, k_mx_upd, G, s->n, ch, v, sc, part_b, in_maxit, loop));
+        MX_TRY(add_kernel(&n_p, body_i, &n_upd, k_mx_p, G, s->n, ch, v, sc));
+    }
 #undef MX_TRY
     *gout = g;
     return cudaSuccess;
@@ -1022,7 +1048,7 @@ vga_status solve_mixed(vga_sim *s, double *base, double *part_a, double *part_b,
     v.q = f + 6 * s->npad;
     v.d = f + 7 * s->npad;
     v.deg = reinterpret_cast<uint8_t *>(f + 8 * s->npad);
-    const int G = (int)std::min<int64_t>(kMxBlocks, grid_for(s->n, kThreads));
+    const int G = (int)std::min<int64_t>(kMxBlocks, grid_for(s->n, kMxNodes));
     const int in_maxit = 200;
     MxScalars *h = reinterpret_cast<MxScalars *>(s->h_cg);
 
