@@ -15,9 +15,9 @@ __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.lau
 
 // Launch with programmatic stream serialisation (the kernel must call pdl_wait first).
 template <typename... KArgs, typename... Args>
-void launch_pdl(void (*kernel)(KArgs...), unsigned grid, unsigned threads, cudaStream_t stream, Args... args) {
+void launch_pdl(void (*kernel)(KArgs...), dim3 grid, unsigned threads, cudaStream_t stream, Args... args) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
+    cfg.gridDim = grid;
     cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = 0;
     cfg.stream = stream;

@@ -25,6 +25,7 @@
 #include <new>
 #include <vector>
 
+#include "pdl.cuh"
 #include "stencil.cuh"
 #include "tagged_words.cuh"
 #include "vga_internal.cuh"
@@ -45,12 +46,10 @@ struct vga_pngm {
     int32_t *rev = nullptr;      // device, nslots
     double *theta = nullptr;     // device, nslots
     double *grad = nullptr;      // device, 2 * nslots (raw, tied)
-    double *work = nullptr;      // device: PCG vectors (5 q), words (2 q and a few thousand) or loss partials, scalars
+    double *work = nullptr;      // device: PCG vectors (5 q), words (2 q and a few thousand); or the objective's vectors
     int64_t work_count = 0;
-    int32_t *d_pairs = nullptr;  // device pair indices
-    int32_t *h_pairs = nullptr;  // pinned staging
-    int32_t pairs_cap = 0;
     double *h_scal = nullptr;    // pinned: loss, PCG iterations, relres, converged
+    cudaEvent_t have_loss = nullptr;  // the loss of an SGD step is in h_scal
     unsigned long long *fx = nullptr;  // restriction: fixed-point sums (q), scale (2), partials
     bool symmetric = true;       // theta_ij == theta_ji for every pair
     // host copies of the geometry (export)
@@ -64,7 +63,9 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kCap = 1024;        // nodes per decoded chunk
-constexpr int kObjBlocks = 1024;  // grid of the objective kernel (grid-stride over rows)
+constexpr int kObjBlocks = 1024;  // blocks per pair of the objective kernels (grid-stride over rows)
+constexpr int32_t kObjPairs = 64;      // pairs of one launch (a kernel argument of 516 bytes)
+constexpr int64_t kObjWords = 1 << 25;  // their ratios and coefficients
 constexpr unsigned long long kEmpty = ~0ull;
 
 inline unsigned grid_for(int64_t count, int threads) { return (unsigned)((count + threads - 1) / threads); }
@@ -583,56 +584,114 @@ __global__ void __launch_bounds__(kPcgThreads, 1) k_scheme4_pcg(PcgArgs a) {
     }
 }
 
-// Objective 1 (KIND 1) or 2 (KIND 2) over the l pairs (data[pairs[2p]], data[pairs[2p+1]]):
-// residual r_i and gradient 2 r_i dr_i/dtheta_s / (l q) for the slots of row i.
+// Objective 1 (KIND 1) or 2 (KIND 2) over pairs (x, y) of records: residual r_i and gradient 2 r_i dr_i/dtheta_s / (l q)
+// for the slots of row i.  a is the vector whose fluxes enter the residual: x for Objective 1, y for Objective 2.
+//
+// The work is 64-bit arithmetic, of which a division is the dearest.  With one thread per row that divides wherever it
+// reads a concentration, 32,768 rows of 6 slots and 4 pairs took 47 us: 14 divisions per slot and pair in one chain, a
+// warp or so per scheduler.  So: k_obj_ratio divides once per row and pair; k_obj_residual has a thread per row and
+// pair; k_obj_grad has one per slot, and ties and applies what it has summed.  All vectors lie pair after pair, so that
+// the threads of a warp read neighbouring rows of one pair.  With the pairs as an argument and the loss written to the
+// host's memory no copies are left: a training epoch at that size 96 -> 47 us, most of it now the host's.
+struct ObjPairs {
+    int32_t l;                    // pairs of this launch
+    int32_t idx[2 * kObjPairs];  // records x, y of each
+};
+
 template <int KIND>
-__global__ void __launch_bounds__(kThreads) k_objective(int32_t q, const int32_t *__restrict__ rp,
-                                                        const int32_t *__restrict__ col, const double *__restrict__ th,
-                                                        const double *__restrict__ vol, double c,
-                                                        const double *__restrict__ data, const int32_t *__restrict__ pairs,
-                                                        int32_t l, double *__restrict__ grad, double *__restrict__ part) {
-    double loss = 0.0;
-    const double inv_lq = 1.0 / ((double)l * (double)q);
-    for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < q; i += gridDim.x * blockDim.x) {
+__global__ void __launch_bounds__(kThreads) k_obj_ratio(int32_t q, const double *__restrict__ vol,
+                                                        const double *__restrict__ data, const __grid_constant__ ObjPairs pr,
+                                                        double *__restrict__ ratio, uint32_t *__restrict__ ticket) {
+    pdl_trigger();
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *ticket = 0u;
+    const int32_t pp = blockIdx.y;
+    const double *a = data + (int64_t)pr.idx[2 * pp + (KIND == 1 ? 0 : 1)] * q;
+    for (int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x; i < q; i += (int64_t)gridDim.x * kThreads)
+        ratio[(int64_t)pp * q + i] = a[i] / vol[i];
+}
+
+// coef = +-2 c r_i / (l q); the last block to finish adds the blocks' sums of r^2 / (l q), in block order, to *loss (from
+// zero if `first`) and copies the loss to the host's word.
+template <int KIND>
+__global__ void __launch_bounds__(kThreads) k_obj_residual(int32_t q, const int32_t *__restrict__ rp,
+                                                           const int32_t *__restrict__ col, const double *__restrict__ th,
+                                                           const double *__restrict__ data, double c, double inv_lq,
+                                                           const __grid_constant__ ObjPairs pr,
+                                                           const double *ratio, double *coef, double *part, double *loss, double *h_loss, bool first,
+                                                           uint32_t *ticket) {
+    __shared__ bool last;
+    pdl_wait();
+    const int32_t pp = blockIdx.y;
+    const double *x = data + (int64_t)pr.idx[2 * pp] * q;
+    const double *y = data + (int64_t)pr.idx[2 * pp + 1] * q;
+    const double *ra = ratio + (int64_t)pp * q;
+    double sum = 0.0;
+    for (int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x; i < q; i += (int64_t)gridDim.x * kThreads) {
         const int32_t k0 = rp[i], k1 = rp[i + 1];
-        for (int32_t k = k0; k < k1; ++k) grad[k] = 0.0;
-        for (int32_t pp = 0; pp < l; ++pp) {
-            const double *x = data + (int64_t)pairs[2 * pp] * q;
-            const double *y = data + (int64_t)pairs[2 * pp + 1] * q;
-            // the vector whose fluxes enter the residual: x for Objective 1, y for Objective 2
-            const double *a = KIND == 1 ? x : y;
-            const double ai = a[i] / vol[i];
-            double fs = 0.0;
-            for (int32_t k = k0; k < k1; ++k) fs += th[k] * (ai - a[col[k]] / vol[col[k]]);
-            const double r = KIND == 1 ? (y[i] - x[i]) + c * fs : (x[i] - y[i]) - c * fs;
-            loss += r * r;
-            const double coef = (KIND == 1 ? 2.0 : -2.0) * c * r * inv_lq;
-            for (int32_t k = k0; k < k1; ++k) grad[k] += coef * (ai - a[col[k]] / vol[col[k]]);
-        }
+        const double ai = ra[i];
+        double fs = 0.0;
+        for (int32_t k = k0; k < k1; ++k) fs += th[k] * (ai - ra[col[k]]);
+        const double r = KIND == 1 ? (y[i] - x[i]) + c * fs : (x[i] - y[i]) - c * fs;
+        sum += r * r;
+        coef[(int64_t)pp * q + i] = (KIND == 1 ? 2.0 : -2.0) * c * r * inv_lq;
     }
-    double v[1] = {loss * inv_lq};
-    block_sum_store<1>(v, part + blockIdx.x);
-}
-
-__global__ void k_sum_partials(const double *__restrict__ part, int32_t count, double *__restrict__ out) {
+    const uint32_t blocks = gridDim.x * gridDim.y, b = blockIdx.y * gridDim.x + blockIdx.x;
+    double v[1] = {sum * inv_lq};
+    block_sum_store<1>(v, part + b);
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(ticket, 1u) == blocks - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
     double s = 0.0;
-    for (int32_t i = threadIdx.x; i < count; i += blockDim.x) s += part[i];
-    double v[1] = {s};
-    block_sum_store<1>(v, out);
+    for (uint32_t k = threadIdx.x; k < blocks; k += kThreads) s += __ldcg(part + k);
+    v[0] = s;
+    block_sum_store<1>(v, part);
+    if (threadIdx.x == 0) {
+        const double t = part[0] + (first ? 0.0 : *loss);
+        *loss = t;
+        *h_loss = t;
+    }
 }
 
-__global__ void k_tie(int32_t ns, const int32_t *__restrict__ rev, const double *__restrict__ g,
-                      double *__restrict__ out) {
-    const int32_t s = (int32_t)(blockIdx.x * blockDim.x + threadIdx.x);
-    if (s < ns) out[s] = g[s] + g[rev[s]];
+__device__ __forceinline__ double sign_step(double th, double g, double lr, double tmin) {
+    const double step = g > 0.0 ? 1.0 : (g < 0.0 ? -1.0 : 0.0);
+    return fmax(th - lr * step, tmin);
 }
 
-__global__ void k_sign_sgd(int32_t ns, const double *__restrict__ g, double *__restrict__ th, double lr, double tmin) {
-    const int32_t s = (int32_t)(blockIdx.x * blockDim.x + threadIdx.x);
+// What becomes of the gradient: the raw gradient of every slot, kept (and added to by the next launch's pairs); or the
+// gradient tied over both directions of an edge (TIED), kept or used at once for the sign step (SGD).
+enum GradUse { GRAD_RAW, GRAD_TIED, SGD_RAW, SGD_TIED };
+
+// One thread per slot; with tied conductances the thread of the lower row does both directions.
+template <int USE>
+__global__ void __launch_bounds__(kThreads) k_obj_grad(int32_t ns, int32_t q, int32_t l, const int32_t *__restrict__ col,
+                                                       const int32_t *__restrict__ rev, const double *__restrict__ ratio,
+                                                       const double *__restrict__ coef, bool first, double *grad,
+                                                       double *th, double lr, double tmin) {
+    constexpr bool TIED = USE == GRAD_TIED || USE == SGD_TIED;
+    const int32_t s = (int32_t)(blockIdx.x * kThreads + threadIdx.x);
     if (s >= ns) return;
-    const double gs = g[s];
-    const double step = gs > 0.0 ? 1.0 : (gs < 0.0 ? -1.0 : 0.0);
-    th[s] = fmax(th[s] - lr * step, tmin);
+    const int32_t o = rev[s], j = col[s], i = col[o];
+    if (TIED && i > j) return;
+    double g = first ? 0.0 : grad[s], gr = first || !TIED ? 0.0 : grad[o];
+#pragma unroll 4
+    for (int32_t pp = 0; pp < l; ++pp) {
+        const double ri = ratio[i], rj = ratio[j];
+        g += coef[i] * (ri - rj);
+        if (TIED) gr += coef[j] * (rj - ri);
+        ratio += q;
+        coef += q;
+    }
+    if (USE == GRAD_RAW) grad[s] = g;
+    if (USE == GRAD_TIED) grad[ns + s] = grad[ns + o] = g + gr;
+    if (USE == SGD_RAW) th[s] = sign_step(th[s], g, lr, tmin);
+    if (USE == SGD_TIED) {
+        th[s] = sign_step(th[s], g + gr, lr, tmin);
+        th[o] = sign_step(th[o], g + gr, lr, tmin);
+    }
 }
 
 vga_status ensure_work(vga_pngm *pg, int64_t count) {
@@ -645,20 +704,6 @@ vga_status ensure_work(vga_pngm *pg, int64_t count) {
     return VGA_OK;
 }
 
-vga_status ensure_pairs(vga_pngm *pg, int32_t l) {
-    if (pg->pairs_cap >= l) return VGA_OK;
-    dfree(pg->d_pairs);
-    if (pg->h_pairs) cudaFreeHost(pg->h_pairs);
-    pg->d_pairs = nullptr;
-    pg->h_pairs = nullptr;
-    pg->pairs_cap = 0;
-    const int32_t cap = std::max<int32_t>(64, l);
-    VGA_TRY(dmalloc((void **)&pg->d_pairs, sizeof(int32_t) * 2 * (size_t)cap, "pair indices"));
-    VGA_CUDA(cudaMallocHost((void **)&pg->h_pairs, sizeof(int32_t) * 2 * (size_t)cap));
-    pg->pairs_cap = cap;
-    return VGA_OK;
-}
-
 // Frees every buffer of the handle; returns the name of the first release call that failed (the
 // runtime's error state is left set for release_status to report).
 const char *pngm_release(vga_pngm *pg) {
@@ -666,12 +711,12 @@ const char *pngm_release(vga_pngm *pg) {
     auto chk = [&](cudaError_t e, const char *what) {
         if (e != cudaSuccess && !bad) bad = what;
     };
-    void *dev[] = {pg->labels, pg->vol, pg->row_ptr, pg->col, pg->rev, pg->theta, pg->grad, pg->work, pg->d_pairs, pg->fx};
-    const char *names[] = {"labels", "vol", "row_ptr", "col", "rev", "theta", "grad", "work", "d_pairs", "fx"};
-    for (int k = 0; k < 10; ++k)
+    void *dev[] = {pg->labels, pg->vol, pg->row_ptr, pg->col, pg->rev, pg->theta, pg->grad, pg->work, pg->fx};
+    const char *names[] = {"labels", "vol", "row_ptr", "col", "rev", "theta", "grad", "work", "fx"};
+    for (int k = 0; k < 9; ++k)
         if (dev[k]) chk(cudaFree(dev[k]), names[k]);
-    if (pg->h_pairs) chk(cudaFreeHost(pg->h_pairs), "h_pairs");
     if (pg->h_scal) chk(cudaFreeHost(pg->h_scal), "h_scal");
+    if (pg->have_loss) chk(cudaEventDestroy(pg->have_loss), "have_loss");
     delete pg;
     return bad;
 }
@@ -825,6 +870,7 @@ vga_status build(vga_pngm *pg, const int32_t *labels, bool on_device) {
     VGA_TRY(dmalloc((void **)&pg->theta, sizeof(double) * ns1, "conductances"));
     VGA_TRY(dmalloc((void **)&pg->grad, sizeof(double) * 2 * ns1, "gradients"));
     VGA_CUDA(cudaMallocHost((void **)&pg->h_scal, sizeof(double) * 8));
+    VGA_CUDA(cudaEventCreateWithFlags(&pg->have_loss, cudaEventDisableTiming));
     VGA_CUDA(cudaMemcpy(pg->vol, pg->h_vol.data(), sizeof(double) * (size_t)q, cudaMemcpyHostToDevice));
     VGA_CUDA(cudaMemcpy(pg->row_ptr, pg->h_row_ptr.data(), sizeof(int32_t) * ((size_t)q + 1), cudaMemcpyHostToDevice));
     if (ns > 0) {
@@ -843,35 +889,55 @@ vga_status check_pairs(const vga_pngm *pg, const int32_t *pairs, int32_t l, int6
     return VGA_OK;
 }
 
-// Loss and gradient (raw per slot in grad[0..ns), tied in grad[ns..2ns) when requested).  The loss
-// stays on the device at h_scal[0] after the copy; the stream is synchronised.
+template <int USE>
+void launch_grad(vga_pngm *pg, int32_t l, const double *ratio, const double *coef, bool first, double lr, double tmin) {
+    if (pg->nslots > 0)
+        k_obj_grad<USE><<<grid_for(pg->nslots, kThreads), kThreads, 0, pg->stream>>>(
+            pg->nslots, pg->q, l, pg->col, pg->rev, ratio, coef, first, pg->grad, pg->theta, lr, tmin);
+}
+
+// Loss, and the gradient (raw per slot in grad[0..ns), tied in grad[ns..2ns)) or one sign step of theta from it (`sgd`).
+// The pairs travel as a kernel argument, kObjPairs at a time: more than that accumulate in grad[0..ns) launch by launch,
+// with the last launch's use of the sum.  Fewer at a time where the ratios and coefficients would need more than 256 MB.
+// Returns with the loss on the host; the gradient is complete then, the sign step is on the stream.
 vga_status objective(vga_pngm *pg, int32_t kind, const double *d_data, int64_t n_records, const int32_t *pairs, int32_t l,
-                     double D, double dt, bool tied, double *loss) {
+                     double D, double dt, bool tied, bool sgd, double lr, double tmin, double *loss) {
     if (kind != 1 && kind != 2) return fail(VGA_ERR_INVALID_ARG, "objective must be 1 or 2");
     if (!d_data) return fail(VGA_ERR_INVALID_ARG, "data is NULL");
     if (!(std::isfinite(D) && D >= 0.0 && std::isfinite(dt) && dt > 0.0)) return fail(VGA_ERR_INVALID_ARG, "need D >= 0, dt > 0");
     VGA_TRY(check_pairs(pg, pairs, l, n_records));
-    VGA_TRY(ensure_pairs(pg, l));
-    VGA_TRY(ensure_work(pg, 6 * (int64_t)pg->q + kObjBlocks + 8));
+    const int64_t q = pg->q;
+    const int32_t at_once = (int32_t)std::min<int64_t>(std::min(l, kObjPairs), std::max<int64_t>(3, kObjWords / (2 * q)));
+    const int64_t gx = std::min<int64_t>(kObjBlocks, grid_for(q, kThreads));
+    VGA_TRY(ensure_work(pg, 2 * at_once * q + at_once * gx + 2));
     cudaStream_t st = pg->stream;
-    std::memcpy(pg->h_pairs, pairs, sizeof(int32_t) * 2 * (size_t)l);
-    VGA_CUDA(cudaMemcpyAsync(pg->d_pairs, pg->h_pairs, sizeof(int32_t) * 2 * (size_t)l, cudaMemcpyHostToDevice, st));
-    const double c = D * dt;
-    double *part = pg->work + 6 * (int64_t)pg->q;
-    double *d_loss = part + kObjBlocks;
-    const unsigned G = (unsigned)std::min<int64_t>(kObjBlocks, std::max<int64_t>(1, grid_for(pg->q, kThreads)));
-    if (kind == 1)
-        k_objective<1><<<G, kThreads, 0, st>>>(pg->q, pg->row_ptr, pg->col, pg->theta, pg->vol, c, d_data, pg->d_pairs, l,
-                                               pg->grad, part);
-    else
-        k_objective<2><<<G, kThreads, 0, st>>>(pg->q, pg->row_ptr, pg->col, pg->theta, pg->vol, c, d_data, pg->d_pairs, l,
-                                               pg->grad, part);
-    k_sum_partials<<<1, kThreads, 0, st>>>(part, (int32_t)G, d_loss);
-    if (tied && pg->nslots > 0)
-        k_tie<<<grid_for(pg->nslots, kThreads), kThreads, 0, st>>>(pg->nslots, pg->rev, pg->grad, pg->grad + pg->nslots);
+    double *ratio = pg->work, *coef = ratio + at_once * q, *part = coef + at_once * q, *d_loss = part + at_once * gx;
+    uint32_t *ticket = reinterpret_cast<uint32_t *>(d_loss + 1);
+    const double c = D * dt, inv_lq = 1.0 / ((double)l * (double)q);
+    ObjPairs pr;
+    for (int32_t p0 = 0; p0 < l; p0 += at_once) {
+        pr.l = std::min(at_once, l - p0);
+        std::memcpy(pr.idx, pairs + 2 * (size_t)p0, sizeof(int32_t) * 2 * (size_t)pr.l);
+        const bool first = p0 == 0, last = p0 + pr.l == l;
+        const dim3 grid((unsigned)gx, (unsigned)pr.l);
+        if (kind == 1) {
+            k_obj_ratio<1><<<grid, kThreads, 0, st>>>(pg->q, pg->vol, d_data, pr, ratio, ticket);
+            launch_pdl(k_obj_residual<1>, grid, kThreads, st, pg->q, pg->row_ptr, pg->col, pg->theta, d_data, c, inv_lq,
+                       pr, ratio, coef, part, d_loss, pg->h_scal, first, ticket);
+        } else {
+            k_obj_ratio<2><<<grid, kThreads, 0, st>>>(pg->q, pg->vol, d_data, pr, ratio, ticket);
+            launch_pdl(k_obj_residual<2>, grid, kThreads, st, pg->q, pg->row_ptr, pg->col, pg->theta, d_data, c, inv_lq,
+                       pr, ratio, coef, part, d_loss, pg->h_scal, first, ticket);
+        }
+        if (last && sgd) VGA_CUDA(cudaEventRecord(pg->have_loss, st));
+        // a launch that others follow, and the raw gradient, need the per-slot sums
+        if (!last || (!sgd && !tied)) launch_grad<GRAD_RAW>(pg, pr.l, ratio, coef, first, lr, tmin);
+        else if (!sgd) launch_grad<GRAD_TIED>(pg, pr.l, ratio, coef, first, lr, tmin);
+        else if (!tied) launch_grad<SGD_RAW>(pg, pr.l, ratio, coef, first, lr, tmin);
+        else launch_grad<SGD_TIED>(pg, pr.l, ratio, coef, first, lr, tmin);
+    }
     VGA_CHECK_LAUNCH();
-    VGA_CUDA(cudaMemcpyAsync(pg->h_scal, d_loss, sizeof(double), cudaMemcpyDeviceToHost, st));
-    VGA_CUDA(cudaStreamSynchronize(st));
+    VGA_CUDA(sgd ? cudaEventSynchronize(pg->have_loss) : cudaStreamSynchronize(st));
     if (loss) *loss = pg->h_scal[0];
     return VGA_OK;
 }
@@ -998,7 +1064,7 @@ vga_status vga_pngm_step(vga_pngm *pg, double *d_m, int64_t n_steps, int32_t sch
     cudaStream_t st = pg->stream;
     const int32_t q = pg->q;
     if (scheme == VGA_SCHEME_EXPLICIT) {
-        VGA_TRY(ensure_work(pg, 6 * (int64_t)q + kObjBlocks + 8));
+        VGA_TRY(ensure_work(pg, q));
         double *a = d_m, *b = pg->work;
         for (int64_t k = 0; k < n_steps; ++k) {
             k_scheme3<<<grid_for(q, kThreads), kThreads, 0, st>>>(q, pg->row_ptr, pg->col, pg->theta, pg->vol, c, a, b);
@@ -1062,7 +1128,7 @@ vga_status vga_pngm_objective(vga_pngm *pg, int32_t objective_kind, const double
                               const int32_t *pairs, int32_t l, double D, double dt, int32_t tied, double *loss,
                               double *d_grad) {
     if (!pg) return fail(VGA_ERR_INVALID_ARG, "pngm is NULL");
-    VGA_TRY(objective(pg, objective_kind, d_data, n_records, pairs, l, D, dt, tied != 0, loss));
+    VGA_TRY(objective(pg, objective_kind, d_data, n_records, pairs, l, D, dt, tied != 0, false, 0.0, 0.0, loss));
     if (d_grad && pg->nslots > 0)
         VGA_CUDA(cudaMemcpy(d_grad, pg->grad + (tied ? pg->nslots : 0), sizeof(double) * pg->nslots,
                             cudaMemcpyDeviceToDevice));
@@ -1075,12 +1141,7 @@ vga_status vga_pngm_sgd_step(vga_pngm *pg, int32_t objective_kind, const double 
     if (!pg) return fail(VGA_ERR_INVALID_ARG, "pngm is NULL");
     if (!(std::isfinite(lr) && lr >= 0.0)) return fail(VGA_ERR_INVALID_ARG, "lr must be finite and >= 0");
     if (std::isnan(theta_min) || theta_min == INFINITY) return fail(VGA_ERR_INVALID_ARG, "theta_min must be < +inf");
-    VGA_TRY(objective(pg, objective_kind, d_data, n_records, pairs, l, D, dt, tied != 0, loss_before));
-    if (pg->nslots > 0) {
-        k_sign_sgd<<<grid_for(pg->nslots, kThreads), kThreads, 0, pg->stream>>>(
-            pg->nslots, pg->grad + (tied ? pg->nslots : 0), pg->theta, lr, theta_min);
-        VGA_CHECK_LAUNCH();
-    }
+    VGA_TRY(objective(pg, objective_kind, d_data, n_records, pairs, l, D, dt, tied != 0, true, lr, theta_min, loss_before));
     if (!tied) pg->symmetric = false;  // a raw update may break the symmetry; re-checked by set_theta
     return VGA_OK;
 }
