@@ -210,22 +210,11 @@ vga_status vga_graph_build(const uint8_t *img, int32_t nx, int32_t ny, int32_t n
     g->nvox = nvox;
     g->flags = flags;
     g->stream = st;
-    uint8_t *d_img = nullptr;
-    vga_status s = VGA_OK;
-    if (flags & VGA_IMAGE_ON_DEVICE) {
-        s = graph_build_device(g, img, st);
-    } else {
-        s = dmalloc((void **)&d_img, (size_t)nvox, "image");
-        if (s == VGA_OK) {
-            const cudaError_t e = cudaMemcpyAsync(d_img, img, (size_t)nvox, cudaMemcpyHostToDevice, st);
-            s = e == cudaSuccess ? graph_build_device(g, d_img, st) : cuda_fail(e, "image upload", __FILE__, __LINE__);
-        }
-    }
+    vga_status s = graph_build_device(g, img, st);
     if (s == VGA_OK) {
         const cudaError_t e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) s = cuda_fail(e, "graph build", __FILE__, __LINE__);
     }
-    dfree(d_img);
     if (s != VGA_OK) {
         vga_graph_free(g);
         return s;
@@ -277,9 +266,7 @@ vga_status vga_graph_free(vga_graph *g) {
     if (!g) return VGA_OK;
     VGA_TRY(release_status("error pending before vga_graph_free"));
     if (g->stream) cudaStreamSynchronize(g->stream);
-    dfree(g->labels);
-    dfree(g->mask);
-    dfree(g->pre);
+    dfree(g->labels);  // with mask and pre
     delete g;
     return release_status("vga_graph_free");
 }
@@ -300,13 +287,22 @@ vga_status vga_sim_create(const vga_graph *g, const vga_params *p, void *stream,
     vga_status st = VGA_OK;
     const size_t bytes = sizeof(float) * 5 * (size_t)std::max<int64_t>(s->npad, 64);
     const size_t lbytes = sizeof(res_t) * 5 * (size_t)std::max<int64_t>(s->npad, 64);
-    for (int b = 0; b < 2 && st == VGA_OK; ++b) st = dmalloc((void **)&s->buf[b], bytes, "state");
-    for (int b = 0; b < 2 && st == VGA_OK; ++b) st = dmalloc((void **)&s->lbuf[b], lbytes, "state residuals");
-    if (st == VGA_OK) st = dmalloc((void **)&s->partials, sizeof(double) * 5 * (size_t)totals_blocks(), "partials");
-    if (st == VGA_OK) st = dmalloc((void **)&s->d_totals, sizeof(double) * 8, "totals");
-    if (st == VGA_OK) st = dmalloc((void **)&s->d_err, sizeof(int32_t) * 4, "error flag");
+    // one allocation (see Parts), what starts at zero first
+    Parts parts;
+    parts.add(bytes);
+    const size_t at_buf1 = parts.add(bytes);
+    const size_t at_lbuf[2] = {parts.add(lbytes), parts.add(lbytes)};
+    const size_t at_err = parts.add(sizeof(int32_t) * 4), zeroed = parts.bytes;
+    const size_t at_partials = parts.add(sizeof(double) * 5 * (size_t)totals_blocks());
+    const size_t at_totals = parts.add(sizeof(double) * 8);
+    st = dmalloc((void **)&s->buf[0], parts.bytes, "state");
     if (st == VGA_OK) {
-        const cudaError_t e = cudaMemsetAsync(s->d_err, 0, sizeof(int32_t) * 4, s->stream);
+        s->buf[1] = part_at<float>(s->buf[0], at_buf1);
+        for (int b = 0; b < 2; ++b) s->lbuf[b] = part_at<res_t>(s->buf[0], at_lbuf[b]);
+        s->d_err = part_at<int32_t>(s->buf[0], at_err);
+        s->partials = part_at<double>(s->buf[0], at_partials);
+        s->d_totals = part_at<double>(s->buf[0], at_totals);
+        const cudaError_t e = cudaMemsetAsync(s->buf[0], 0, zeroed, s->stream);
         if (e != cudaSuccess) st = cuda_fail(e, "cudaMemsetAsync", __FILE__, __LINE__);
     }
     if (st == VGA_OK) {
@@ -314,11 +310,6 @@ vga_status vga_sim_create(const vga_graph *g, const vga_params *p, void *stream,
         if (e != cudaSuccess) st = cuda_fail(e, "cudaMallocHost", __FILE__, __LINE__);
     }
     if (st == VGA_OK) st = build_chunks(g->topo(), kDefaultCap, &s->chunks, s->stream);
-    for (int b = 0; b < 2 && st == VGA_OK; ++b) {
-        cudaError_t e = cudaMemsetAsync(s->buf[b], 0, bytes, s->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(s->lbuf[b], 0, lbytes, s->stream);
-        if (e != cudaSuccess) st = cuda_fail(e, "cudaMemsetAsync", __FILE__, __LINE__);
-    }
     if (st == VGA_OK) {
         const cudaError_t e = cudaStreamSynchronize(s->stream);
         if (e != cudaSuccess) st = cuda_fail(e, "sim create", __FILE__, __LINE__);
@@ -769,13 +760,7 @@ vga_status vga_sim_free(vga_sim *s) {
         cudaEventDestroy(p.b);
     }
     for (auto e : s->event_pool) cudaEventDestroy(e);
-    dfree(s->buf[0]);
-    dfree(s->buf[1]);
-    dfree(s->lbuf[0]);
-    dfree(s->lbuf[1]);
-    dfree(s->partials);
-    dfree(s->d_totals);
-    dfree(s->d_err);
+    dfree(s->buf[0]);  // with the other buffers that vga_sim_create carved from it
     dfree(s->nbr_table);
     step_graphs_free(s);
     small_free(s);

@@ -328,22 +328,34 @@ void free_chunks(Chunks *ch) {
     ch->count = 0;
 }
 
-// Builds the graph into g (fields nx, ny, nz, flags set by the caller).  d_img is a device image.
-vga_status graph_build_device(vga_graph *g, const uint8_t *d_img, cudaStream_t st) {
+// Builds the graph into g (fields nx, ny, nz, flags set by the caller) from an image on the device or, without
+// VGA_IMAGE_ON_DEVICE, on the host.  Two allocations of size: the graph's and the build's (see Parts).
+vga_status graph_build_device(vga_graph *g, const uint8_t *img, cudaStream_t st) {
     const int64_t nvox = g->nvox;
     const int64_t nrows = (int64_t)g->ny * g->nz;
     const int32_t W = (g->nx + 31) / 32;
     const int64_t nwords_lin = (nvox + 31) / 32;
     const int64_t nwords_row = nrows * W;
 
-    int32_t *err = nullptr, *root_rank = nullptr, *scratch = nullptr, *size = nullptr;
-    uint32_t *root_bits = nullptr;
-    unsigned long long *best = nullptr;
-    int32_t *h_small = nullptr;
+    const size_t scr = std::max(scan_scratch_ints(nwords_lin), scan_scratch_ints(nwords_row));
+    const bool upload = !(g->flags & VGA_IMAGE_ON_DEVICE);
+    Parts keep, tmp;
+    keep.add(sizeof(int32_t) * (size_t)nvox);  // labels
+    const size_t at_mask = keep.add(sizeof(uint32_t) * (size_t)std::max<int64_t>(nwords_row, 1));
+    const size_t at_pre = keep.add(sizeof(int32_t) * (size_t)(nwords_row + 1));
+    const size_t at_bits = tmp.add(sizeof(uint32_t) * (size_t)(nwords_lin + 1));
+    const size_t at_rank = tmp.add(sizeof(int32_t) * (size_t)(nwords_lin + 1));
+    const size_t at_scratch = tmp.add(sizeof(int32_t) * scr);
+    const size_t flag_bytes = sizeof(unsigned long long) + sizeof(int32_t) * 4;
+    const size_t at_flags = tmp.add(flag_bytes);
+    const size_t at_img = upload ? tmp.add((size_t)nvox) : 0;
+
+    void *work = nullptr;
+    int32_t *size = nullptr;
     vga_status status = VGA_OK;
     auto cleanup = [&]() {
-        dfree(err); dfree(root_rank); dfree(scratch); dfree(size); dfree(root_bits); dfree(best);
-        if (h_small) cudaFreeHost(h_small);
+        dfree(work);
+        dfree(size);
     };
 #define STEP(expr)                  \
     do {                            \
@@ -363,18 +375,21 @@ vga_status graph_build_device(vga_graph *g, const uint8_t *d_img, cudaStream_t s
         }                                                             \
     } while (0)
 
-    STEP(dmalloc((void **)&g->labels, sizeof(int32_t) * (size_t)nvox, "labels"));
-    STEP(dmalloc((void **)&g->mask, sizeof(uint32_t) * (size_t)std::max<int64_t>(nwords_row, 1), "node mask"));
-    STEP(dmalloc((void **)&g->pre, sizeof(int32_t) * (size_t)(nwords_row + 1), "node prefix"));
-    STEP(dmalloc((void **)&err, sizeof(int32_t) * 4, "flags"));
-    STEP(dmalloc((void **)&root_bits, sizeof(uint32_t) * (size_t)(nwords_lin + 1), "root bits"));
-    STEP(dmalloc((void **)&root_rank, sizeof(int32_t) * (size_t)(nwords_lin + 1), "root ranks"));
-    const size_t scr = std::max(scan_scratch_ints(nwords_lin), scan_scratch_ints(nwords_row));
-    STEP(dmalloc((void **)&scratch, sizeof(int32_t) * scr, "scan scratch"));
-    STEP(dmalloc((void **)&best, sizeof(unsigned long long), "largest"));
-    STEPC(cudaMallocHost((void **)&h_small, sizeof(int32_t) * 8));
-    STEPC(cudaMemsetAsync(err, 0, sizeof(int32_t) * 4, st));
-    STEPC(cudaMemsetAsync(best, 0, sizeof(unsigned long long), st));
+    STEP(dmalloc((void **)&g->labels, keep.bytes, "graph"));
+    g->mask = part_at<uint32_t>(g->labels, at_mask);
+    g->pre = part_at<int32_t>(g->labels, at_pre);
+    STEP(dmalloc(&work, tmp.bytes, "graph build"));
+    uint32_t *root_bits = part_at<uint32_t>(work, at_bits);
+    int32_t *root_rank = part_at<int32_t>(work, at_rank), *scratch = part_at<int32_t>(work, at_scratch);
+    unsigned long long *best = part_at<unsigned long long>(work, at_flags);  // the largest component
+    int32_t *err = reinterpret_cast<int32_t *>(best + 1);
+    const uint8_t *d_img = img;
+    if (upload) {
+        uint8_t *d = part_at<uint8_t>(work, at_img);
+        STEPC(cudaMemcpyAsync(d, img, (size_t)nvox, cudaMemcpyHostToDevice, st));
+        d_img = d;
+    }
+    STEPC(cudaMemsetAsync(best, 0, flag_bytes, st));
 
     const unsigned gv = grid_for(nvox, kThreads);
     k_init_labels<<<gv, kThreads, 0, st>>>(d_img, g->nx, nvox, g->labels);
@@ -385,6 +400,7 @@ vga_status graph_build_device(vga_graph *g, const uint8_t *d_img, cudaStream_t s
     k_root_bits<<<gv, kThreads, 0, st>>>(g->labels, nvox, root_bits);
     STEPC(cudaGetLastError());
     STEP(scan_popc(root_bits, nwords_lin, root_rank, scratch, st));
+    int32_t h_small[2] = {0, 0};
     STEPC(cudaMemcpyAsync(h_small, root_rank + nwords_lin, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
     STEPC(cudaMemcpyAsync(h_small + 1, err, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
     STEPC(cudaStreamSynchronize(st));

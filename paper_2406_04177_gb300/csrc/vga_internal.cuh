@@ -172,6 +172,20 @@ struct DevBuf {
 };
 
 vga_status dmalloc(void **p, size_t bytes, const char *what);
+// Parts of one allocation, each 256-byte aligned.  An allocation above 2 MB takes 80 to 110 us, whatever its size, and
+// its release nearly as much, so what lives and dies together is allocated together.
+struct Parts {
+    size_t bytes = 0;
+    size_t add(size_t count) {  // the part's offset
+        const size_t at = bytes;
+        bytes += (count + 255) & ~(size_t)255;
+        return at;
+    }
+};
+template <typename T>
+T *part_at(void *base, size_t offset) {
+    return reinterpret_cast<T *>(static_cast<char *>(base) + offset);
+}
 void dfree(void *p);
 
 // Exclusive prefix sum of popcount(words[q]) over q in [0, nwords): out[q], out[nwords] = total.
@@ -200,7 +214,7 @@ struct vga_graph {
     int32_t n_components = 0;
     int32_t largest = -1;
     uint32_t flags = 0;
-    int32_t *labels = nullptr;  // device, nvox
+    int32_t *labels = nullptr;  // device, nvox; the allocation that holds mask and pre too
     uint32_t *mask = nullptr;   // device, nrows*W
     int32_t *pre = nullptr;     // device, nrows*W + 1
     cudaStream_t stream = nullptr;
@@ -224,7 +238,7 @@ struct vga_sim {
     cudaStream_t stream = nullptr;
     int64_t n = 0;
     int64_t npad = 0;         // row stride of the state arrays (multiple of 64 floats)
-    float *buf[2] = {nullptr, nullptr};     // two state buffers of 5*npad FP32 values
+    float *buf[2] = {nullptr, nullptr};     // two state buffers of 5*npad FP32 values (buf[0]: see vga_sim_create)
     vga::res_t *lbuf[2] = {nullptr, nullptr};  // their residuals (compensated precision)
     int cur[5] = {0, 0, 0, 0, 0};           // which buffer holds compartment c
     StepGraph step_graphs[4];               // graphs of whole explicit step calls (small graphs)
