@@ -974,8 +974,9 @@ static SparseRecord sparse_record(const AdjointBuffers *a, int64_t j) {
 template <int WM, int PREC>
 static void launch_sparse_rec(vga_sim *s, const NbrTable &tb, const BlockTable &bt, const StateIO &io,
                               const SparseState &ss, const SparseRecord &rec, int pass, cudaStream_t st) {
-    auto kern = tb.tz ? (sparse_streams(s->n) ? k_sparse_pass_rec<WM, PREC, 1, true> : k_sparse_pass_rec<WM, PREC, 1, false>)
-                      : (sparse_streams(s->n) ? k_sparse_pass_rec<WM, PREC, 0, true> : k_sparse_pass_rec<WM, PREC, 0, false>);
+    const bool str = sparse_streams(s->n, WM == W_BLOCK, true);
+    auto kern = tb.tz ? (str ? k_sparse_pass_rec<WM, PREC, 1, true> : k_sparse_pass_rec<WM, PREC, 1, false>)
+                      : (str ? k_sparse_pass_rec<WM, PREC, 0, true> : k_sparse_pass_rec<WM, PREC, 0, false>);
     launch_pdl(kern, grid_for(s->n, kSparseNodes), kSparseThreads, st, s->n, tb, bt, s->sp, io, ss, rec, sparse_ahead(pass));
 }
 

@@ -392,7 +392,7 @@ vga_status launch_batch(vga_batch *b, int32_t pass0, int32_t pass1, int32_t npas
 // One sparse fused pass, reading state buffer bi.
 template <int TR, int PREC>
 void launch_sparse_pass_t(const vga_batch *b, const BatchArgs &a, int bi, cudaStream_t st) {
-    const bool str = sparse_streams(b->total);
+    const bool str = sparse_streams(b->total, false, false);
     auto kern = b->tz ? (str ? k_batch_sparse_pass<TR, PREC, 1, true> : k_batch_sparse_pass<TR, PREC, 1, false>)
                       : (str ? k_batch_sparse_pass<TR, PREC, 0, true> : k_batch_sparse_pass<TR, PREC, 0, false>);
     launch_pdl(kern, (unsigned)((b->total + kSparseNodes - 1) / kSparseNodes), kSparseThreads, st, a, bi, sparse_ahead(bi));

@@ -15,7 +15,7 @@
 // the marked nodes' DOM (a 32-byte sector of each array per node).
 // What bounds it: at 512^3 the compulsory 20 B per node (12 DOM + 8 table) would take 62 us at the
 // measured copy rate; issue slots are half busy, the L1 pipe 55%; the rest is the latency of two
-// dependent trips to memory per block (streams, then the gathers).  So above kSparseStreamNodes, where
+// dependent trips to memory per block (streams, then the gathers).  So above kSparseStreamBytes, where
 // the pass does not stay in L2:
 //   - thread 0 prefetches the streams of the block kSparseAhead blocks further on into L2 (about
 //     two thirds of the resident blocks, so it arrives before that block starts), and the lines its
@@ -68,13 +68,17 @@ __device__ __forceinline__ void l2_prefetch(const void *p, uint32_t bytes) {
 __device__ __forceinline__ void l2_prefetch_line(const void *p) {
     asm volatile("prefetch.global.L2 [%0];" ::"l"(__cvta_generic_to_global(p)) : "memory");
 }
-constexpr int64_t kSparseStreamNodes = (int64_t)5 << 20;  // 20 B per node above 3/4 of the 129 MB L2
+constexpr int64_t kSparseStreamBytes = (int64_t)100 << 20;  // what a pass touches above 3/4 of the 129 MB L2
 constexpr int kSparseAhead = 608;
 
 // Prefetch distance of pass number `pass` of an AHEAD launch in blocks; negative: the pass takes its
 // blocks in descending order.
 inline int sparse_ahead(int64_t pass) { return (pass & 1) ? -kSparseAhead : kSparseAhead; }
-inline bool sparse_streams(int64_t n) { return n >= kSparseStreamNodes; }
+// Per node: DOM in and out 12 B, offsets 8, the block word of W_BLOCK 4, the record 4 (320^3 at 17%, block
+// conductances: forward sweep with its recorded steps 50.4 -> 46.8 us a step from the prefetch, 296^3 42.2 -> 41.1).
+inline bool sparse_streams(int64_t n, bool block, bool rec) {
+    return n * (20 + 4 * (int)block + 4 * (int)rec) >= kSparseStreamBytes;
+}
 
 // Record of a sparse pass for the discrete adjoint: the transformed DOM of every node (h + l) and X^k
 // (MB, DOM, SOM, FOM) of the marked nodes in rank order, row q at xc + q * xcap.

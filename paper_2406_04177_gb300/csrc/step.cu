@@ -638,7 +638,8 @@ template <int MODE, int WM, int TR, int PREC, int TF, int K>
 void launch_tablev_t(vga_sim *s, const StateIO &io, const NbrTable &tb, const BlockTable &bt) {
     if constexpr (MODE == 1 && K == 4) {
         if (s->sparse_call) {
-            launch_pdl(sparse_streams(s->n) ? k_sparse_pass<WM, TR, PREC, TF, true> : k_sparse_pass<WM, TR, PREC, TF, false>,
+            const bool str = sparse_streams(s->n, WM == W_BLOCK, false);
+            launch_pdl(str ? k_sparse_pass<WM, TR, PREC, TF, true> : k_sparse_pass<WM, TR, PREC, TF, false>,
                        grid_for(s->n, kSparseNodes), kSparseThreads, s->stream, s->n, tb, bt, s->sp, io, sparse_state(s),
                        sparse_ahead(s->cur[1]));
             return;
