@@ -112,10 +112,7 @@ static vga_status harvest_timing(vga_sim *s) {
 }
 
 // Reads the device error flag written by bounded waits; a nonzero value means a kernel gave up.
-static vga_status check_device_error(vga_sim *s) {
-    int32_t h = 0;
-    VGA_CUDA(cudaMemcpyAsync(&h, s->d_err, sizeof(int32_t), cudaMemcpyDeviceToHost, s->stream));
-    VGA_CUDA(cudaStreamSynchronize(s->stream));
+static vga_status device_error(vga_sim *s, int32_t h) {
     if (h != 0) {
         cudaMemsetAsync(s->d_err, 0, sizeof(int32_t), s->stream);
         small_reset(s);
@@ -124,6 +121,12 @@ static vga_status check_device_error(vga_sim *s) {
                                               : "a bounded device wait timed out (bulk copy did not complete)");
     }
     return VGA_OK;
+}
+
+static vga_status check_device_error(vga_sim *s) {
+    VGA_CUDA(cudaMemcpyAsync(&s->report->err, s->d_err, sizeof(int32_t), cudaMemcpyDeviceToHost, s->stream));
+    VGA_CUDA(cudaStreamSynchronize(s->stream));
+    return device_error(s, s->report->err);
 }
 
 static bool finite_nonneg(double v) { return std::isfinite(v) && v >= 0.0; }
@@ -294,19 +297,17 @@ vga_status vga_sim_create(const vga_graph *g, const vga_params *p, void *stream,
     const size_t at_lbuf[2] = {parts.add(lbytes), parts.add(lbytes)};
     const size_t at_err = parts.add(sizeof(int32_t) * 4), zeroed = parts.bytes;
     const size_t at_partials = parts.add(sizeof(double) * 5 * (size_t)totals_blocks());
-    const size_t at_totals = parts.add(sizeof(double) * 8);
     st = dmalloc((void **)&s->buf[0], parts.bytes, "state");
     if (st == VGA_OK) {
         s->buf[1] = part_at<float>(s->buf[0], at_buf1);
         for (int b = 0; b < 2; ++b) s->lbuf[b] = part_at<res_t>(s->buf[0], at_lbuf[b]);
         s->d_err = part_at<int32_t>(s->buf[0], at_err);
         s->partials = part_at<double>(s->buf[0], at_partials);
-        s->d_totals = part_at<double>(s->buf[0], at_totals);
         const cudaError_t e = cudaMemsetAsync(s->buf[0], 0, zeroed, s->stream);
         if (e != cudaSuccess) st = cuda_fail(e, "cudaMemsetAsync", __FILE__, __LINE__);
     }
     if (st == VGA_OK) {
-        const cudaError_t e = cudaMallocHost((void **)&s->h_totals, sizeof(double) * 8);
+        const cudaError_t e = cudaMallocHost((void **)&s->report, sizeof(TotalsReport));
         if (e != cudaSuccess) st = cuda_fail(e, "cudaMallocHost", __FILE__, __LINE__);
     }
     if (st == VGA_OK) st = build_chunks(g->topo(), kDefaultCap, &s->chunks, s->stream);
@@ -625,8 +626,9 @@ vga_status vga_sim_step(vga_sim *s, int64_t n_steps) {
 
 vga_status vga_sim_totals(vga_sim *s, double *totals) {
     if (!s || !totals) return fail(VGA_ERR_INVALID_ARG, "sim or totals is NULL");
-    VGA_TRY(sim_totals(s, totals));
-    return check_device_error(s);
+    int32_t err = 0;
+    VGA_TRY(sim_totals(s, totals, &err));
+    return device_error(s, err);
 }
 
 vga_status vga_sim_sync(vga_sim *s) {
@@ -769,7 +771,7 @@ vga_status vga_sim_free(vga_sim *s) {
     dfree(s->bnode);
     dfree(s->bface);
     dfree(s->btheta6);
-    if (s->h_totals) cudaFreeHost(s->h_totals);
+    if (s->report) cudaFreeHost(s->report);
     dfree(s->stage);
     dfree(s->theta);
     dfree(s->cg);

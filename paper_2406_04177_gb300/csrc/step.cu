@@ -496,8 +496,12 @@ template <int PREC>
 // fraction of its FP32 rate, and the FP64 form took 0.8 ms for 21 M nodes.
 // The same pass scans the state: flags bit 0 is set when a value is not finite, bit 1 when one is
 // negative (the schemes keep every compartment >= 0 within the stability bound).
-__global__ void __launch_bounds__(kThreads) k_totals(int64_t n, StateIO io, double *__restrict__ partials,
-                                                     int32_t *__restrict__ flags) {
+// The last block to finish sums the blocks in block order and writes the totals, the flags and the error flag of
+// bounded waits to the host's memory: the call is one launch and one synchronisation (31,000 nodes: 40.4 us as two
+// launches, three copies and two synchronisations, 22.0 now).
+// dev: error flag, scan flags, ticket.
+__global__ void __launch_bounds__(kThreads) k_totals(int64_t n, StateIO io, double *partials, int32_t *dev,
+                                                     TotalsReport *report) {
     float sh[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f}, sl[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
     uint32_t f = 0u;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -513,23 +517,32 @@ __global__ void __launch_bounds__(kThreads) k_totals(int64_t n, StateIO io, doub
         }
     }
     f = __reduce_or_sync(0xffffffffu, f);
-    if ((threadIdx.x & 31) == 0 && f) atomicOr(flags, (int32_t)f);
+    if ((threadIdx.x & 31) == 0 && f) atomicOr(dev + 1, (int32_t)f);
     double s[5];
 #pragma unroll
     for (int c = 0; c < 5; ++c) s[c] = (double)sh[c] + (double)sl[c];
     __shared__ double out[5];
     block_sum_store<5>(s, out);
     if (threadIdx.x < 5) partials[(int64_t)blockIdx.x * 5 + threadIdx.x] = out[threadIdx.x];
-}
-
-__global__ void __launch_bounds__(kThreads) k_totals_final(const double *__restrict__ partials, int nblocks,
-                                                           double *__restrict__ out) {
-    double s[5] = {0, 0, 0, 0, 0};
-    for (int b = threadIdx.x; b < nblocks; b += blockDim.x)
-        for (int c = 0; c < 5; ++c) s[c] += partials[(int64_t)b * 5 + c];
-    __shared__ double o[5];
-    block_sum_store<5>(s, o);
-    if (threadIdx.x < 5) out[threadIdx.x] = o[threadIdx.x];
+    __shared__ bool last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(reinterpret_cast<uint32_t *>(dev + 2), 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+#pragma unroll
+    for (int c = 0; c < 5; ++c) s[c] = 0.0;
+    for (uint32_t b = threadIdx.x; b < gridDim.x; b += blockDim.x)
+#pragma unroll
+        for (int c = 0; c < 5; ++c) s[c] += __ldcg(partials + (int64_t)b * 5 + c);
+    block_sum_store<5>(s, out);
+    if (threadIdx.x < 5) report->total[threadIdx.x] = out[threadIdx.x];
+    if (threadIdx.x == 0) {
+        report->err = __ldcg(dev);
+        report->flags = __ldcg(dev + 1);
+        dev[2] = 0;
+    }
 }
 
 // ---- conversions ---------------------------------------------------------------------------
@@ -1113,7 +1126,8 @@ static vga_status step_body(vga_sim *s, int64_t n_steps, bool sparse) {
     return VGA_OK;
 }
 
-vga_status sim_totals(vga_sim *s, double *h_out) {
+vga_status sim_totals(vga_sim *s, double *h_out, int32_t *err) {
+    *err = 0;
     if (s->n == 0) {
         for (int c = 0; c < 5; ++c) h_out[c] = 0.0;
         return VGA_OK;
@@ -1121,21 +1135,17 @@ vga_status sim_totals(vga_sim *s, double *h_out) {
     const int nb = (int)std::min<int64_t>(kTotBlocks, (int64_t)grid_for(s->n, kThreads));
     StateIO io = state_io(s);
     timing_begin(s, VGA_KERNEL_TOTALS);
-    int32_t *flags = s->d_err + 1;  // state scan of the totals pass
-    if (s->precision() == P_COMP) k_totals<P_COMP><<<nb, kThreads, 0, s->stream>>>(s->n, io, s->partials, flags);
-    else k_totals<P_F32><<<nb, kThreads, 0, s->stream>>>(s->n, io, s->partials, flags);
-    k_totals_final<<<1, kThreads, 0, s->stream>>>(s->partials, nb, s->d_totals);
+    if (s->precision() == P_COMP) k_totals<P_COMP><<<nb, kThreads, 0, s->stream>>>(s->n, io, s->partials, s->d_err, s->report);
+    else k_totals<P_F32><<<nb, kThreads, 0, s->stream>>>(s->n, io, s->partials, s->d_err, s->report);
     timing_end(s);
     VGA_CHECK_LAUNCH();
-    s->launches += 2;
-    int32_t *h_flags = reinterpret_cast<int32_t *>(s->h_totals + 6);
-    VGA_CUDA(cudaMemcpyAsync(s->h_totals, s->d_totals, 5 * sizeof(double), cudaMemcpyDeviceToHost, s->stream));
-    VGA_CUDA(cudaMemcpyAsync(h_flags, flags, sizeof(int32_t), cudaMemcpyDeviceToHost, s->stream));
+    ++s->launches;
     VGA_CUDA(cudaStreamSynchronize(s->stream));
-    for (int c = 0; c < 5; ++c) h_out[c] = s->h_totals[c];
-    if (*h_flags) {
-        const int32_t fl = *h_flags;
-        VGA_CUDA(cudaMemsetAsync(flags, 0, sizeof(int32_t), s->stream));
+    *err = s->report->err;
+    for (int c = 0; c < 5; ++c) h_out[c] = s->report->total[c];
+    if (s->report->flags) {
+        const int32_t fl = s->report->flags;
+        VGA_CUDA(cudaMemsetAsync(s->d_err + 1, 0, sizeof(int32_t), s->stream));
         VGA_CUDA(cudaStreamSynchronize(s->stream));
         if (fl & 2) ++s->negative_reports;
         if (fl & 1) return fail(VGA_ERR_NONFINITE, "the state holds a non-finite mass (found by the totals pass)");

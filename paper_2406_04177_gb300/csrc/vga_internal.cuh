@@ -104,6 +104,12 @@ struct StepParams {
 // Stored residual of a compensated value: the BF16 bits of its value (physics.cuh).
 typedef uint16_t res_t;
 
+// What the device tells the host at the end of a totals pass or an error check.
+struct TotalsReport {
+    double total[5];
+    int32_t err, flags;
+};
+
 // Input and output compartment arrays of one pass over the state.
 struct StateIO {
     const float *in[5];   // FP32 values
@@ -258,8 +264,7 @@ struct vga_sim {
     // reductions
     double *partials = nullptr;  // per-block FP64 partial sums
     int64_t partials_cap = 0;
-    double *d_totals = nullptr;  // 8 doubles (device)
-    double *h_totals = nullptr;  // pinned host mirror
+    vga::TotalsReport *report = nullptr;  // pinned: what the totals pass and the error checks report to the host
     // staging for FP64 input/output
     double *stage = nullptr;
     // implicit-scheme work vectors (FP64), allocated on first use
@@ -296,7 +301,7 @@ struct vga_sim {
     bool timing_hold = false;      // inside a span timed as a whole (per-launch events off)
     // adjoint work buffers (adjoint.cu), allocated on first use
     vga::AdjointBuffers *adj = nullptr;
-    int32_t *d_err = nullptr;     // device error flag of bounded waits (nonzero: timed out)
+    int32_t *d_err = nullptr;     // device error flag of bounded waits (nonzero: timed out), flags and ticket of k_totals
     int kernel_variant = 5;       // explicit stencil: 0 decode + direct loads, 1 decode + staged, 2 table,
                                   // 3 table passes as an L2 wavefront (wave.cu), 4 / 5 table, two /
                                   // four nodes per thread
@@ -340,7 +345,7 @@ vga_status sim_prepare_params(vga_sim *s, const vga_params *p);
 void step_graphs_free(vga_sim *s);
 vga_status sim_step_explicit(vga_sim *s, int64_t n_steps);
 vga_status sim_diffuse_pass(vga_sim *s);  // last pass of a step call (DOM diffusion only)
-vga_status sim_totals(vga_sim *s, double *h_out);
+vga_status sim_totals(vga_sim *s, double *h_out, int32_t *err);  // err: the device error flag
 vga_status sim_convert_in(vga_sim *s, const double *d_x);    // device FP64 (5 x n) -> state
 vga_status sim_convert_out(vga_sim *s, double *d_x);         // state -> device FP64 (5 x n)
 vga_status sim_pack_f32(vga_sim *s, float *d_x, bool to_state);
