@@ -202,8 +202,8 @@ __global__ void __launch_bounds__(kSparseThreads, 5)
 }
 
 // Block sums of K compensated per-thread accumulators into out[0..K) (FP64, by thread 0 .. K-1): a
-// warp butterfly of the (sum, error) pairs in FP32, merged by TwoSum at each level, then one FP64
-// conversion per value and warp and the warps' sums in FP64.  The FP64 work is a few instructions
+// reduction over the warp (warp_sums: the bits of a butterfly, a quarter of its steps) of the (sum, error)
+// pairs in FP32, merged by TwoSum at each level, then one FP64 conversion and the warps' sums in FP64.  The FP64 work is a few instructions
 // per warp instead of five FP64 shuffle-adds per value and thread, which at one warp-group of nodes
 // per thread (small graphs) cost more than the step itself.
 template <int K>
@@ -211,22 +211,18 @@ __device__ __forceinline__ void block_sum_cacc(const CAcc (&a)[K], double *out) 
     __shared__ double sh[K][32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int nw = (blockDim.x + 31) >> 5;
-    double mine = 0.0;
+    const CAcc w = warp_sums<16>(a, [](CAcc x, CAcc y) {
+        CAcc r;
+        r.s = __fadd_rn(x.s, y.s);
+        const float bp = __fsub_rn(r.s, x.s);
+        const float err = __fadd_rn(__fsub_rn(x.s, __fsub_rn(r.s, bp)), __fsub_rn(y.s, bp));
+        r.c = __fadd_rn(__fadd_rn(x.c, y.c), err);
+        return r;
+    });
+    const double mine = (double)w.s + (double)w.c;
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-        float s = a[k].s, c = a[k].c;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const float s2 = __shfl_xor_sync(0xffffffffu, s, o), c2 = __shfl_xor_sync(0xffffffffu, c, o);
-            const float t = __fadd_rn(s, s2);
-            const float bp = __fsub_rn(t, s);
-            const float err = __fadd_rn(__fsub_rn(s, __fsub_rn(t, bp)), __fsub_rn(s2, bp));
-            s = t;
-            c = __fadd_rn(__fadd_rn(c, c2), err);
-        }
-        if (lane == k) mine = (double)s + (double)c;  // every lane holds the warp's pair
-    }
-    if (lane < K) sh[lane][wid] = mine;
+    for (int k = 0; k < K; ++k)
+        if (lane == warp_sum_lane(K, k)) sh[k][wid] = mine;
     __syncthreads();
     if (threadIdx.x < K) {
         double b = 0.0;

@@ -27,6 +27,13 @@ __device__ __forceinline__ void cacc_add_prod(CAcc &a, float x, float y) {
     a.c = __fadd_rn(a.c, e);
 }
 
+__device__ __forceinline__ CAcc shfl_value(CAcc a, int o) {
+    CAcc b;
+    b.s = __shfl_xor_sync(0xffffffffu, a.s, o);
+    b.c = __shfl_xor_sync(0xffffffffu, a.c, o);
+    return b;
+}
+
 // FP32 value as FP64, built with integer operations: exact for normal values, infinities and NaN;
 // subnormal values (below 2^-126 in magnitude) become zeros of their sign.  The conversion
 // instruction would issue on the FP64 pipe, which GB300 runs at a small fraction of its FP32 rate.

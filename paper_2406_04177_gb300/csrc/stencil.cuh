@@ -172,17 +172,54 @@ __device__ __forceinline__ double warp_sum_d(double v) {
     return v;
 }
 
-// Block-wide sum of K doubles per thread; thread 0 writes the K results to out[0..K).
+// K sums over a warp at once.  A butterfly per value takes 5 K additions, of which only one lane's results are wanted;
+// here a step halves the values a lane carries instead: lanes with bit O keep the upper half of the values and send the
+// lower one, so K values take K / 2 + K / 4 + ... additions (12 for 9, 8 for 5).  Each sum's tree, and so its bits, are
+// the butterfly's.  join(a, b) adds and must commute; the sum of value k ends up in lane warp_sum_lane(K, k).
+__device__ __forceinline__ double shfl_value(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+
+constexpr int warp_sum_lane(int K, int k) {
+    int lane = 0;
+    for (int o = 16; o > 0; o >>= 1) {
+        const int h = (K + 1) / 2;
+        if (k >= h) {
+            lane |= o;
+            k -= h;
+        }
+        K = h;
+    }
+    return lane;
+}
+
+template <int O, int K, class T, class Join>
+__device__ __forceinline__ T warp_sums(const T (&v)[K], Join join) {
+    if constexpr (O == 0) {
+        static_assert(K == 1, "at most 32 values");
+        return v[0];
+    } else {
+        constexpr int H = (K + 1) / 2;
+        const bool upper = K > 1 && (threadIdx.x & O);
+        T w[H];
+#pragma unroll
+        for (int k = 0; k < H; ++k) {
+            const T lo = v[k], hi = K == 1 ? v[k] : H + k < K ? v[H + k] : T{};
+            w[k] = join(upper ? hi : lo, shfl_value(K == 1 ? lo : upper ? lo : hi, O));
+        }
+        return warp_sums<O / 2>(w, join);
+    }
+}
+
+// Block-wide sum of K doubles per thread; the first K threads write the results to out[0..K).  The block is a multiple
+// of 32 threads.
 template <int K>
 __device__ __forceinline__ void block_sum_store(const double (&v)[K], double *out) {
     __shared__ double sh[K][32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int nw = (blockDim.x + 31) >> 5;
+    const double w = warp_sums<16>(v, [](double a, double b) { return a + b; });
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-        const double w = warp_sum_d(v[k]);
-        if (lane == 0) sh[k][wid] = w;
-    }
+    for (int k = 0; k < K; ++k)
+        if (lane == warp_sum_lane(K, k)) sh[k][wid] = w;
     __syncthreads();
     if (threadIdx.x < K) {
         double b = 0.0;

@@ -20,6 +20,7 @@
 #include <cmath>
 #include <cstring>
 
+#include "adjoint_sums.cuh"
 #include "pdl.cuh"
 #include "physics.cuh"
 #include "small_graph.cuh"
@@ -489,7 +490,12 @@ __global__ void k_table_pack_z(int64_t n, const uint32_t *__restrict__ tzm, cons
 }
 
 // ---- FP64 totals ---------------------------------------------------------------------------
-template <int PREC>
+// FP32 as FP64 by integer operations where they give it (the conversion instruction issues at the FP64 rate).
+__device__ __forceinline__ double f32_to_f64(float f) {
+    const uint32_t u = __float_as_uint(f) & 0x7fffffffu;
+    return u != 0u && u < 0x00800000u ? (double)f : f32_to_f64_alu(f);  // subnormal
+}
+
 // Each thread sums its nodes in float-float (TwoSum of the high parts; the low parts and the sum
 // errors added in FP32), about 2^-48 relative for the tens of terms a thread takes; threads and
 // blocks are summed in FP64.  No FP64 arithmetic per node: the FP64 rate of this part is a small
@@ -499,28 +505,40 @@ template <int PREC>
 // The last block to finish sums the blocks in block order and writes the totals, the flags and the error flag of
 // bounded waits to the host's memory: the call is one launch and one synchronisation (31,000 nodes: 40.4 us as two
 // launches, three copies and two synchronisations, 22.0 now).
+// A thread takes K nodes at a time: four, in wide loads, where every thread of the grid has that many, so that no
+// thread's float-float sum is longer than with one.  On graphs where a thread has a node or two the block's 64-bit
+// additions and conversions were most of the kernel (25 + 15 a warp; see warp_sums, f32_to_f64): TOT2.
 // dev: error flag, scan flags, ticket.
+template <int PREC, int K>
 __global__ void __launch_bounds__(kThreads) k_totals(int64_t n, StateIO io, double *partials, int32_t *dev,
                                                      TotalsReport *report) {
     float sh[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f}, sl[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
     uint32_t f = 0u;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    auto add = [&](int c, const V &v) {
+        f |= ((__float_as_uint(v.h) & 0x7f800000u) == 0x7f800000u ? 1u : 0u) | (v.h < 0.0f ? 2u : 0u);
+        const float t = __fadd_rn(sh[c], v.h);
+        const float bb = __fsub_rn(t, sh[c]);
+        const float e = __fadd_rn(__fsub_rn(sh[c], __fsub_rn(t, bb)), __fsub_rn(v.h, bb));
+        sh[c] = t;
+        sl[c] = __fadd_rn(sl[c], __fadd_rn(e, v.l));
+    };
+    const int64_t groups = (n + K - 1) / K;
+    for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < groups; g += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t i0 = (uint32_t)(K * g);
 #pragma unroll
         for (int c = 0; c < 5; ++c) {
-            const V v = vload<PREC>(io.in[c], io.lin[c], i);
-            f |= ((__float_as_uint(v.h) & 0x7f800000u) == 0x7f800000u ? 1u : 0u) | (v.h < 0.0f ? 2u : 0u);
-            const float t = __fadd_rn(sh[c], v.h);
-            const float bb = __fsub_rn(t, sh[c]);
-            const float e = __fadd_rn(__fsub_rn(sh[c], __fsub_rn(t, bb)), __fsub_rn(v.h, bb));
-            sh[c] = t;
-            sl[c] = __fadd_rn(sl[c], __fadd_rn(e, v.l));
+            V v[K];
+            if (K > 1 && i0 + K <= n) vload_k<PREC, K, true>(io.in[c], io.lin[c], i0, (uint32_t)n, v);
+            else vload_k<PREC, K, false>(io.in[c], io.lin[c], i0, (uint32_t)n, v);
+#pragma unroll
+            for (int k = 0; k < K; ++k) add(c, v[k]);
         }
     }
     f = __reduce_or_sync(0xffffffffu, f);
     if ((threadIdx.x & 31) == 0 && f) atomicOr(dev + 1, (int32_t)f);
     double s[5];
 #pragma unroll
-    for (int c = 0; c < 5; ++c) s[c] = (double)sh[c] + (double)sl[c];
+    for (int c = 0; c < 5; ++c) s[c] = f32_to_f64(sh[c]) + f32_to_f64(sl[c]);
     __shared__ double out[5];
     block_sum_store<5>(s, out);
     if (threadIdx.x < 5) partials[(int64_t)blockIdx.x * 5 + threadIdx.x] = out[threadIdx.x];
@@ -1135,8 +1153,10 @@ vga_status sim_totals(vga_sim *s, double *h_out, int32_t *err) {
     const int nb = (int)std::min<int64_t>(kTotBlocks, (int64_t)grid_for(s->n, kThreads));
     StateIO io = state_io(s);
     timing_begin(s, VGA_KERNEL_TOTALS);
-    if (s->precision() == P_COMP) k_totals<P_COMP><<<nb, kThreads, 0, s->stream>>>(s->n, io, s->partials, s->d_err, s->report);
-    else k_totals<P_F32><<<nb, kThreads, 0, s->stream>>>(s->n, io, s->partials, s->d_err, s->report);
+    const bool wide = s->n >= (int64_t)4 * kTotBlocks * kThreads;
+    auto kern = s->precision() == P_COMP ? (wide ? k_totals<P_COMP, 4> : k_totals<P_COMP, 1>)
+                                         : (wide ? k_totals<P_F32, 4> : k_totals<P_F32, 1>);
+    kern<<<nb, kThreads, 0, s->stream>>>(s->n, io, s->partials, s->d_err, s->report);
     timing_end(s);
     VGA_CHECK_LAUNCH();
     ++s->launches;
