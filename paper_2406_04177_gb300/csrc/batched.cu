@@ -641,8 +641,8 @@ vga_status vga_batch_create(const vga_graph *const *graphs, const vga_params *pa
     }
     for (int k = 0; k < count && st == VGA_OK; ++k) {
         const int64_t s0 = b->start[k];
-        st = build_nbr_table(graphs[k]->topo(), b->table + s0, b->table + b->npad + s0, b->table + 2 * b->npad + s0,
-                             b->stream);
+        st = build_nbr_table(graphs[k]->topo(), nullptr, b->table + s0, b->table + b->npad + s0,
+                             b->table + 2 * b->npad + s0, nullptr, b->stream);
     }
     // padding entries between instances are zero, so the compact form covers the whole range
     if (st == VGA_OK) st = build_compact_z(b->npad, b->npad, b->table + b->npad, b->table + 2 * b->npad, &b->tz, b->stream);

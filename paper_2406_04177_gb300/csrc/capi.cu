@@ -766,7 +766,7 @@ vga_status vga_sim_free(vga_sim *s) {
     dfree(s->nbr_table);
     step_graphs_free(s);
     small_free(s);
-    dfree(s->nbr_tz);
+    dfree(s->nbr_tz_own);
     activity_free(&s->act);
     dfree(s->bnode);
     dfree(s->bface);

@@ -348,14 +348,16 @@ vga_status graph_build_device(vga_graph *g, const uint8_t *img, cudaStream_t st)
     const size_t at_scratch = tmp.add(sizeof(int32_t) * scr);
     const size_t flag_bytes = sizeof(unsigned long long) + sizeof(int32_t) * 4;
     const size_t at_flags = tmp.add(flag_bytes);
-    const size_t at_img = upload ? tmp.add((size_t)nvox) : 0;
+    // the uploaded image, then the component sizes: room for nvox / 8 of them (more are allocated on their own)
+    const size_t img_bytes = (size_t)(upload ? nvox : (nvox + 1) / 2);
+    const size_t at_img = tmp.add(img_bytes);
 
     void *work = nullptr;
-    int32_t *size = nullptr;
+    int32_t *size = nullptr, *own_size = nullptr;
     vga_status status = VGA_OK;
     auto cleanup = [&]() {
         dfree(work);
-        dfree(size);
+        dfree(own_size);
     };
 #define STEP(expr)                  \
     do {                            \
@@ -407,8 +409,14 @@ vga_status graph_build_device(vga_graph *g, const uint8_t *img, cudaStream_t st)
     if (h_small[1]) STEP(fail(VGA_ERR_CUDA, "graph build: union-find retry bound exceeded"));
     const int32_t ncomp = h_small[0];
     g->n_components = ncomp;
-    STEP(dmalloc((void **)&size, sizeof(int32_t) * (size_t)std::max(ncomp, 1), "component sizes"));
-    STEPC(cudaMemsetAsync(size, 0, sizeof(int32_t) * (size_t)std::max(ncomp, 1), st));
+    const size_t size_bytes = sizeof(int32_t) * (size_t)std::max(ncomp, 1);
+    if (size_bytes <= img_bytes) {
+        size = part_at<int32_t>(work, at_img);
+    } else {
+        STEP(dmalloc((void **)&own_size, size_bytes, "component sizes"));
+        size = own_size;
+    }
+    STEPC(cudaMemsetAsync(size, 0, size_bytes, st));
     k_label<<<grid_for(nvox, kThreads * kLabelItems), kThreads, 0, st>>>(nvox, g->labels, root_bits, root_rank, size);
     if (ncomp > 0) k_largest<<<grid_for(ncomp, kThreads), kThreads, 0, st>>>(size, ncomp, best);
     STEPC(cudaGetLastError());

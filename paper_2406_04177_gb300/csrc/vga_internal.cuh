@@ -315,6 +315,7 @@ struct vga_sim {
     int32_t wave_reach = 0;
     uint32_t *nbr_table = nullptr;  // 3 x npad words (NbrTable), built on first use
     uint32_t *nbr_tz = nullptr;     // compact z offsets (NbrTable.tz) when they fit in 16 bits
+    uint32_t *nbr_tz_own = nullptr;  // its allocation, unless it is the table's fourth row
     int nbr_tz_state = 0;           // 0 not examined, 1 built, 2 offsets too large
     uint32_t *bnode = nullptr;      // BlockTable.node (npad), built for the current block side
     int32_t *bface = nullptr;       // BlockTable.face (6 x blocks)
@@ -373,7 +374,9 @@ bool wave_params_valid(int chunk, int depth, int ctas_per_sm);
 vga_status sim_block_table(vga_sim *s, BlockTable *out, bool *ok);
 // Writes the neighbour-offset table of a node set (offsets are relative, so the arrays may start at
 // any node offset of a larger concatenated range).  Synchronises the stream.
-vga_status build_nbr_table(const Topo &t, uint32_t *ty, uint32_t *tzm, uint32_t *tzp, cudaStream_t st);
+// (with the chunks of the caller when they have the right size; tz: the compact z offsets too, or NULL)
+vga_status build_nbr_table(const Topo &t, const Chunks *have, uint32_t *ty, uint32_t *tzm, uint32_t *tzp, uint32_t *tz,
+                           cudaStream_t st);
 // Compact z offsets (NbrTable.tz) of a table of n entries (allocating cap entries) when every z
 // offset is below 2^16; *out stays NULL otherwise.
 vga_status build_compact_z(int64_t n, int64_t cap, const uint32_t *tzm, const uint32_t *tzp, uint32_t **out,
