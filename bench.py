@@ -109,7 +109,7 @@ def load_peaks():
 
 def kernel_source_hash() -> str:
     h = hashlib.sha256()
-    for name in ("step.cu", "stencil.cuh", "physics.cuh", "vga_internal.cuh"):
+    for name in ("step.cu", "sparse_pass.cuh", "stencil.cuh", "physics.cuh", "vga_internal.cuh"):
         with open(os.path.join(ROOT, "paper_2406_04177_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]
@@ -350,7 +350,8 @@ def bench_ours(a):
     kname = {0: "k_stencil (chunk decode, direct loads)", 1: "k_stencil_staged (chunk decode, bulk-copy staging)",
              2: "k_stencil_table (neighbour-offset table)",
              4: "k_stencil_tablev (neighbour-offset table, two nodes per thread, 8-byte vector streams)",
-             5: "k_stencil_tablev (neighbour-offset table, four nodes per thread, 16-byte vector streams)",
+             5: ("k_sparse_pass" if sparse else "k_stencil_tablev")
+                + " (neighbour-offset table, four nodes per thread, 16-byte vector streams)",
              6: "k_dom_block (temporally blocked: tiles of 32x16x16 voxels with a 3-voxel halo in shared memory, "
                 "up to 3 fused passes per launch; tile-order permutation of the DOM per step call included)",
              3: f"k_wave (neighbour-offset table; {S - 1} fused passes per persistent launch as an L2 wavefront, "

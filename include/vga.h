@@ -321,10 +321,12 @@ vga_status vga_sim_set_kernel(vga_sim *s, int32_t variant, int32_t chunk);
  * transformation is the identity, and it stays so while stepping (no flux can make them nonzero).
  * The first step after a state upload (vga_sim_set_masses, vga_sim_set_state_f32,
  * vga_sim_load_state) marks the other nodes in a bit mask (one extra pass, one synchronisation); a
- * fused pass then diffuses the DOM of every node, transforms only the marked nodes (a second kernel
- * over them in rank order, their MB, SOM, FOM and CO2 held in a compact rank-ordered copy during the
- * call), and leaves the MB, SOM, FOM and CO2 of the others unread and unwritten.  Results are bit-identical with the mask off (also a node whose values are negative
- * zeros is marked).  on = 0 transforms every node every pass. */
+ * fused pass then diffuses the DOM of every node, transforms only the marked nodes (their MB, SOM, FOM
+ * and CO2 held in a compact rank-ordered copy during the call), and leaves the MB, SOM, FOM and CO2 of
+ * the others unread and unwritten.  A call whose mask marks five eighths of the nodes or more runs dense
+ * passes; on graphs of up to 0.3 M nodes a call's passes are one launch.  Results are bit-identical with the
+ * mask off (also a node whose values are negative zeros is marked).  on = 0 transforms every node every
+ * pass. */
 vga_status vga_sim_set_activity_skip(vga_sim *s, int32_t on);
 
 /* Selects variant 3 with `chunk` nodes per work item (a power of two in [256, 8192]; CTAs of

@@ -13,8 +13,9 @@
 // This is the multi-step, transformation-coupled form of the closed-form gradients of Sec. V.A.
 //
 // Memory: the forward stores the state every `ckpt` steps; each segment is recomputed once from
-// its checkpoint, recording X^k (FP32) and the transformed DOM y2^k, and then reversed step by
-// step.  The adjoint state is carried like the forward state (FP32 value + BF16 residual) and every
+// its checkpoint, recording X^k (FP32; of the marked nodes only in a sparse sweep) and the transformed DOM
+// y2^k, and then reversed step by step: k_adjoint_vec, or without dL/dX^0 the lean kernels below, or on
+// small graphs one launch per segment (small_graph.cu).  The adjoint state is carried like the forward state (FP32 value + BF16 residual) and every
 // parameter gradient is accumulated in FP64 (per-block partials, FP64 atomics for the faces).
 #include <cuda_runtime.h>
 

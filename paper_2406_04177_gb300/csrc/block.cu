@@ -19,8 +19,8 @@
 // launch of S passes recomputes the nodes of rows within distance S - s of the tile (the halo
 // shrinks by one voxel per pass, so every value it reads is exact), and the marked nodes of the
 // sparse pass (MB, SOM, FOM or CO2 nonzero) are transformed from a list in shared memory.  Per node
-// the arithmetic is that of the two-kernel sparse pass (stencil.cuh MODE 4, then
-// k_transform_compact), so the results are the same bits for finite states.
+// the arithmetic is that of the sparse pass (sparse_pass.cuh), so the results are the same bits for finite
+// states.
 //
 // Tiles whose tile-plus-halo node count exceeds the capacity of the two-blocks-per-SM instance run
 // in a second launch with twice the capacity (one block per SM).

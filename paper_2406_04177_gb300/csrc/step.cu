@@ -10,9 +10,10 @@
 // Every intermediate Y already holds the transformed DOM that the neighbours read, so each fused
 // pass reads and writes the 5-compartment state once, and N steps cost N+1 passes.
 //
-// The stencil kernel works on chunks of `cap` consecutive nodes; decode_chunk() (stencil.cuh)
-// turns the row bitmask into per-node neighbour indices in shared memory, so no per-node
-// neighbour table is read from memory.
+// The default kernels read a table of neighbour offsets, four consecutive nodes per thread: dense passes
+// here (k_stencil_tablev), sparse ones in sparse_pass.cuh, the calls of small graphs as one launch in
+// small_graph.cu.  k_stencil works on chunks of `cap` consecutive nodes instead: decode_chunk()
+// (stencil.cuh) turns the row bitmask into per-node neighbour indices in shared memory.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -510,7 +511,8 @@ __device__ __forceinline__ double f32_to_f64(float f) {
 // launches, three copies and two synchronisations, 22.0 now).
 // A thread takes K nodes at a time: four, in wide loads, where every thread of the grid has that many, so that no
 // thread's float-float sum is longer than with one.  On graphs where a thread has a node or two the block's 64-bit
-// additions and conversions were most of the kernel (25 + 15 a warp; see warp_sums, f32_to_f64): TOT2.
+// additions and conversions were most of the kernel (25 and 15 a warp, now 13 and none: warp_sums, f32_to_f64).  A call
+// at 298,000 nodes 40.6 -> 30.4 us, 2.4 M 47.6 -> 35.9, 20.8 M 210.4 -> 170.7 (93 at the copy rate).
 // dev: error flag, scan flags, ticket.
 template <int PREC, int K>
 __global__ void __launch_bounds__(kThreads) k_totals(int64_t n, StateIO io, double *partials, int32_t *dev,

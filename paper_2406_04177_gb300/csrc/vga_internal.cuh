@@ -134,7 +134,7 @@ struct SparseState {
 // stepping), the marked nodes before each mask word, and the compact state they use during a step
 // call.  One per simulation or batch; built per state upload.
 struct Activity {
-    uint32_t *words = nullptr;  // nw mask words, nw prefix words, then a 64-bit counter
+    uint32_t *words = nullptr;  // nw mask words, nw prefix words, four words the build reports, its tile sums
     int64_t nw = 0;
     char *state = nullptr;      // compact MB, SOM, FOM, CO2: 4 x cap values, 4 x cap residuals, cap nodes
     int64_t cap = 0;
@@ -277,7 +277,7 @@ struct vga_sim {
     bool mx_graph_failed = false;  // graph construction failed once: host-driven loop from then on
     void *mx_graph = nullptr;      // cached graphs of the mixed solve (pcg.cu)
     int64_t graph_launches = 0;    // CUDA graph launches of the mixed solve
-    // Sparse fused pass (stencil.cuh MODE 4 and the marked-node half): activity mask and compact state
+    // Sparse fused pass (sparse_pass.cuh): activity mask and compact state
     vga::Activity act;
     bool activity_skip = true;     // use it (vga_sim_set_activity_skip)
     bool sparse_call = false;      // the fused passes of the running step call are sparse
