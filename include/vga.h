@@ -329,6 +329,15 @@ vga_status vga_sim_set_kernel(vga_sim *s, int32_t variant, int32_t chunk);
  * pass. */
 vga_status vga_sim_set_activity_skip(vga_sim *s, int32_t on);
 
+/* Test hook of the bounded waits (no counterpart in the paper).  The blocks of a small-graph launch
+ * (see vga_sim_set_activity_skip) wait for one another's values, each wait bounded.  With skip_block
+ * >= 0, block skip_block of every such launch leaves before it publishes anything, so the waits of the
+ * blocks beside it (where the graph takes several blocks of 512, 1024 or 2048 nodes) run out after
+ * spin_limit rounds (0: the default limit); the launch then ends, the next call that synchronises
+ * returns VGA_ERR_TIMEOUT, and the state is undefined until the next upload.  skip_block = -1
+ * switches the hook off (spin_limit still applies).  Nothing faults, traps or hangs. */
+vga_status vga_sim_set_wait_test(vga_sim *s, int32_t skip_block, uint32_t spin_limit);
+
 /* Selects variant 3 with `chunk` nodes per work item (a power of two in [256, 8192]; CTAs of
  * min(chunk, 1024) threads), `depth`
  * passes per block of the skewed order (1..64: the passes whose intermediate states stay in L2),
@@ -517,6 +526,12 @@ vga_status vga_pngm_restrict(vga_pngm *pg, vga_sim *s, int32_t comp, double *d_o
  * iterate), VGA_ERR_CUDA. */
 vga_status vga_pngm_step(vga_pngm *pg, double *d_m, int64_t n_steps, int32_t scheme, double D, double dt, double cg_rtol,
                          int32_t cg_maxit);
+
+/* Test hook of the bounded waits (no counterpart in the paper), as vga_sim_set_wait_test: the blocks of
+ * a Scheme 4 launch wait for one another's values; block skip_block (-1: none) leaves first, and
+ * vga_pngm_step returns VGA_ERR_TIMEOUT once a wait of spin_limit polls (0: the default limit) has run
+ * out; the masses are undefined then. */
+vga_status vga_pngm_set_wait_test(vga_pngm *pg, int32_t skip_block, uint32_t spin_limit);
 
 /* Objective 1 or 2 (objective_kind) over the l pairs X^p = record pairs[2p], Y^p = record
  * pairs[2p+1] of d_data (device, FP64, n_records x q, row-major); pairs is a host array of 2l

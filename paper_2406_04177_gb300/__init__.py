@@ -144,6 +144,8 @@ _SIGNATURES = {
     "vga_batch_free": [_P],
     "vga_state_totals_noalloc": [_P, _P, _I64, _I64, _P, _P],
     "vga_batch_set_wait_test": [_P, _I32, C.c_uint32],
+    "vga_sim_set_wait_test": [_P, _I32, C.c_uint32],
+    "vga_pngm_set_wait_test": [_P, _I32, C.c_uint32],
     "vga_sim_set_face_conductances": [_P, _P],
     "vga_pngm_create": [_P, _P, _I32, _I32, _P, _P],
     "vga_pngm_get_info": [_P, _P],
@@ -484,6 +486,16 @@ def vga_batch_set_wait_test(b, skip_block: int, spin_limit: int = 0):
     _check(load_library().vga_batch_set_wait_test(b, int(skip_block), int(spin_limit)), "vga_batch_set_wait_test")
 
 
+def vga_sim_set_wait_test(s, skip_block: int, spin_limit: int = 0):
+    """Bounded-wait test hook of the small-graph launches; skip_block = -1 switches it off."""
+    _check(load_library().vga_sim_set_wait_test(s, int(skip_block), int(spin_limit)), "vga_sim_set_wait_test")
+
+
+def vga_pngm_set_wait_test(h, skip_block: int, spin_limit: int = 0):
+    """Bounded-wait test hook of the Scheme 4 launches; skip_block = -1 switches it off."""
+    _check(load_library().vga_pngm_set_wait_test(h, int(skip_block), int(spin_limit)), "vga_pngm_set_wait_test")
+
+
 def vga_state_totals_noalloc(values, residuals, n: int, row_stride: int, totals, stream=None):
     """values / residuals / totals are CUDA tensors (float32; 16-bit residual bits or None;
     float64 with at least 5 entries), contiguous; compartment c occupies
@@ -696,6 +708,10 @@ class Sim:
     def set_activity_skip(self, on: bool):
         vga_sim_set_activity_skip(self.handle, on)
 
+    def set_wait_test(self, skip_block: int, spin_limit: int = 0):
+        """Bounded-wait test hook (vga_sim_set_wait_test); skip_block = -1 switches it off."""
+        vga_sim_set_wait_test(self.handle, skip_block, spin_limit)
+
     def set_wavefront(self, chunk: int, depth: int, ctas_per_sm: int = 0):
         vga_sim_set_wavefront(self.handle, chunk, depth, ctas_per_sm)
 
@@ -906,6 +922,10 @@ class Pngm:
 
     def step(self, m, n_steps: int, scheme: int, D: float, dt: float, cg_rtol: float = 1e-12, cg_maxit: int = 10000):
         return vga_pngm_step(self.handle, m, self.q, n_steps, scheme, D, dt, cg_rtol, cg_maxit)
+
+    def set_wait_test(self, skip_block: int, spin_limit: int = 0):
+        """Bounded-wait test hook (vga_pngm_set_wait_test); skip_block = -1 switches it off."""
+        vga_pngm_set_wait_test(self.handle, skip_block, spin_limit)
 
     def objective(self, kind: int, data, pairs, D: float, dt: float, tied: bool = False, grad=None) -> float:
         return vga_pngm_objective(self.handle, self.q, self.n_slots, kind, data, pairs, D, dt, tied, grad)

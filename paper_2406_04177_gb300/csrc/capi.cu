@@ -608,6 +608,14 @@ vga_status vga_sim_set_activity_skip(vga_sim *s, int32_t on) {
     return VGA_OK;
 }
 
+vga_status vga_sim_set_wait_test(vga_sim *s, int32_t skip_block, uint32_t spin_limit) {
+    if (!s) return fail(VGA_ERR_INVALID_ARG, "sim is NULL");
+    if (skip_block < -1) return fail(VGA_ERR_INVALID_ARG, "skip_block must be -1 or a block index");
+    s->wait_test_block = skip_block;
+    s->wait_test_spin = spin_limit;
+    return VGA_OK;
+}
+
 vga_status vga_sim_set_solver(vga_sim *s, int32_t solver) {
     if (!s) return fail(VGA_ERR_INVALID_ARG, "sim is NULL");
     if (solver != VGA_SOLVER_FP64_PCG && solver != VGA_SOLVER_MIXED_REFINEMENT && solver != VGA_SOLVER_MIXED_HOST_LOOP)

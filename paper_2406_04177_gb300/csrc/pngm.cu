@@ -52,6 +52,8 @@ struct vga_pngm {
     cudaEvent_t have_loss = nullptr;  // the loss of an SGD step is in h_scal
     unsigned long long *fx = nullptr;  // restriction: fixed-point sums (q), scale (2), partials
     bool symmetric = true;       // theta_ij == theta_ji for every pair
+    int32_t wait_test_block = -1;  // vga_pngm_set_wait_test
+    uint32_t wait_test_spin = 0;
     // host copies of the geometry (export)
     std::vector<double> h_vol, h_cen, h_S, h_dist;
     std::vector<int32_t> h_row_ptr, h_col, h_rev;
@@ -394,7 +396,7 @@ __global__ void __launch_bounds__(kThreads) k_scheme3(int32_t q, const int32_t *
 // are spread over every SM (in one block a solve at q = 32,632 took 4.9 ms, nearly all of it FP64 issue on
 // one SM).  A block owns contiguous rows; u, r, p and the inverse diagonal stay in the global work vectors,
 // read and written by the row's own thread.  What crosses blocks, the entries of u or p that rows
-// multiply and the partial sums of the dot products, is exchanged as tagged words (double_words): the
+// multiply and the partial sums of the dot products, is exchanged as tagged words (st_double, ld_double): the
 // reader polls the word itself, so an iteration costs three trips through L2 (p, p.Ap, r.z with r.r) and
 // no barrier.  Every block adds the blocks' partial sums in block order, so all hold the same bits and
 // decide alike, and a run is deterministic.  Waits are bounded: one that gives up sets *err and the blocks
@@ -414,6 +416,8 @@ struct PcgArgs {
     int64_t n_steps;
     double *stats;               // iterations, relative residual, converged
     int32_t *err;
+    int32_t skip_block;          // test of the bounded waits: this block leaves before it publishes anything (-1: none)
+    uint32_t spin_limit;         // polls of a word before a wait gives up
 };
 
 // A double as two words of 32 bits of it and a 32-bit tag each; either may arrive first.
@@ -423,14 +427,14 @@ __device__ __forceinline__ void st_double(unsigned long long *w, double v, uint3
     st_word_raw(w + 1, t | (b >> 32));
 }
 
-__device__ __forceinline__ bool ld_double(const unsigned long long *w, uint32_t tag, double &v, const int32_t *err) {
-    for (uint32_t it = 0; it < kPcgSpin; ++it) {
+__device__ __forceinline__ bool ld_double(const PcgArgs &p, const unsigned long long *w, uint32_t tag, double &v) {
+    for (uint32_t it = 0; it < p.spin_limit; ++it) {
         const unsigned long long a = ld_word(w), b = ld_word(w + 1);
         if ((uint32_t)(a >> 32) == tag && (uint32_t)(b >> 32) == tag) {
             v = __longlong_as_double((long long)((b << 32) | (a & 0xffffffffull)));
             return true;
         }
-        if ((it & 1023u) == 1023u && *(volatile const int32_t *)err) break;
+        if ((it & 1023u) == 1023u && *(volatile const int32_t *)p.err) break;
     }
     v = 0.0;
     return false;
@@ -456,9 +460,9 @@ __device__ __forceinline__ bool grid_sum2(const PcgArgs &a, uint32_t tag, double
     double px = 0.0, py = 0.0;
     for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) {  // at most one per thread (grid <= SMs <= 256)
         double v;
-        ok &= ld_double(slots + 4 * (size_t)b, tag, v, a.err);
+        ok &= ld_double(a, slots + 4 * (size_t)b, tag, v);
         px += v;
-        ok &= ld_double(slots + 4 * (size_t)b + 2, tag, v, a.err);
+        ok &= ld_double(a, slots + 4 * (size_t)b + 2, tag, v);
         py += v;
     }
     px = warp_sum_d(px);
@@ -500,7 +504,7 @@ __device__ __forceinline__ double apply_row(const PcgArgs &a, int32_t i, double 
             if (k0 + j < k1) {
                 double xj = __longlong_as_double((long long)((hi[j] << 32) | (lo[j] & 0xffffffffull)));
                 if ((uint32_t)(lo[j] >> 32) != tag || (uint32_t)(hi[j] >> 32) != tag)
-                    ok &= ld_double(a.xw + 2 * (size_t)__ldg(a.col + k0 + j), tag, xj, a.err);
+                    ok &= ld_double(a, a.xw + 2 * (size_t)__ldg(a.col + k0 + j), tag, xj);
                 s += __ldg(a.th + k0 + j) * (xi - xj);
             }
     }
@@ -509,6 +513,7 @@ __device__ __forceinline__ double apply_row(const PcgArgs &a, int32_t i, double 
 
 __global__ void __launch_bounds__(kPcgThreads, 1) k_scheme4_pcg(PcgArgs a) {
     __shared__ double sh[64];
+    if ((int32_t)blockIdx.x == a.skip_block) return;
     const int32_t q = a.q, per = (q + (int32_t)gridDim.x - 1) / (int32_t)gridDim.x;
     const int32_t i0 = (int32_t)blockIdx.x * per + (int32_t)threadIdx.x, i1 = min((int32_t)blockIdx.x * per + per, q);
     double *u = a.w, *r = a.w + q, *p = a.w + 2 * (int64_t)q, *dinv = a.w + 3 * (int64_t)q;
@@ -1100,6 +1105,8 @@ vga_status vga_pngm_step(vga_pngm *pg, double *d_m, int64_t n_steps, int32_t sch
     a.err = reinterpret_cast<int32_t *>(a.stats + 3);
     a.maxit = cg_maxit;
     a.n_steps = n_steps;
+    a.skip_block = pg->wait_test_block;
+    a.spin_limit = pg->wait_test_spin ? pg->wait_test_spin : kPcgSpin;
     VGA_CUDA(cudaMemsetAsync(a.xw, 0, sizeof(double) * (size_t)(words + 8), st));
     if (n_steps > 0) {
         cudaLaunchConfig_t cfg = {};
@@ -1121,6 +1128,14 @@ vga_status vga_pngm_step(vga_pngm *pg, double *d_m, int64_t n_steps, int32_t sch
     pg->last_iters = (int64_t)pg->h_scal[0];
     pg->last_relres = pg->h_scal[1];
     if (n_steps > 0 && pg->h_scal[2] == 0.0) return fail(VGA_ERR_NOT_CONVERGED, "Scheme 4 solve reached cg_maxit before cg_rtol");
+    return VGA_OK;
+}
+
+vga_status vga_pngm_set_wait_test(vga_pngm *pg, int32_t skip_block, uint32_t spin_limit) {
+    if (!pg) return fail(VGA_ERR_INVALID_ARG, "pngm is NULL");
+    if (skip_block < -1) return fail(VGA_ERR_INVALID_ARG, "skip_block must be -1 or a block index");
+    pg->wait_test_block = skip_block;
+    pg->wait_test_spin = spin_limit;
     return VGA_OK;
 }
 

@@ -54,6 +54,8 @@ struct SmallArgs {
     unsigned long long *pub;
     int32_t *err;
     const uint32_t *prefix, *mask, *list;  // of the marked nodes
+    int32_t skip_block;   // test of the bounded waits: this block leaves before it publishes anything (-1: none)
+    uint32_t spin_limit;  // rounds of loads before a wait gives up
     StepParams p;
 };
 
@@ -124,7 +126,7 @@ __device__ __forceinline__ bool gather(const SmallArgs &a, const NodeTable<K> &t
                 far.v[q] = __uint_as_float((uint32_t)w[q]);
                 pending &= ~(1u << q);
             }
-        gave_up = it > kSmallSpin || ((it & 1023u) == 1023u && *(volatile int32_t *)a.err != 0);
+        gave_up = it > a.spin_limit || ((it & 1023u) == 1023u && *(volatile int32_t *)a.err != 0);
     }
     if (pending) {
         atomicExch(a.err, 3);
@@ -227,6 +229,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_forward(SmallArgs a,
     extern __shared__ float sg[];  // W_BLOCK: conductances, 6 K rows
     const uint32_t tid = threadIdx.x, v0 = blockIdx.x * (kSmallThreads * K), i0 = v0 + tid;
     const int64_t npad = a.npad;
+    if ((int32_t)blockIdx.x == a.skip_block) return;
     NodeTable<K> t;
     t.load(a, i0);
     if (WM == W_BLOCK) load_conductances<K>(a, t, i0, sg, nullptr);  // read by the thread that wrote them
@@ -401,6 +404,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_reverse(SmallArgs a,
     // first) add both nodes' terms, the second's handed over by a shuffle (shared memory).  Otherwise per thread.
     int64_t slot = (int64_t)blockIdx.x * kSmallThreads + tid;
     const StepParams &p = a.p;
+    if ((int32_t)blockIdx.x == a.skip_block) return;
     NodeTable<K> t;
     t.load(a, i0);
     if (WM == W_BLOCK) load_conductances<K>(a, t, i0, sg, sf);  // read by the thread that wrote them
@@ -670,6 +674,8 @@ vga_status small_args(vga_sim *s, const Activity &act, SmallArgs *a, SmallWork *
     a->prefix = ss.prefix;
     a->mask = ss.mask;
     a->list = ss.list;
+    a->skip_block = s->wait_test_block;
+    a->spin_limit = s->wait_test_spin ? s->wait_test_spin : kSmallSpin;
     a->p = s->sp;
     return VGA_OK;
 }

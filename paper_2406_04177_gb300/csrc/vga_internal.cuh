@@ -323,6 +323,8 @@ struct vga_sim {
     int64_t btheta6_gen = -1;       // param_gen btheta6 was built for
     int32_t btable_bs = 0;          // block side the block table was built for (0: none)
     void *small = nullptr;          // small-graph launches (small_graph.cu)
+    int32_t wait_test_block = -1;   // vga_sim_set_wait_test
+    uint32_t wait_test_spin = 0;
     double *loss_work = nullptr;  // block-mass objective scratch
     int64_t loss_cap = 0;
     int64_t param_gen = 0;  // bumped by every change of parameters or conductances
