@@ -214,7 +214,11 @@ vga_status vga_sim_save_state(vga_sim *s, void *buf, int64_t bytes);
 vga_status vga_sim_load_state(vga_sim *s, const void *buf, int64_t bytes);
 
 /* Advances n_steps >= 0 time steps (Sec. III: transformation, then diffusion of DOM).
- * Asynchronous on the simulation's stream.  Implicit scheme: synchronises to test convergence
+ * Asynchronous on the simulation's stream.  Explicit scheme: kernels whose blocks wait for one another
+ * (small graphs, variant 3) bound every wait; if one gives up, the next call that synchronises
+ * (vga_sim_sync, vga_sim_totals, the host forms of the read-outs, vga_sim_save_state,
+ * vga_loss_block_mass, vga_adjoint_backward, an implicit step) returns VGA_ERR_TIMEOUT once, and the state is
+ * undefined until the next upload.  Implicit scheme: synchronises to test convergence
  * and returns VGA_ERR_NOT_CONVERGED if any solve hit cg_maxit (the state then holds the last
  * iterate). */
 vga_status vga_sim_step(vga_sim *s, int64_t n_steps);
@@ -226,7 +230,8 @@ vga_status vga_sim_step(vga_sim *s, int64_t n_steps);
  * a few ulps below zero, so a negative value is reported, not an error). */
 vga_status vga_sim_totals(vga_sim *s, double *totals);
 
-/* Waits for the simulation's stream; reports errors of previously enqueued work. */
+/* Waits for the simulation's stream; reports errors of previously enqueued work (VGA_ERR_TIMEOUT: see
+ * vga_sim_step). */
 vga_status vga_sim_sync(vga_sim *s);
 
 typedef struct vga_sim_stats {
@@ -333,8 +338,8 @@ vga_status vga_sim_set_activity_skip(vga_sim *s, int32_t on);
  * (see vga_sim_set_activity_skip) wait for one another's values, each wait bounded.  With skip_block
  * >= 0, block skip_block of every such launch leaves before it publishes anything, so the waits of the
  * blocks beside it (where the graph takes several blocks of 512, 1024 or 2048 nodes) run out after
- * spin_limit rounds (0: the default limit); the launch then ends, the next call that synchronises
- * returns VGA_ERR_TIMEOUT, and the state is undefined until the next upload.  skip_block = -1
+ * spin_limit rounds (0: the default limit); the launch then ends and VGA_ERR_TIMEOUT is reported as
+ * vga_sim_step says.  skip_block = -1
  * switches the hook off (spin_limit still applies).  Nothing faults, traps or hangs. */
 vga_status vga_sim_set_wait_test(vga_sim *s, int32_t skip_block, uint32_t spin_limit);
 
@@ -523,7 +528,8 @@ vga_status vga_pngm_restrict(vga_pngm *pg, vga_sim *s, int32_t comp, double *d_o
  * ||r||_2 <= cg_rtol ||m^k||_2 or after cg_maxit iterations).  Scheme 4 needs symmetric theta.
  * Synchronises the handle's stream.  Errors: VGA_ERR_INVALID_ARG, VGA_ERR_UNSUPPORTED (Scheme 4
  * with theta_ij != theta_ji), VGA_ERR_NOT_CONVERGED (a solve hit cg_maxit; m holds its last
- * iterate), VGA_ERR_CUDA. */
+ * iterate), VGA_ERR_TIMEOUT (Scheme 4: a bounded wait between the blocks of the launch gave up; m is
+ * undefined), VGA_ERR_CUDA. */
 vga_status vga_pngm_step(vga_pngm *pg, double *d_m, int64_t n_steps, int32_t scheme, double D, double dt, double cg_rtol,
                          int32_t cg_maxit);
 

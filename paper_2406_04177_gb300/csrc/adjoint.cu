@@ -1408,19 +1408,17 @@ static vga_status adjoint_backward_impl(vga_sim *s, const double *d_lamN, double
     VGA_CHECK_LAUNCH();
     s->launches += 2;
     double h[kPar];
-    int32_t flag = 0, gave_up = 0;
+    int32_t flag = 0;
     if (flag_dev) VGA_CUDA(cudaMemcpyAsync(&flag, flag_dev, sizeof(flag), cudaMemcpyDeviceToHost, st));
-    if (small) VGA_CUDA(cudaMemcpyAsync(&gave_up, s->d_err, sizeof(gave_up), cudaMemcpyDeviceToHost, st));
+    VGA_TRY(sim_fetch_device_error(s));  // of this sweep, and of the forward one in whatever form it ran
     VGA_CUDA(cudaMemcpyAsync(h, a->gsum, sizeof(double) * kPar, cudaMemcpyDeviceToHost, st));
     if (s->face_mode) VGA_TRY(sim_face_mirror(s, a->gtheta));  // both slots of every edge
     if (h_gtheta && s->n_theta > 0 && s->wmode == W_BLOCK)
         VGA_CUDA(cudaMemcpyAsync(h_gtheta, a->gtheta, sizeof(double) * (size_t)s->n_theta, cudaMemcpyDeviceToHost, st));
     VGA_CUDA(cudaStreamSynchronize(st));
-    if (gave_up) {
-        VGA_CUDA(cudaMemsetAsync(s->d_err, 0, sizeof(int32_t), st));
-        small_reset(s);
+    if (s->report->err) {
         a->valid = false;
-        return fail(VGA_ERR_TIMEOUT, "a bounded device wait timed out (small-graph launch)");
+        return sim_device_error(s, s->report->err);
     }
     if (flag) {
         *redo = true;

@@ -111,8 +111,9 @@ static vga_status harvest_timing(vga_sim *s) {
     return VGA_OK;
 }
 
-// Reads the device error flag written by bounded waits; a nonzero value means a kernel gave up.
-static vga_status device_error(vga_sim *s, int32_t h) {
+// Reports what the device error flag of bounded waits held (nonzero: a kernel gave up) and resets what such a launch
+// leaves behind.
+vga_status sim_device_error(vga_sim *s, int32_t h) {
     if (h != 0) {
         cudaMemsetAsync(s->d_err, 0, sizeof(int32_t), s->stream);
         small_reset(s);
@@ -123,10 +124,18 @@ static vga_status device_error(vga_sim *s, int32_t h) {
     return VGA_OK;
 }
 
-static vga_status check_device_error(vga_sim *s) {
+// The flag goes to s->report->err, for a caller that synchronises later anyway.
+vga_status sim_fetch_device_error(vga_sim *s) {
     VGA_CUDA(cudaMemcpyAsync(&s->report->err, s->d_err, sizeof(int32_t), cudaMemcpyDeviceToHost, s->stream));
+    return VGA_OK;
+}
+
+// Waits for the stream; every host read-out ends with it, so that no state that a launch left unfinished is
+// returned as a result.
+static vga_status sync_checked(vga_sim *s) {
+    VGA_TRY(sim_fetch_device_error(s));
     VGA_CUDA(cudaStreamSynchronize(s->stream));
-    return device_error(s, s->report->err);
+    return sim_device_error(s, s->report->err);
 }
 
 static bool finite_nonneg(double v) { return std::isfinite(v) && v >= 0.0; }
@@ -510,8 +519,7 @@ vga_status vga_sim_get_masses(vga_sim *s, double *x, int32_t on_device) {
     VGA_TRY(ensure_stage(s));
     VGA_TRY(sim_convert_out(s, s->stage));
     VGA_CUDA(cudaMemcpyAsync(x, s->stage, sizeof(double) * 5 * (size_t)s->n, cudaMemcpyDeviceToHost, s->stream));
-    VGA_CUDA(cudaStreamSynchronize(s->stream));
-    return VGA_OK;
+    return sync_checked(s);
 }
 
 vga_status vga_sim_set_state_f32(vga_sim *s, const float *x, int32_t on_device) {
@@ -534,8 +542,7 @@ vga_status vga_sim_get_state_f32(vga_sim *s, float *x, int32_t on_device) {
     float *st = reinterpret_cast<float *>(s->stage);
     VGA_TRY(sim_pack_f32(s, st, false));
     VGA_CUDA(cudaMemcpyAsync(x, st, sizeof(float) * 5 * (size_t)s->n, cudaMemcpyDeviceToHost, s->stream));
-    VGA_CUDA(cudaStreamSynchronize(s->stream));
-    return VGA_OK;
+    return sync_checked(s);
 }
 
 namespace {
@@ -574,8 +581,7 @@ vga_status vga_sim_save_state(vga_sim *s, void *buf, int64_t bytes) {
     uint16_t *st = reinterpret_cast<uint16_t *>(s->stage);
     VGA_TRY(sim_res_export(s, st));
     VGA_CUDA(cudaMemcpyAsync(p, st, sizeof(uint16_t) * 5 * (size_t)s->n, cudaMemcpyDeviceToHost, s->stream));
-    VGA_CUDA(cudaStreamSynchronize(s->stream));
-    return VGA_OK;
+    return sync_checked(s);
 }
 
 vga_status vga_sim_load_state(vga_sim *s, const void *buf, int64_t bytes) {
@@ -628,21 +634,25 @@ vga_status vga_sim_set_solver(vga_sim *s, int32_t solver) {
 vga_status vga_sim_step(vga_sim *s, int64_t n_steps) {
     if (!s) return fail(VGA_ERR_INVALID_ARG, "sim is NULL");
     if (n_steps < 0) return fail(VGA_ERR_INVALID_ARG, "n_steps must be >= 0");
-    if (s->params.scheme == VGA_SCHEME_IMPLICIT_PCG) return sim_step_implicit(s, n_steps);
-    return sim_step_explicit(s, n_steps);
+    if (s->params.scheme != VGA_SCHEME_IMPLICIT_PCG) return sim_step_explicit(s, n_steps);
+    if (n_steps == 0 || s->n == 0) return sim_step_implicit(s, n_steps);
+    VGA_TRY(sim_fetch_device_error(s));  // of the steps before: this call synchronises
+    const vga_status st = sim_step_implicit(s, n_steps);
+    VGA_TRY(sim_device_error(s, s->report->err));
+    return st;
 }
 
 vga_status vga_sim_totals(vga_sim *s, double *totals) {
     if (!s || !totals) return fail(VGA_ERR_INVALID_ARG, "sim or totals is NULL");
     int32_t err = 0;
-    VGA_TRY(sim_totals(s, totals, &err));
-    return device_error(s, err);
+    const vga_status st = sim_totals(s, totals, &err);
+    VGA_TRY(sim_device_error(s, err));  // first: the state it left may hold anything
+    return st;
 }
 
 vga_status vga_sim_sync(vga_sim *s) {
     if (!s) return fail(VGA_ERR_INVALID_ARG, "sim is NULL");
-    VGA_CUDA(cudaStreamSynchronize(s->stream));
-    return check_device_error(s);
+    return sync_checked(s);
 }
 
 vga_status vga_sim_get_stats(vga_sim *s, vga_sim_stats *out) {
@@ -738,7 +748,9 @@ vga_status vga_loss_block_mass(vga_sim *s, int32_t block_side, uint32_t comp_mas
     }
     double *d_target = s->loss_work + 2 * count + 64;
     VGA_CUDA(cudaMemcpyAsync(d_target, target, sizeof(double) * (size_t)count, cudaMemcpyHostToDevice, s->stream));
-    return sim_block_mass_loss(s, block_side, comp_mask, d_target, s->loss_work, loss, block_mass, dL_dX);
+    VGA_TRY(sim_fetch_device_error(s));
+    VGA_TRY(sim_block_mass_loss(s, block_side, comp_mask, d_target, s->loss_work, loss, block_mass, dL_dX));
+    return sim_device_error(s, s->report->err);
 }
 
 vga_status vga_sim_enable_timing(vga_sim *s, int32_t on) {

@@ -349,6 +349,8 @@ void step_graphs_free(vga_sim *s);
 vga_status sim_step_explicit(vga_sim *s, int64_t n_steps);
 vga_status sim_diffuse_pass(vga_sim *s);  // last pass of a step call (DOM diffusion only)
 vga_status sim_totals(vga_sim *s, double *h_out, int32_t *err);  // err: the device error flag
+vga_status sim_fetch_device_error(vga_sim *s);
+vga_status sim_device_error(vga_sim *s, int32_t err);
 vga_status sim_convert_in(vga_sim *s, const double *d_x);    // device FP64 (5 x n) -> state
 vga_status sim_convert_out(vga_sim *s, double *d_x);         // state -> device FP64 (5 x n)
 vga_status sim_pack_f32(vga_sim *s, float *d_x, bool to_state);

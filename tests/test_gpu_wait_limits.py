@@ -16,8 +16,7 @@ SHAPE = (16, 16, 20)  # 10 blocks of 512 nodes
 
 
 def _masses(n, seed=3):
-    X = synth.random_masses(n, seed, density=0.1)
-    return np.ascontiguousarray(X)
+    return synth.random_masses(n, seed, density=0.03)  # at most 512 marked nodes in a block
 
 
 def _timeout(call):
@@ -100,4 +99,47 @@ def test_scheme4_wait_runs_out_and_the_handle_recovers(skip):
         out.append(m.cpu().numpy())
         h.close()
     assert np.array_equal(out[0], out[1])
+    g.close()
+
+
+READERS = {
+    "get_masses": lambda s: s.get_masses(),
+    "get_state_f32": lambda s: s.get_state_f32(),
+    "save_state": lambda s: s.save_state(),
+    "totals": lambda s: s.totals(),
+    "loss_block_mass": lambda s: s.loss_block_mass(8, 2, np.zeros(12)),
+    "implicit step": lambda s: (s.set_params(synth.paper_params(scheme=vga.VGA_SCHEME_IMPLICIT_PCG)), s.step(1)),
+}
+
+
+@pytest.mark.parametrize("reader", READERS)
+def test_host_read_outs_report_an_unfinished_step_call(reader):
+    """None of the calls that hand a result to the host may return a state that a launch left half-way."""
+    g = vga.Graph(np.zeros(SHAPE, dtype=np.uint8))
+    sim = vga.Sim(g, synth.paper_params())
+    sim.set_masses(_masses(g.n))
+    sim.set_wait_test(4, SPIN)
+    sim.step(20)
+    _timeout(lambda: READERS[reader](sim))
+    sim.sync()
+    sim.close()
+    g.close()
+
+
+@pytest.mark.parametrize("shape", [SHAPE, (64, 64, 76)])
+def test_a_sweep_by_launches_reports_an_unfinished_forward_sweep(shape):
+    """(64, 64, 76), four nodes per thread with dL/dX^0: the reverse sweep takes launches; with timing on
+    it does at every size."""
+    g = vga.Graph(np.zeros(shape, dtype=np.uint8))
+    lam = torch.ones((5, g.n), device="cuda", dtype=torch.float64)
+    sim = vga.Sim(g, synth.paper_params())
+    sim.set_masses(_masses(g.n))
+    sim.set_wait_test(4, SPIN)
+    sim.adjoint_forward(11, 4)
+    sim.set_wait_test(-1, 0)
+    sim.enable_timing(shape == SHAPE)
+    _timeout(lambda: sim.adjoint_backward(lam, torch.zeros_like(lam)))
+    with pytest.raises(vga.VgaError):  # no sweep to reverse is left
+        sim.adjoint_backward(lam)
+    sim.close()
     g.close()
