@@ -1056,7 +1056,7 @@ vga_status sim_adjoint_forward(vga_sim *s, int64_t N, int64_t ckpt) {
             a->xcap = std::max<int64_t>(a->act.n_active, 1);
         }
     }
-    const bool small = a->sparse && small_ok(s, a->act);
+    const bool small = a->sparse && small_ok(s, a->act) && std::min(ckpt, N) <= kSmallSteps;
     for (int64_t sg = 0; sg < nseg; ++sg) {
         const int64_t len = std::min(ckpt, N - sg * ckpt);
         if (small) {  // the checkpoint and the segment as one launch
@@ -1224,7 +1224,7 @@ static vga_status adjoint_backward_impl(vga_sim *s, const double *d_lamN, double
     // small graphs: a segment's recomputation and its reverse steps are one launch each
     const bool may_lean = lean && sparse && !d_lam0;
     // (with dL/dX^0 its sums are one per pair of nodes: k_adjoint_vec's, when each of its threads takes one pair)
-    const bool small = sparse && small_ok(s, a->act) && small_reverse_ok(s, !may_lean) &&
+    const bool small = sparse && small_ok(s, a->act) && std::min(ckpt, N) <= kSmallSteps && small_reverse_ok(s, !may_lean) &&
                        (may_lean || (kAdjK == 2 && (int64_t)Gt * kThreads * 2 >= s->n));
     // Above a quarter of the nodes marked a lean step moves as much as a full one (36 B per node and about
     // 120 B per marked node against 66 B per node); on small graphs its second launch costs more than it

@@ -402,7 +402,10 @@ __global__ void __launch_bounds__(kThreads) k_scheme3(int32_t q, const int32_t *
 // decide alike, and a run is deterministic.  Waits are bounded: one that gives up sets *err and the blocks
 // leave.
 constexpr int kPcgThreads = 256;
-constexpr uint32_t kPcgSpin = 1u << 21;
+constexpr uint32_t kPcgSpin = 1u << 25;  // polls, about a quarter of a minute (see kSmallSpin in small_graph.cu)
+// Steps of one launch: 36 ms at 30,719 rows and 27 iterations a step.  Other streams get the SMs in between; 256 steps
+// take 145.8 ms as one launch and as four.
+constexpr int64_t kPcgSteps = 64, kPcgRows = 32768;
 
 struct PcgArgs {
     int32_t q;
@@ -414,7 +417,7 @@ struct PcgArgs {
     unsigned long long *sw;      // 2 x grid x 4 words: partial sums of two reductions in flight
     int32_t maxit;
     int64_t n_steps;
-    double *stats;               // iterations, relative residual, converged
+    double *stats;               // iterations, the last relative residual, solves that did not converge: over the call
     int32_t *err;
     int32_t skip_block;          // test of the bounded waits: this block leaves before it publishes anything (-1: none)
     uint32_t spin_limit;         // polls of a word before a wait gives up
@@ -514,12 +517,13 @@ __device__ __forceinline__ double apply_row(const PcgArgs &a, int32_t i, double 
 __global__ void __launch_bounds__(kPcgThreads, 1) k_scheme4_pcg(PcgArgs a) {
     __shared__ double sh[64];
     if ((int32_t)blockIdx.x == a.skip_block) return;
+    if (__syncthreads_or(*(volatile int32_t *)a.err)) return;  // a launch before this one gave up
     const int32_t q = a.q, per = (q + (int32_t)gridDim.x - 1) / (int32_t)gridDim.x;
     const int32_t i0 = (int32_t)blockIdx.x * per + (int32_t)threadIdx.x, i1 = min((int32_t)blockIdx.x * per + per, q);
     double *u = a.w, *r = a.w + q, *p = a.w + 2 * (int64_t)q, *dinv = a.w + 3 * (int64_t)q;
     uint32_t xtag = 0, stag = 0;  // words are zero when the launch starts
-    double iters = 0.0, rel = 0.0;
-    bool converged = true, ok = true;
+    double iters = 0.0, rel = 0.0, failed = 0.0;
+    bool ok = true;
     for (int32_t i = i0; i < i1; i += blockDim.x) {
         double s = 0.0;
         for (int32_t k = a.rp[i]; k < a.rp[i + 1]; ++k) s += a.th[k];
@@ -580,12 +584,12 @@ __global__ void __launch_bounds__(kPcgThreads, 1) k_scheme4_pcg(PcgArgs a) {
         for (int32_t i = i0; i < i1; i += blockDim.x) a.m[i] = a.vol[i] * u[i];
         iters += (double)it;
         rel = bb > 0.0 ? sqrt(rr / bb) : 0.0;
-        if (!(rr <= tol2)) converged = false;
+        if (!(rr <= tol2)) failed += 1.0;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-        a.stats[0] = iters;
+        a.stats[0] += iters;
         a.stats[1] = rel;
-        a.stats[2] = converged ? 1.0 : 0.0;
+        a.stats[2] += failed;
     }
 }
 
@@ -1104,11 +1108,13 @@ vga_status vga_pngm_step(vga_pngm *pg, double *d_m, int64_t n_steps, int32_t sch
     a.stats = pg->work + 5 * (int64_t)q + words;
     a.err = reinterpret_cast<int32_t *>(a.stats + 3);
     a.maxit = cg_maxit;
-    a.n_steps = n_steps;
     a.skip_block = pg->wait_test_block;
     a.spin_limit = pg->wait_test_spin ? pg->wait_test_spin : kPcgSpin;
-    VGA_CUDA(cudaMemsetAsync(a.xw, 0, sizeof(double) * (size_t)(words + 8), st));
-    if (n_steps > 0) {
+    VGA_CUDA(cudaMemsetAsync(a.stats, 0, sizeof(double) * 8, st));
+    const int64_t per_launch = std::max<int64_t>(1, kPcgSteps * kPcgRows / std::max<int64_t>(q, kPcgRows));
+    for (int64_t k = 0; k < n_steps; k += per_launch) {
+        a.n_steps = std::min(per_launch, n_steps - k);
+        VGA_CUDA(cudaMemsetAsync(a.xw, 0, sizeof(double) * (size_t)words, st));
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)G);
         cfg.blockDim = dim3(kPcgThreads);
@@ -1127,7 +1133,7 @@ vga_status vga_pngm_step(vga_pngm *pg, double *d_m, int64_t n_steps, int32_t sch
     if (gave_up) return fail(VGA_ERR_TIMEOUT, "a bounded device wait timed out (Scheme 4 solve)");
     pg->last_iters = (int64_t)pg->h_scal[0];
     pg->last_relres = pg->h_scal[1];
-    if (n_steps > 0 && pg->h_scal[2] == 0.0) return fail(VGA_ERR_NOT_CONVERGED, "Scheme 4 solve reached cg_maxit before cg_rtol");
+    if (pg->h_scal[2] != 0.0) return fail(VGA_ERR_NOT_CONVERGED, "Scheme 4 solve reached cg_maxit before cg_rtol");
     return VGA_OK;
 }
 

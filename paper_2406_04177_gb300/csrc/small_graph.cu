@@ -37,7 +37,9 @@ namespace vga {
 
 namespace {
 
-constexpr uint32_t kSmallSpin = 1u << 21;  // rounds of loads before a wait gives up (about a second)
+// Rounds of loads before a wait gives up, about a quarter of a minute.  A launch whose blocks do not all find room at
+// once, because other streams' kernels hold SMs, waits in its first pass for as long as these run.
+constexpr uint32_t kSmallSpin = 1u << 25;
 
 struct SmallWork {
     int K = 0, G = 0;

@@ -7,6 +7,10 @@ namespace vga {
 
 constexpr int kSmallThreads = 512;
 constexpr int kSmallWords = kSmallThreads / 32;  // mask words of a block per node of a thread
+// Steps of one launch (19 ms at 64^3, 39 at 128^3, a reverse sweep 118): other streams get the SMs in between, and a
+// launch that shares them with this one waits far less than the limit of its waits.  65,536 steps at 64^3 take 77.6 ms
+// as one launch and as four.
+constexpr int64_t kSmallSteps = (int64_t)1 << 14;
 
 // Nodes per thread (1, 2 or 4) and blocks of a small-graph launch; false when n nodes do not fit.
 bool small_shape(int64_t n, int *K, int *G);

@@ -1073,14 +1073,17 @@ vga_status sim_step_explicit(vga_sim *s, int64_t n_steps) {
     // pass, 256^3 at 20% / 320^3 at 17%: 76% marked 35.8 / 55.0 us sparse, 32.9 / 48.3 dense; 48% marked
     // 24.4 / 42.5 sparse, 32.8 / 48.3 dense.  The line lies between, at five eighths.
     if (sparse && s->act.n_active * 8 >= s->n * 5) sparse = false;
-    if (sparse && n_steps <= (int64_t)1 << 30 && small_ok(s, s->act)) {  // the whole call as one launch
+    if (sparse && small_ok(s, s->act)) {  // the whole call as one launch, or a few
         StateRows rows;
         for (int c = 0; c < 5; ++c) {
             rows.h[c] = s->comp(c);
             rows.l[c] = s->lcomp(c);
         }
-        VGA_TRY(small_forward(s, s->act, rows, rows, StateRows{}, n_steps - 1, true, nullptr, nullptr, 0));
-        s->steps_done += n_steps;
+        for (int64_t k = 0; k < n_steps; k += kSmallSteps) {
+            const int64_t len = std::min(kSmallSteps, n_steps - k);
+            VGA_TRY(small_forward(s, s->act, rows, rows, StateRows{}, len - 1, true, nullptr, nullptr, 0));
+            s->steps_done += len;
+        }
         return VGA_OK;
     }
     if (step_graph_eligible(s, n_steps)) return step_graphed(s, n_steps, sparse);
