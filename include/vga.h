@@ -330,8 +330,9 @@ vga_status vga_sim_set_kernel(vga_sim *s, int32_t variant, int32_t chunk);
  * and CO2 held in a compact rank-ordered copy during the call), and leaves the MB, SOM, FOM and CO2 of
  * the others unread and unwritten.  A call whose mask marks five eighths of the nodes or more runs dense
  * passes; on graphs of up to 0.3 M nodes a call's passes are one launch.  Results are bit-identical with the
- * mask off (also a node whose values are negative zeros is marked).  on = 0 transforms every node every
- * pass. */
+ * mask off (also a node whose values are negative zeros is marked), as long as no mass is negative: an
+ * unmarked node whose DOM is negative transforms in the first pass of each call only.  on = 0 transforms every
+ * node every pass. */
 vga_status vga_sim_set_activity_skip(vga_sim *s, int32_t on);
 
 /* Test hook of the bounded waits (no counterpart in the paper).  The blocks of a small-graph launch

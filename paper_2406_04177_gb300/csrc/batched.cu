@@ -64,6 +64,7 @@ struct BatchArgs {
     int32_t *err;
     StateIO io[2];  // a pass whose input is state buffer k reads io[k] (kept as kernel parameters)
     SparseState ss;    // the sparse fused pass of the SPARSE instantiations (compact state, rank list)
+    int32_t others;       // sparse call: state buffer of MB, SOM, FOM and CO2 in the last pass (-1: the pass's input)
     int32_t skip_block;   // test of the bounded waits: this block leaves before any barrier (-1: none)
     uint32_t spin_limit;  // polls of a grid barrier before it gives up
 };
@@ -206,7 +207,7 @@ __global__ void __launch_bounds__(kTile, SPARSE ? 5 : 1) k_batch(BatchArgs a, in
                         vstore<PREC>(a.h[bo] + a.npad, a.l[bo] + a.npad, i, x[1]);
     #pragma unroll
                         for (int c = 0; c < 5; ++c) {
-                            if (c == 1) continue;
+                            if (c == 1 || a.others == bo) continue;
                             a.h[bo][c * a.npad + i] = a.h[bi][c * a.npad + i];
                             if (PREC == P_COMP) a.l[bo][c * a.npad + i] = a.l[bi][c * a.npad + i];
                         }
@@ -348,6 +349,7 @@ BatchArgs batch_args(const vga_batch *b) {
     a.bar = b->bar;
     a.err = b->err;
     a.ss = activity_state(b->act);
+    a.others = -1;
     a.skip_block = b->wait_test_block;
     a.spin_limit = b->wait_test_spin ? b->wait_test_spin : kBarrierSpin;
     for (int k = 0; k < 2; ++k) {
@@ -361,8 +363,9 @@ BatchArgs batch_args(const vga_batch *b) {
     return a;
 }
 
-vga_status launch_batch(vga_batch *b, int32_t pass0, int32_t pass1, int32_t npass, int32_t cur0, bool sparse) {
-    const BatchArgs a = batch_args(b);
+vga_status launch_batch(vga_batch *b, int32_t pass0, int32_t pass1, int32_t npass, int32_t cur0, bool sparse, int32_t others = -1) {
+    BatchArgs a = batch_args(b);
+    a.others = others;
     // the first and the last pass of a call need the full kernel; the others run the fused-only one
     const bool fused_only = pass0 > 0 && pass1 < npass;
     cudaLaunchConfig_t cfg = {};
@@ -451,7 +454,8 @@ StateIO batch_io(const vga_batch *b, int k) {
 }
 
 // sparse: the fused passes run sparse; the marked nodes' MB, SOM, FOM, CO2 go to the compact state
-// after the first pass and back before the last.
+// after the first pass and back before the last, into the buffer (cur0 + 1) & 1 where the first pass left every
+// node's (it may have changed them at an unmarked node whose DOM was negative).
 vga_status enqueue_steps(vga_batch *b, int64_t n_steps, int cur0, bool sparse) {
     const int64_t npass = n_steps + 1;
     const int S = persistent_steps(b);
@@ -462,10 +466,8 @@ vga_status enqueue_steps(vga_batch *b, int64_t n_steps, int cur0, bool sparse) {
         const int64_t p1 = std::min(npass - 1, p0 + S);
         VGA_TRY(launch_batch(b, (int32_t)p0, (int32_t)p1, (int32_t)npass, cur0, sparse));
     }
-    // the state after pass npass - 2 is buffer (cur0 + npass - 1) & 1: the out side of the other
-    if (sparse)
-        VGA_TRY(activity_copy(b->act, b->total, batch_io(b, 1 - (int)((cur0 + npass - 1) & 1)), false, comp, b->stream));
-    return launch_batch(b, (int32_t)(npass - 1), (int32_t)npass, (int32_t)npass, cur0, false);
+    if (sparse) VGA_TRY(activity_copy(b->act, b->total, batch_io(b, cur0 & 1), false, comp, b->stream));  // the out side
+    return launch_batch(b, (int32_t)(npass - 1), (int32_t)npass, (int32_t)npass, cur0, false, sparse ? (cur0 + 1) & 1 : -1);
 }
 
 // A call in per-pass launches: the fused passes as replays of one graph of kPassGraph passes (an even
@@ -508,9 +510,8 @@ vga_status step_per_pass(vga_batch *b, int64_t n_steps, int cur0) {
         }
     }
     VGA_TRY(launch_sparse_passes(b, left, bi, b->stream));
-    // the state after pass npass - 2 is buffer (cur0 + npass - 1) & 1: the out side of the other
-    VGA_TRY(activity_copy(b->act, b->total, batch_io(b, 1 - (int)((cur0 + npass - 1) & 1)), false, comp, b->stream));
-    return launch_batch(b, npass - 1, npass, npass, cur0, false);
+    VGA_TRY(activity_copy(b->act, b->total, batch_io(b, cur0 & 1), false, comp, b->stream));  // see enqueue_steps
+    return launch_batch(b, npass - 1, npass, npass, cur0, false, (cur0 + 1) & 1);
 }
 
 vga_status check_err(vga_batch *b) {

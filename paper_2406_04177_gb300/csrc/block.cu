@@ -921,8 +921,7 @@ vga_status sim_block_fused(vga_sim *s, int64_t P, bool *done) {
     }
     timing_end_weighted(s, P);
     s->blocked_passes += P;
-    if (P & 1)
-        for (int c = 0; c < 5; ++c) s->cur[c] ^= 1;
+    if (P & 1) s->cur[1] ^= 1;  // as a sparse pass
     *done = true;
     return VGA_OK;
 }

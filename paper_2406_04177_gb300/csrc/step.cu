@@ -1134,7 +1134,10 @@ static vga_status step_body(vga_sim *s, int64_t n_steps, bool sparse) {
         for (int64_t k = 1; k < n_steps && !blocked; ++k) {
             if (sub) s->sp.ntrans = sim_ticks_of_step(s, k0 + k);
             VGA_TRY(launch_stencil<1>(s, state_io(s)));
-            for (int c = 0; c < 5; ++c) s->cur[c] ^= 1;
+            // a sparse pass moves the DOM only: the others stay where the first transformation put them (it may have
+            // changed them at an unmarked node whose DOM was negative)
+            for (int c = 0; c < 5; ++c)
+                if (!sparse || c == 1) s->cur[c] ^= 1;
         }
         if (span.on) {
             s->timing_hold = false;
