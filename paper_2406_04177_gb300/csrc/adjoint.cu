@@ -1062,7 +1062,7 @@ vga_status sim_adjoint_forward(vga_sim *s, int64_t N, int64_t ckpt) {
         if (small) {  // the checkpoint and the segment as one launch
             const bool rec = sg == nseg - 1;
             if (rec) VGA_TRY(ensure_records(a));
-            VGA_TRY(small_forward(s, a->act, rows_of(s), rows_of(s), rows_of(ck_slot(a, sg), s->npad), len - 1, true,
+            VGA_TRY(small_forward(s, a->act, rows_of(s), rows_of(s), rows_of(ck_slot(a, sg), s->npad), len - 1, true, true,
                                   rec ? a->rec_y2 : nullptr, rec ? a->rec_xc : nullptr, a->xcap));
             s->steps_done += len;
             a->last_recorded = rec;
@@ -1279,8 +1279,8 @@ static vga_status adjoint_backward_impl(vga_sim *s, const double *d_lamN, double
         const bool recorded = sg == nseg - 1 && a->last_recorded;
         if (small) {
             if (!recorded)
-                VGA_TRY(small_forward(s, a->act, rows_of(cks, npad), StateRows{}, StateRows{}, len - 1, false, a->rec_y2,
-                                      a->rec_xc, a->xcap));
+                VGA_TRY(small_forward(s, a->act, rows_of(cks, npad), StateRows{}, StateRows{}, len - 1, false, true,
+                                      a->rec_y2, a->rec_xc, a->xcap));
             VGA_TRY(small_reverse(s, a->act, rows_of(a->lam[0], npad), cks.h, a->rec_y2, a->rec_xc, a->xcap, len, !may_lean,
                                   tacc, Ts, a->gtheta, flag_dev));
             continue;

@@ -218,7 +218,7 @@ __device__ __forceinline__ void block_marks(const SmallArgs &a, uint32_t v0, uin
 
 struct SmallFwd {
     StateRows in, out, ck;
-    int32_t passes, diffuse;
+    int32_t passes, diffuse, first;
     float *rec_y2, *rec_xc;
     int64_t xcap;
 };
@@ -331,10 +331,41 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_forward(SmallArgs a,
         return ok;
     };
 
-    // pass 0: the transformation alone.  At an unmarked node it adds zero to the loaded pair.
+    // pass 0: the transformation alone, of every node as in k_transform: the mask tells of the state it was built from, and
+    // since then an implicit solve, a call at the stability bound or a negative FOM nearby may have left an unmarked node with
+    // a DOM below zero, which the transformation clamps at the cost of the biomass (nothing else changes there, so the
+    // store is rare; the loads are 24 B per node and launch).  In the middle of a call unmarked nodes do not transform
+    // in any form: that adds zero to the pair.
 #pragma unroll
-    for (int k = 0; k < K; ++k)
-        if (!((act >> k) & 1u)) x2[k] = V{__fadd_rn(x2[k].h, 0.0f), __fadd_rn(x2[k].l, 0.0f)};
+    for (int k = 0; k < K; ++k) {
+        const uint32_t i = node_of(i0, k);
+        if ((act >> k) & 1u) continue;
+        if (!f.first || i >= a.n) {
+            x2[k] = V{__fadd_rn(x2[k].h, 0.0f), __fadd_rn(x2[k].l, 0.0f)};
+            continue;
+        }
+        V u[4];
+        res_t l[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int c = q > 0 ? q + 1 : 0;  // MB, SOM, FOM, CO2
+            u[q].h = f.in.h[c][i];
+            l[q] = f.in.l[c][i];
+            u[q].l = res_decode(l[q], u[q].h);
+        }
+        const V was[4] = {u[0], u[1], u[2], u[3]};
+        transform<TR, PREC>(u[0], x2[k], u[1], u[2], u[3], a.p);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            vround<PREC>(u[q]);
+            const int c = q > 0 ? q + 1 : 0;
+            const bool moved = __float_as_uint(u[q].h) != __float_as_uint(was[q].h) || res_encode(u[q].l, u[q].h) != l[q];
+            if (moved && f.out.h[c]) {
+                f.out.h[c][i] = u[q].h;
+                f.out.l[c][i] = res_encode(u[q].l, u[q].h);
+            }
+        }
+    }
     publish(0, 0, false, true);
     const int last = f.passes + (f.diffuse ? 1 : 0);
     for (int s = 1; s <= last; ++s) {
@@ -746,16 +777,16 @@ bool small_shape(int64_t n, int *K, int *G) {
 }
 
 bool small_ok(const vga_sim *s, const Activity &act) {
-    // nx: see Far.  max_block: the marked nodes of a block must fit its threads (-1: the graph does not fit).  A DOM below
-    // zero, or a step so near the stability bound that rounding can make one, needs the passes that
-    // transform every node first.
+    // nx: see Far.  max_block: the marked nodes of a block must fit its threads (-1: the graph does not fit).  With a DOM below
+    // zero in the uploaded state, or a step so near the stability bound that rounding can make one, a sweep without
+    // dL/dX^0 would be repeated; step calls keep to the same rule.
     return s->kernel_variant == 5 && s->activity_skip && !s->timing && !s->subcycled() && s->precision() == P_COMP &&
            s->g->nx <= kSmallThreads && act.max_block >= 0 && act.max_block <= kSmallThreads && !act.negative_dom &&
            6.0 * s->params.D * s->params.dt * s->max_g <= 0.999;
 }
 
 vga_status small_forward(vga_sim *s, const Activity &act, StateRows in, StateRows out, StateRows ck, int64_t passes,
-                         bool diffuse, float *rec_y2, float *rec_xc, int64_t xcap) {
+                         bool diffuse, bool first, float *rec_y2, float *rec_xc, int64_t xcap) {
     SmallArgs a;
     SmallWork *w = nullptr;
     VGA_TRY(small_args(s, act, &a, &w));
@@ -764,6 +795,7 @@ vga_status small_forward(vga_sim *s, const Activity &act, StateRows in, StateRow
     f.out = out;
     f.ck = ck;
     f.diffuse = diffuse ? 1 : 0;
+    f.first = first ? 1 : 0;
     f.rec_y2 = rec_y2;
     f.rec_xc = rec_xc;
     f.xcap = xcap;

@@ -1081,7 +1081,7 @@ vga_status sim_step_explicit(vga_sim *s, int64_t n_steps) {
         }
         for (int64_t k = 0; k < n_steps; k += kSmallSteps) {
             const int64_t len = std::min(kSmallSteps, n_steps - k);
-            VGA_TRY(small_forward(s, s->act, rows, rows, StateRows{}, len - 1, true, nullptr, nullptr, 0));
+            VGA_TRY(small_forward(s, s->act, rows, rows, StateRows{}, len - 1, true, k == 0, nullptr, nullptr, 0));
             s->steps_done += len;
         }
         return VGA_OK;
