@@ -440,8 +440,8 @@ __global__ void __launch_bounds__(kThreads, VGA_ADJ_MIN_BLOCKS) k_adjoint_vec(in
 // The step is then two kernels: the diffusion of every node's DOM adjoint, and J_T at the marked nodes in
 // rank order, their other adjoints in a compact state.  36 B per node instead of 66 and about half the
 // instructions.  dL/dD, the rate and conductance gradients are those of k_adjoint_vec (the sums take the
-// nodes in another order).  A node that breaks the premise (unmarked, DOM negative) sets *flag, and the
-// caller repeats the sweep with k_adjoint_vec.
+// nodes in another order).  A node that breaks the premise (unmarked, DOM negative, in a step or, k_lean_check, where a
+// segment starts with the transformation of every node) sets *flag, and the caller repeats the sweep with k_adjoint_vec.
 // dL/dD is summed in one compensated pair per thread (dslot), carried from launch to launch in memory
 // and reduced once after the sweep: a block reduction per launch costs as much as the diffusion.
 // Neither the grid nor the node of a thread changes, so the sums are the same bits on every run.
@@ -558,6 +558,22 @@ __global__ void __launch_bounds__(kThreads, 5) k_lean_dom(int64_t n, NbrTable tb
     if (full) vstore_k<PREC, K, true>(io.out[1], io.lout[1], i0, end, l2);
     else vstore_k<PREC, K, false>(io.out[1], io.lout[1], i0, end, l2);
     if (neg) atomicOr(a.flag, 1);
+}
+
+// Where a segment starts every node transforms, and step 0 of its reverse takes the marked nodes only: the others must
+// have been left as they were.  (If their DOM is in order at every segment's start, so are MB, SOM and FOM, which are
+// zero at the sweep's start.)  4 B per node and segment, four nodes per thread (rows are padded to 64 values).
+__global__ void __launch_bounds__(kThreads) k_lean_check(int64_t n, const float *__restrict__ dom, const uint32_t *__restrict__ mask,
+                                                         int32_t *flag) {
+    const int64_t i = 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
+    if (i >= n) return;
+    const float4 y = __ldg(reinterpret_cast<const float4 *>(dom + i));
+    const uint32_t act = __ldg(mask + (i >> 5)) >> (i & 31);
+    const float v[4] = {y.x, y.y, y.z, y.w};
+    bool bad = false;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) bad |= i + k < n && !((act >> k) & 1u) && !unmarked_identity(v[k]);
+    if (bad) atomicOr(flag, 1);
 }
 
 // J_T at the marked nodes.  Everything but mu2 was written before k_lean_dom started (which waited for
@@ -836,7 +852,8 @@ struct AdjointBuffers {
     int64_t lean_bytes = 0;
     cudaStream_t cap_stream = nullptr;  // private stream the backward sweep's loops are captured on
     double *gtheta = nullptr; // ntheta
-    double *gsum = nullptr;   // kPar, then the flag of a sweep without dL/dX^0
+    double *gsum = nullptr;   // kPar, then the flags of a sweep without dL/dX^0 and of a forward sweep of small-graph launches
+    bool small_fwd = false;   // the forward sweep was one of those
     double *lamstage = nullptr;  // 5 n FP64 (host-pointer staging)
 };
 
@@ -1057,13 +1074,16 @@ vga_status sim_adjoint_forward(vga_sim *s, int64_t N, int64_t ckpt) {
         }
     }
     const bool small = a->sparse && small_ok(s, a->act) && std::min(ckpt, N) <= kSmallSteps;
+    a->small_fwd = small;
+    int32_t *odd = reinterpret_cast<int32_t *>(a->gsum + kPar) + 1;
+    if (small) VGA_CUDA(cudaMemsetAsync(odd, 0, sizeof(int32_t), s->stream));
     for (int64_t sg = 0; sg < nseg; ++sg) {
         const int64_t len = std::min(ckpt, N - sg * ckpt);
         if (small) {  // the checkpoint and the segment as one launch
             const bool rec = sg == nseg - 1;
             if (rec) VGA_TRY(ensure_records(a));
             VGA_TRY(small_forward(s, a->act, rows_of(s), rows_of(s), rows_of(ck_slot(a, sg), s->npad), len - 1, true, true,
-                                  rec ? a->rec_y2 : nullptr, rec ? a->rec_xc : nullptr, a->xcap));
+                                  rec ? a->rec_y2 : nullptr, rec ? a->rec_xc : nullptr, a->xcap, odd));
             s->steps_done += len;
             a->last_recorded = rec;
             continue;
@@ -1165,11 +1185,11 @@ static vga_status lean_work(vga_sim *s, AdjointBuffers *a, LeanWork *w) {
     return VGA_OK;
 }
 
-// lean: without dL/dX^0 where that pays (k_lean_dom, k_small_reverse); *redo is set when its premise did not
-// hold (call again with lean = false).
+// lean: without dL/dX^0 where that pays (k_lean_dom, k_small_reverse); plain: neither that nor one launch per
+// segment.  *redo is set when a premise of those did not hold (call again with plain).
 template <int WM>
 static vga_status adjoint_backward_impl(vga_sim *s, const double *d_lamN, double *d_lam0, double *grad8,
-                                        double *h_gtheta, bool lean, bool *redo) {
+                                        double *h_gtheta, bool lean, bool plain, bool *redo) {
     *redo = false;
     constexpr int PREC = P_COMP;
     AdjointBuffers *a = s->adj;
@@ -1222,20 +1242,21 @@ static vga_status adjoint_backward_impl(vga_sim *s, const double *d_lamN, double
     }
     VGA_TRY(ensure_records(a));
     // small graphs: a segment's recomputation and its reverse steps are one launch each
-    const bool may_lean = lean && sparse && !d_lam0;
+    const bool may_lean = lean && sparse && !d_lam0 && !plain;
     // (with dL/dX^0 its sums are one per pair of nodes: k_adjoint_vec's, when each of its threads takes one pair)
-    const bool small = sparse && small_ok(s, a->act) && std::min(ckpt, N) <= kSmallSteps && small_reverse_ok(s, !may_lean) &&
+    const bool small = sparse && !plain && a->small_fwd && small_ok(s, a->act) && std::min(ckpt, N) <= kSmallSteps && small_reverse_ok(s, !may_lean) &&
                        (may_lean || (kAdjK == 2 && (int64_t)Gt * kThreads * 2 >= s->n));
     // Above a quarter of the nodes marked a lean step moves as much as a full one (36 B per node and about
     // 120 B per marked node against 66 B per node); on small graphs its second launch costs more than it
     // saves.  Backward sweep per step, recomputation included, 6% marked, 8^3 blocks: 0.57 M nodes 19.9 us
     // lean, 21.9 full; 1.0 M 26.8 / 32.5; 4.7 M 96 / 147; 20.8 M 349 / 581.
     lean = may_lean && !small && s->n >= kLeanNodes && m * 4 < s->n;
-    int32_t *flag_dev = lean || (small && may_lean) ? reinterpret_cast<int32_t *>(a->gsum + kPar) : nullptr;
+    int32_t *flag_dev = lean || small ? reinterpret_cast<int32_t *>(a->gsum + kPar) : nullptr;  // then the forward sweep's
     if (flag_dev) VGA_CUDA(cudaMemsetAsync(flag_dev, 0, sizeof(int32_t), st));
     LeanWork lw;
     if (lean) VGA_TRY(lean_work(s, a, &lw));
-    k_lam_in<<<grid_for(s->n, kThreads), kThreads, 0, st>>>(s->n, d_lamN, io_from(a->lam[0], a->lam[0], npad), flag_dev);
+    k_lam_in<<<grid_for(s->n, kThreads), kThreads, 0, st>>>(s->n, d_lamN, io_from(a->lam[0], a->lam[0], npad),
+                                                        may_lean ? flag_dev : nullptr);
     if (lean && m > 0) k_lean_gather<<<grid_for(m, kThreads), kThreads, 0, st>>>(m, lw.ss, io_from(a->lam[0], a->lam[0], npad));
     VGA_CHECK_LAUNCH();
     // k_lean_marked: the gradient partials bound its grid; a thread takes a few nodes, so that the block sums
@@ -1361,11 +1382,14 @@ static vga_status adjoint_backward_impl(vga_sim *s, const double *d_lamN, double
             lb = (int)(lb0 ^ ((len - 1) & 1));
             const StateIO io = lam_io(a->lam, lb, npad);
             timing_begin(s, VGA_KERNEL_ADJOINT);
-            if (lean)
+            if (lean) {
+                k_lean_check<<<grid_for(s->n, 4 * kThreads), kThreads, 0, st>>>(s->n, cks.h + npad, lw.ss.mask, flag_dev);
                 lean_step(st, 0, lb, cks.h);
-            else
+                ++s->launches;
+            } else {
                 launch_reverse<WM, PREC, 0>(G, st, tb.tz != nullptr, tacc != nullptr, s->n, tb, bt, s->sp, io, npad, cks.h,
                                             a->rec_y2, SparseState{}, 1, tacc, a->gpart, a->gtheta);
+            }
             timing_end(s);
             VGA_CHECK_LAUNCH();
             ++s->launches;
@@ -1408,8 +1432,8 @@ static vga_status adjoint_backward_impl(vga_sim *s, const double *d_lamN, double
     VGA_CHECK_LAUNCH();
     s->launches += 2;
     double h[kPar];
-    int32_t flag = 0;
-    if (flag_dev) VGA_CUDA(cudaMemcpyAsync(&flag, flag_dev, sizeof(flag), cudaMemcpyDeviceToHost, st));
+    int32_t flag[2] = {0, 0};
+    if (flag_dev) VGA_CUDA(cudaMemcpyAsync(flag, flag_dev, (small ? 2 : 1) * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
     VGA_TRY(sim_fetch_device_error(s));  // of this sweep, and of the forward one in whatever form it ran
     VGA_CUDA(cudaMemcpyAsync(h, a->gsum, sizeof(double) * kPar, cudaMemcpyDeviceToHost, st));
     if (s->face_mode) VGA_TRY(sim_face_mirror(s, a->gtheta));  // both slots of every edge
@@ -1420,7 +1444,7 @@ static vga_status adjoint_backward_impl(vga_sim *s, const double *d_lamN, double
         a->valid = false;
         return sim_device_error(s, s->report->err);
     }
-    if (flag) {
+    if (flag[0] || flag[1]) {
         *redo = true;
         return VGA_OK;
     }
@@ -1455,12 +1479,13 @@ vga_status sim_adjoint_backward(vga_sim *s, const double *d_lamN, double *d_lam0
         return fail(VGA_ERR_INVALID_ARG, "parameters or conductances changed since the adjoint forward pass");
     // So near the stability bound that rounding can make a DOM negative (as in small_ok), a lean sweep would likely be
     // repeated: 95 us a step for nothing before the 137 of the full form (4.7 M nodes).
-    bool lean = !d_lam0 && 6.0 * s->params.D * s->params.dt * s->max_g <= 0.999, redo = false;
+    const bool lean = !d_lam0 && 6.0 * s->params.D * s->params.dt * s->max_g <= 0.999;
+    bool plain = false, redo = false;
     for (;;) {
-        VGA_TRY(s->wmode == W_BLOCK ? adjoint_backward_impl<W_BLOCK>(s, d_lamN, d_lam0, grad8, h_gtheta, lean, &redo)
-                                    : adjoint_backward_impl<W_UNIT>(s, d_lamN, d_lam0, grad8, h_gtheta, lean, &redo));
+        VGA_TRY(s->wmode == W_BLOCK ? adjoint_backward_impl<W_BLOCK>(s, d_lamN, d_lam0, grad8, h_gtheta, lean, plain, &redo)
+                                    : adjoint_backward_impl<W_UNIT>(s, d_lamN, d_lam0, grad8, h_gtheta, lean, plain, &redo));
         if (!redo) return VGA_OK;
-        lean = false;
+        plain = true;
     }
 }
 

@@ -59,6 +59,9 @@ __device__ __forceinline__ void face_atomic_add_f(double *gtheta, int32_t f, flo
     if (f >= 0) atomicAdd(gtheta + f, f32_to_f64_alu(v));
 }
 
+// Whether the transformation of an unmarked node with this DOM is the identity (a NaN's is not either).
+__device__ __forceinline__ bool unmarked_identity(float y) { return y >= 0.0f && y <= 3.4028235e38f; }
+
 // transform_sync_reverse at an unmarked node, x = (0, y, 0, 0, .) with +0, without the operations whose
 // results are known there: every flux is zero, the mortality and turnover branches are the free ones, and
 // dL/dx2 gets a term only when the uptake is clamped (y < 0).  A sum that starts at +0 and gets one

@@ -221,6 +221,7 @@ struct SmallFwd {
     int32_t passes, diffuse, first;
     float *rec_y2, *rec_xc;
     int64_t xcap;
+    int32_t *flag;
 };
 
 template <int WM, int TR, int K, bool REC>
@@ -354,6 +355,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_forward(SmallArgs a,
             u[q].l = res_decode(l[q], u[q].h);
         }
         const V was[4] = {u[0], u[1], u[2], u[3]};
+        if (f.flag && !unmarked_identity(x2[k].h)) atomicOr(f.flag, 1);
         transform<TR, PREC>(u[0], x2[k], u[1], u[2], u[3], a.p);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -786,7 +788,7 @@ bool small_ok(const vga_sim *s, const Activity &act) {
 }
 
 vga_status small_forward(vga_sim *s, const Activity &act, StateRows in, StateRows out, StateRows ck, int64_t passes,
-                         bool diffuse, bool first, float *rec_y2, float *rec_xc, int64_t xcap) {
+                         bool diffuse, bool first, float *rec_y2, float *rec_xc, int64_t xcap, int32_t *flag) {
     SmallArgs a;
     SmallWork *w = nullptr;
     VGA_TRY(small_args(s, act, &a, &w));
@@ -799,6 +801,7 @@ vga_status small_forward(vga_sim *s, const Activity &act, StateRows in, StateRow
     f.rec_y2 = rec_y2;
     f.rec_xc = rec_xc;
     f.xcap = xcap;
+    f.flag = flag;
     f.passes = (int32_t)passes;
     const bool block = s->wmode == W_BLOCK;
     if (rec_y2)

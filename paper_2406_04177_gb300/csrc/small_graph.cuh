@@ -28,9 +28,10 @@ struct StateRows {
 // diffusion-only pass with the resulting state written to `out` (may be `in`).  first: the launch starts a step call (or
 // a segment), whose first transformation is that of every node; otherwise it goes on with one.  ck (may be empty): receives
 // a copy of `in`.  rec_y2 / rec_xc (may be NULL): records of steps 0 .. passes for the adjoint, rec_y2 in
-// rows of npad, X^k of the marked nodes (steps 1 ..) in 4 rows of xcap per step.
+// rows of npad, X^k of the marked nodes (steps 1 ..) in 4 rows of xcap per step.  *flag (may be NULL) |= 1 where
+// the first transformation of an unmarked node was not the identity: small_reverse must not be used then.
 vga_status small_forward(vga_sim *s, const Activity &act, StateRows in, StateRows out, StateRows ck, int64_t passes,
-                         bool diffuse, bool first, float *rec_y2, float *rec_xc, int64_t xcap);
+                         bool diffuse, bool first, float *rec_y2, float *rec_xc, int64_t xcap, int32_t *flag = nullptr);
 
 // Reverse steps len - 1 .. 0 of a segment whose records are rec_y2, rec_xc and whose X^0 is x0 (rows of
 // npad), on the adjoint state lam (in place; the CO2 row is read only).  full: every compartment of every
