@@ -64,8 +64,9 @@ __device__ __forceinline__ bool unmarked_identity(float y) { return y >= 0.0f &&
 
 // transform_sync_reverse at an unmarked node, x = (0, y, 0, 0, .) with +0, without the operations whose
 // results are known there: every flux is zero, the mortality and turnover branches are the free ones, and
-// dL/dx2 gets a term only when the uptake is clamped (y < 0).  A sum that starts at +0 and gets one
-// product keeps the product's value (0 + t), as there.  The same bits for finite values.
+// dL/dx2 gets a term only when the uptake is clamped (y < 0), else w_upt times zero, which passes on what is not
+// finite.  A sum that starts at +0 and gets one product keeps the product's value (0 + t), as there.  The same bits for
+// finite values.
 template <int PREC>
 __device__ __forceinline__ void reverse_unmarked(float y, const V (&mu)[5], V (&lam)[5], const StepParams &p) {
     const float sat = __fdividef(y, __fadd_rn(p.K, y));
@@ -74,7 +75,7 @@ __device__ __forceinline__ void reverse_unmarked(float y, const V (&mu)[5], V (&
     const float w_resp = __fsub_rn(mu[4].h, mu[0].h);
     const bool clamped = 0.0f > y;
     const float du = clamped ? 0.0f : __fadd_rn(0.0f, __fmul_rn(w_upt, __fmul_rn(p.a, sat)));
-    const float d1 = clamped ? __fadd_rn(0.0f, w_upt) : 0.0f;
+    const float d1 = __fadd_rn(0.0f, clamped ? w_upt : __fmul_rn(w_upt, 0.0f));
     const float d0 = __fadd_rn(du, __fadd_rn(__fmul_rn(w_mor, p.m), __fmul_rn(w_resp, p.r)));
     const float d3 = __fadd_rn(0.0f, __fmul_rn(__fsub_rn(mu[1].h, mu[3].h), p.f));
     const float d2 = __fadd_rn(0.0f, __fmul_rn(__fsub_rn(mu[1].h, mu[2].h), p.s));

@@ -67,3 +67,26 @@ def test_small_graph_with_negative_stocks(shape, state_gradient):
     if state_gradient:
         assert torch.equal(out[0][2], out[1][2])
     g.close()
+
+
+@pytest.mark.parametrize("shape", [(9, 11, 13), (40, 44, 52), (79, 84, 85)])
+@pytest.mark.parametrize("state_gradient", [False, True])
+@pytest.mark.parametrize("value", [float("inf"), float("nan")])
+def test_an_adjoint_that_is_not_finite_spreads(shape, state_gradient, value):
+    """dL/dMB^N at an unmarked node: J_T multiplies it by zero on its way to the DOM, which makes a NaN of it,
+    not nothing."""
+    g = vga.Graph(np.zeros(shape, dtype=np.uint8))
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    X, _ = _state(g.n, gen)
+    lam = torch.randn((5, g.n), generator=gen, device="cuda", dtype=torch.float64)
+    lam[0, 7] = value
+    sim = vga.Sim(g, synth.paper_params())
+    sim.set_masses(X)
+    sim.adjoint_forward(7, 3)
+    dx = torch.zeros_like(lam) if state_gradient else None
+    grad, _ = sim.adjoint_backward(lam, dx)
+    assert np.isnan(grad["D"])
+    if state_gradient:
+        assert torch.isnan(dx[1]).any()
+    sim.close()
+    g.close()
