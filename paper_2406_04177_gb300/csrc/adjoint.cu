@@ -212,14 +212,7 @@ __device__ __forceinline__ void block_sum_cacc(const CAcc (&a)[K], double *out) 
     __shared__ double sh[K][32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int nw = (blockDim.x + 31) >> 5;
-    const CAcc w = warp_sums<16>(a, [](CAcc x, CAcc y) {
-        CAcc r;
-        r.s = __fadd_rn(x.s, y.s);
-        const float bp = __fsub_rn(r.s, x.s);
-        const float err = __fadd_rn(__fsub_rn(x.s, __fsub_rn(r.s, bp)), __fsub_rn(y.s, bp));
-        r.c = __fadd_rn(__fadd_rn(x.c, y.c), err);
-        return r;
-    });
+    const CAcc w = warp_sums<16>(a, [](CAcc x, CAcc y) { return cacc_join(x, y); });
     const double mine = (double)w.s + (double)w.c;
 #pragma unroll
     for (int k = 0; k < K; ++k)
@@ -442,8 +435,12 @@ __global__ void __launch_bounds__(kThreads, VGA_ADJ_MIN_BLOCKS) k_adjoint_vec(in
 // instructions.  dL/dD, the rate and conductance gradients are those of k_adjoint_vec (the sums take the
 // nodes in another order).  A node that breaks the premise (unmarked, DOM negative, in a step or, k_lean_check, where a
 // segment starts with the transformation of every node) sets *flag, and the caller repeats the sweep with k_adjoint_vec.
-// dL/dD is summed in one compensated pair per thread (dslot), carried from launch to launch in memory
-// and reduced once after the sweep: a block reduction per launch costs as much as the diffusion.
+// dL/dD is summed in one compensated pair per thread (dslot), carried from launch to launch in memory: a block
+// reduction per launch costs as much as the diffusion.  The pairs go to FP64 (k_reduce_lean) when they hold as many
+// terms as a thread of k_adjoint_vec adds before its block sum, so that no sum is carried in FP32 pairs for longer
+// than there.  Per step 48.7 -> 50.2 us at 3.7 M nodes, 97.1 -> 99.4 at 8.1 M, 245.6 -> 246.2 at 20.8 M; the error of a
+// strongly cancelling dL/dD over 2000 steps at 3.7 M nodes against the same terms summed in FP64 8.1e-14 -> 6e-16 (full
+// form 1.4e-14).
 // Neither the grid nor the node of a thread changes, so the sums are the same bits on every run.
 constexpr int kLeanK = 2;  // consecutive nodes per thread: 2 at 5 blocks per SM 250 us per step, 4 at 3 blocks 285 (512^3)
 
@@ -618,14 +615,24 @@ __global__ void __launch_bounds__(kThreads) k_lean_marked(int64_t m, StepParams 
     if (threadIdx.x < GR_COUNT) a.gpart[(int64_t)blockIdx.x * kPar + threadIdx.x] += out[threadIdx.x];
 }
 
-// After a lean sweep: the dslot pairs into the dL/dD column of the per-block FP64 partials gpart[grid x kPar].
-__global__ void __launch_bounds__(kThreads) k_reduce_lean(int64_t T, const float2 *__restrict__ dslot, double *__restrict__ gpart) {
+// The dslot pairs, cleared, into the dL/dD column of the per-block FP64 partials gpart[grid x kPar].  T is a multiple of
+// kThreads.  Four pairs are joined as in the block sums (FP64 issues at a 64th of the FP32 rate): 16 B per slot at the
+// copy rate are 25 us for 20.8 M nodes.
+__global__ void __launch_bounds__(kThreads) k_reduce_lean(int64_t T, float2 *__restrict__ dslot, double *__restrict__ gpart) {
     double s[1] = {0.0};
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < T; t += (int64_t)gridDim.x * blockDim.x)
-        s[0] += (double)dslot[t].x + (double)dslot[t].y;
+    float4 *d4 = reinterpret_cast<float4 *>(dslot);
+    const float4 zero = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll 2
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < T / 4; t += (int64_t)gridDim.x * blockDim.x) {
+        const float4 a = d4[2 * t], b = d4[2 * t + 1];
+        d4[2 * t] = zero;
+        d4[2 * t + 1] = zero;
+        const CAcc w = cacc_join(cacc_join(CAcc{a.x, a.y}, CAcc{a.z, a.w}), cacc_join(CAcc{b.x, b.y}, CAcc{b.z, b.w}));
+        s[0] += (double)w.s + (double)w.c;
+    }
     __shared__ double out[1];
     block_sum_store<1>(s, out);
-    if (threadIdx.x == 0) gpart[(int64_t)blockIdx.x * kPar + GR_COUNT] = out[0];
+    if (threadIdx.x == 0) gpart[(int64_t)blockIdx.x * kPar + GR_COUNT] += out[0];
 }
 
 // The marked nodes' adjoints of MB, SOM, FOM and CO2 into the compact state (rank order).
@@ -1290,6 +1297,14 @@ static vga_status adjoint_backward_impl(vga_sim *s, const double *d_lamN, double
         tacc = a->tacc;
     }
     VGA_CUDA(cudaMemsetAsync(a->gtheta, 0, sizeof(double) * (size_t)a->ntheta, st));
+    // lean steps whose terms may stay in the pairs: those of one launch of the full form (which keeps pairs for the
+    // sweep where it has slots)
+    const int64_t hold = groups_per_thread <= kSlotGroups ? INT64_MAX : groups_per_thread * kAdjK / kLeanK;
+    int64_t held = 0;
+    auto reduce_lean = [&](cudaStream_t cs) {
+        k_reduce_lean<<<G, kThreads, 0, cs>>>(lw.T, lw.args.dslot, a->gpart);
+        ++s->launches;
+    };
     int lb = 0;
     for (int64_t sg = nseg - 1; sg >= 0; --sg) {
         const int64_t len = std::min(ckpt, N - sg * ckpt);
@@ -1356,6 +1371,13 @@ static vga_status adjoint_backward_impl(vga_sim *s, const double *d_lamN, double
         // the adjoint buffers), then step 0, whose X^0 is the segment's checkpoint
         if (table) {
             const int lb0 = lb;
+            if (lean) {  // room for the segment's steps, or for `hold` of them
+                if (held > hold - std::min(len, hold)) {
+                    reduce_lean(st);
+                    held = 0;
+                }
+                held = len < hold ? held + len : len % hold;
+            }
             auto issue = [&](cudaStream_t cs) -> vga_status {
                 int l = lb0;
                 for (int64_t j = len - 1; j >= 1; --j) {
@@ -1363,9 +1385,10 @@ static vga_status adjoint_backward_impl(vga_sim *s, const double *d_lamN, double
                     const float *y2k = a->rec_y2 + (size_t)j * npad;
                     const StateIO io = lam_io(a->lam, l, npad);
                     timing_begin(s, VGA_KERNEL_ADJOINT);
-                    if (lean)
+                    if (lean) {
                         lean_step(cs, j, l, nullptr);
-                    else if (sparse)
+                        if ((len - j) % hold == 0) reduce_lean(cs);
+                    } else if (sparse)
                         launch_reverse<WM, PREC, 1>(G, cs, tb.tz != nullptr, tacc != nullptr, s->n, tb, bt, s->sp, io,
                                                     npad, xk, y2k, ss, a->xcap, tacc, a->gpart, a->gtheta);
                     else
@@ -1385,6 +1408,7 @@ static vga_status adjoint_backward_impl(vga_sim *s, const double *d_lamN, double
             if (lean) {
                 k_lean_check<<<grid_for(s->n, 4 * kThreads), kThreads, 0, st>>>(s->n, cks.h + npad, lw.ss.mask, flag_dev);
                 lean_step(st, 0, lb, cks.h);
+                if (len % hold == 0) reduce_lean(st);
                 ++s->launches;
             } else {
                 launch_reverse<WM, PREC, 0>(G, st, tb.tz != nullptr, tacc != nullptr, s->n, tb, bt, s->sp, io, npad, cks.h,
@@ -1421,13 +1445,8 @@ static vga_status adjoint_backward_impl(vga_sim *s, const double *d_lamN, double
         k_reduce_tacc<<<(unsigned)(Ts / kThreads), kThreads, 0, st>>>(tacc, a->gpart);
         ++s->launches;
     }
-    const int Gr = lean    ? (int)std::max<int64_t>(Gm, std::min<int64_t>(G, 304))
-                   : tacc ? (int)(Ts / kThreads)
-                           : G;
-    if (lean) {
-        k_reduce_lean<<<Gr, kThreads, 0, st>>>(lw.T, lw.args.dslot, a->gpart);
-        ++s->launches;
-    }
+    if (lean) reduce_lean(st);
+    const int Gr = tacc ? (int)(Ts / kThreads) : G;
     k_reduce_gpart<<<1, kThreads, 0, st>>>(a->gpart, Gr, a->gsum);
     VGA_CHECK_LAUNCH();
     s->launches += 2;

@@ -27,6 +27,16 @@ __device__ __forceinline__ void cacc_add_prod(CAcc &a, float x, float y) {
     a.c = __fadd_rn(a.c, e);
 }
 
+// The sum of two accumulators.
+__device__ __forceinline__ CAcc cacc_join(CAcc x, CAcc y) {
+    CAcc r;
+    r.s = __fadd_rn(x.s, y.s);
+    const float bp = __fsub_rn(r.s, x.s);
+    const float err = __fadd_rn(__fsub_rn(x.s, __fsub_rn(r.s, bp)), __fsub_rn(y.s, bp));
+    r.c = __fadd_rn(__fadd_rn(x.c, y.c), err);
+    return r;
+}
+
 __device__ __forceinline__ CAcc shfl_value(CAcc a, int o) {
     CAcc b;
     b.s = __shfl_xor_sync(0xffffffffu, a.s, o);
