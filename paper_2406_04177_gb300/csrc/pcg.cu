@@ -472,6 +472,16 @@ __device__ __forceinline__ FF ff_mul(FF a, FF b) {
     return two_sum(p, __fadd_rn(e, __fadd_rn(__fmul_rn(a.h, b.l), __fmul_rn(a.l, b.h))));
 }
 
+// Adds x to a sum kept with its rounding errors.  A thread of the solver kernels takes up to 134 nodes at 20.8 M
+// nodes; a plain FP32 sum of so many terms would lose 7 bits.  It leaves as FP32, rounded once: a second FP64
+// conversion and addition per thread cost 0.8 us an iteration.
+__device__ __forceinline__ void ff_acc(FF &a, float x) {
+    const FF t = two_sum(a.h, x);
+    a = {t.h, __fadd_rn(a.l, t.l)};
+}
+
+__device__ __forceinline__ double ff_value(FF a) { return (double)__fadd_rn(a.h, a.l); }
+
 // Sum over the neighbours of node i of x_j in float-float (TwoSum chain of the high parts; low parts
 // and the chain's errors added in FP32), and their number.
 template <int TF>
@@ -526,7 +536,7 @@ __global__ void __launch_bounds__(kThreads) k_mx_res(int64_t n, NbrTable tb, FF 
     if (FIRST && blockIdx.x == 0 && threadIdx.x == 0) sc->fresh = 1;
     FF rr = {0.0f, 0.0f};  // |r|^2 per thread in float-float (no FP64 arithmetic per node)
     double bb = 0.0;       // |b|^2, once per solve
-    float rz = 0.0f;
+    FF rz = {0.0f, 0.0f};
     const int64_t ntile = (n + kThreads - 1) / kThreads;
     const float *__restrict__ sh = FIRST ? v.bh : v.xh;  // FIRST: x = b, neighbours read from b
     const float *__restrict__ sl = FIRST ? v.bl : v.xl;
@@ -563,10 +573,10 @@ __global__ void __launch_bounds__(kThreads) k_mx_res(int64_t n, NbrTable tb, FF 
                 const double b = (double)bi.h + (double)bi.l;
                 bb = fma(b, b, bb);
             }
-            rz = __fmaf_rn(r32, __fmul_rn(ti, r32), rz);
+            ff_acc(rz, __fmul_rn(r32, __fmul_rn(ti, r32)));
         }
     }
-    double acc[3] = {(double)rr.h + (double)rr.l, bb, (double)rz};
+    double acc[3] = {(double)rr.h + (double)rr.l, bb, ff_value(rz)};
     __shared__ double out[3];
     block_sum_store<3>(acc, out);
     if (threadIdx.x < 3) part[(int64_t)blockIdx.x * 3 + threadIdx.x] = out[threadIdx.x];
@@ -686,7 +696,7 @@ __global__ void __launch_bounds__(kThreads) k_mx_spmv(int64_t n, NbrTable tb, fl
                                                       double *__restrict__ part, MxScalars *sc) {
     if (sc->inner_done) return;
     constexpr int K = 4;
-    float acc = 0.0f;
+    FF acc = {0.0f, 0.0f};
     const float *__restrict__ p = v.p;
     float *__restrict__ q = v.q;
     const uint32_t nn = (uint32_t)n;
@@ -730,7 +740,7 @@ __global__ void __launch_bounds__(kThreads) k_mx_spmv(int64_t n, NbrTable tb, fl
         float pr = __shfl_down_sync(0xffffffffu, pv[0], 1);
         if (lane == 0 && ((ty[0] >> 15) & 1u)) pl = __ldg(p + (i0 - 1));
         if (lane == 31 && (ty[K - 1] >> 31)) pr = __ldg(p + (i0 + K));
-        float qv[K];
+        float qv[K], pq = 0.0f;
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             const uint32_t dym = ty[k] & 0x7fffu, dyp = (ty[k] >> 16) & 0x7fffu;
@@ -743,8 +753,9 @@ __global__ void __launch_bounds__(kThreads) k_mx_spmv(int64_t n, NbrTable tb, fl
             if (zm[k]) sum += vi - __ldg(p + (i0 + k - zm[k]));
             if (zp[k]) sum += vi - __ldg(p + (i0 + k + zp[k]));
             qv[k] = vi + c * sum;
-            if (i0 + k < nn) acc += vi * qv[k];
+            if (i0 + k < nn) pq += vi * qv[k];
         }
+        ff_acc(acc, pq);
         if (full) {
             st_floats<K>(q + i0, qv);
         } else {
@@ -753,7 +764,7 @@ __global__ void __launch_bounds__(kThreads) k_mx_spmv(int64_t n, NbrTable tb, fl
                 if (i0 + k < nn) q[i0 + k] = qv[k];
         }
     }
-    double a[1] = {(double)acc};
+    double a[1] = {ff_value(acc)};
     __shared__ double out[1];
     block_sum_store<1>(a, out);
     if (threadIdx.x == 0) part[blockIdx.x] = out[0];
@@ -777,7 +788,7 @@ __global__ void __launch_bounds__(kThreads) k_mx_upd(int64_t n, float c, MxVecs 
     if (threadIdx.x < 8) tdeg[threadIdx.x] = jacobi_t(c, (int)threadIdx.x);
     __syncthreads();
     const float alpha = (float)sc->alpha;
-    float a0 = 0.0f, a1 = 0.0f;
+    FF a0 = {0.0f, 0.0f}, a1 = {0.0f, 0.0f};
     const int64_t n4 = n >> 2;
     const int64_t g0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, gs = (int64_t)gridDim.x * blockDim.x;
     float4 *__restrict__ r4 = reinterpret_cast<float4 *>(v.r);
@@ -794,16 +805,16 @@ __global__ void __launch_bounds__(kThreads) k_mx_upd(int64_t n, float c, MxVecs 
         r.z -= alpha * q.z;
         r.w -= alpha * q.w;
         r4[k] = r;
-        a0 += r.x * (tdeg[g.x] * r.x) + r.y * (tdeg[g.y] * r.y) + r.z * (tdeg[g.z] * r.z) + r.w * (tdeg[g.w] * r.w);
-        a1 += r.x * r.x + r.y * r.y + r.z * r.z + r.w * r.w;
+        ff_acc(a0, r.x * (tdeg[g.x] * r.x) + r.y * (tdeg[g.y] * r.y) + r.z * (tdeg[g.z] * r.z) + r.w * (tdeg[g.w] * r.w));
+        ff_acc(a1, r.x * r.x + r.y * r.y + r.z * r.z + r.w * r.w);
     }
     for (int64_t i = 4 * n4 + g0; i < n; i += gs) {
         const float ri = v.r[i] - alpha * v.q[i];
         v.r[i] = ri;
-        a0 += ri * (tdeg[v.deg[i]] * ri);
-        a1 += ri * ri;
+        ff_acc(a0, ri * (tdeg[v.deg[i]] * ri));
+        ff_acc(a1, ri * ri);
     }
-    double a[2] = {(double)a0, (double)a1};
+    double a[2] = {ff_value(a0), ff_value(a1)};
     __shared__ double out[2];
     block_sum_store<2>(a, out);
     if (threadIdx.x < 2) part[(int64_t)blockIdx.x * 2 + threadIdx.x] = out[threadIdx.x];
