@@ -1071,8 +1071,11 @@ vga_status sim_step_explicit(vga_sim *s, int64_t n_steps) {
     // Where most nodes are marked the dense pass (68 B per node at the copy rate) beats the sparse one, whose
     // marked nodes are taken 256 at a time and move 52 B each on top of the 20 B of the diffusion.  Per
     // pass, 256^3 at 20% / 320^3 at 17%: 76% marked 35.8 / 55.0 us sparse, 32.9 / 48.3 dense; 48% marked
-    // 24.4 / 42.5 sparse, 32.8 / 48.3 dense.  The line lies between, at five eighths.
-    if (sparse && s->act.n_active * 8 >= s->n * 5) sparse = false;
+    // 24.4 / 42.5 sparse, 32.8 / 48.3 dense.  The line lies between, at five eighths.  (Variant 5's passes were measured;
+    // variant 6 asks for its own.  Below 0.3 M nodes 70 to 100% marked: 3.5 us a dense pass at 8,000 nodes, 3.2 at 76,000,
+    // 4.0 at 262,000; by the two-kernel sparse pass before 3.4, 3.7 and 6.2; one launch for the call, to which the rule
+    // does not let them, 1.4 and 1.5 at half marked.)
+    if (sparse && s->kernel_variant == 5 && s->act.n_active * 8 >= s->n * 5) sparse = false;
     if (sparse && small_ok(s, s->act)) {  // the whole call as one launch, or a few
         StateRows rows;
         for (int c = 0; c < 5; ++c) {
