@@ -329,7 +329,8 @@ vga_status vga_sim_set_kernel(vga_sim *s, int32_t variant, int32_t chunk);
  * fused pass then diffuses the DOM of every node, transforms only the marked nodes (their MB, SOM, FOM
  * and CO2 held in a compact rank-ordered copy during the call), and leaves the MB, SOM, FOM and CO2 of
  * the others unread and unwritten.  A call of variant 5 whose mask marks five eighths of the nodes or more runs
- * dense passes; on graphs of up to 0.3 M nodes a call's passes are one launch.  Results are bit-identical with the
+ * dense passes; on graphs of up to 0.3 M nodes a call's passes are one launch (on a stream of
+ * its own a simulation's up to some 38,000 nodes, so that several such simulations overlap).  Results are bit-identical with the
  * mask off (also a node whose values are negative zeros is marked), as long as no mass is negative: an
  * unmarked node whose DOM is negative transforms in the first pass of each call only.  on = 0 transforms every
  * node every pass. */

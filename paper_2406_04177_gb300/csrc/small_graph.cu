@@ -18,7 +18,7 @@
 // sweep per step with recomputation, 8^3 blocks, without / with dL/dX^0: 64^3 3.2 / 3.8 us (9.2 by launches), 96^3
 // 4.2 / 5.1, 128^3 7.2 / - (13.2).  The line at four nodes per thread lies where registers end.
 // The first transformation, the last diffusion-only pass, the checkpoint of a segment and the moves to and
-// from the compact state are part of the launch.  The arithmetic and its order are those of
+// from the compact state are part of the launch.  Several simulations at once: see small_step_ok.  The arithmetic and its order are those of
 // k_transform, sparse_pass.cuh and k_adjoint_vec, so states and adjoints are the same bits.  With dL/dX^0 the
 // gradient sums are also those of k_adjoint_vec, one per pair of consecutive nodes; without it they take
 // the nodes in another order.
@@ -785,6 +785,23 @@ bool small_ok(const vga_sim *s, const Activity &act) {
     return s->kernel_variant == 5 && s->activity_skip && !s->timing && !s->subcycled() && s->precision() == P_COMP &&
            s->g->nx <= kSmallThreads && act.max_block >= 0 && act.max_block <= kSmallThreads && !act.negative_dom &&
            6.0 * s->params.D * s->params.dt * s->max_g <= 0.999;
+}
+
+// A launch takes its blocks' SMs whole, so simulations that step on streams of their own run beside each other only as far
+// as their blocks fit, and otherwise take turns; launches per pass overlap.  One stream keeps the launch at every size;
+// with a stream of its own, which a program gives a simulation to overlap it with other work, a simulation whose launch
+// takes more than half of the SMs steps by launches.  us per step and simulation, 20 steps a call, 1 / 2 / 4 / 8
+// streams, one launch per call | launches (two a pass, before there was the other form):
+//   64^3 (62 blocks)   1.36 / 0.70 / 0.61 / 0.61 | - (4.16 / 2.14 / 1.12 / 0.60)
+//   96^3 (77 blocks)   1.66 / 1.44 / 1.44 / 1.44 | 2.89 / 1.54 / 0.92 / 0.56 (4.06 / 2.20 / 1.22 / 0.68)
+//   128^3 (149 blocks) 2.59 / 2.41 / 2.39 / 2.60 | 3.31 / 2.33 / 1.31 / 1.19 (4.54 / 3.04 / 1.72 / 1.22)
+// Adjoint sweeps, which synchronise, gain at every number of threads and streams (96^3, 8 of them: 4.7 us a step against
+// 9.6).
+bool small_step_ok(const vga_sim *s) {
+    int dev = 0, sms = 0, K = 0, G = 0;
+    if (!s->stream) return true;
+    return cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+           small_shape(s->n, &K, &G) && 2 * G <= sms;
 }
 
 vga_status small_forward(vga_sim *s, const Activity &act, StateRows in, StateRows out, StateRows ck, int64_t passes,

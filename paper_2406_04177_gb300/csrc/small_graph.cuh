@@ -18,6 +18,9 @@ bool small_shape(int64_t n, int *K, int *G);
 // Whether step calls of this simulation may run as small-graph launches with the marked set `act`.
 bool small_ok(const vga_sim *s, const Activity &act);
 
+// Whether a step call may hold the launch's SMs, given the simulation's stream.
+bool small_step_ok(const vga_sim *s);
+
 // The five rows of a compensated state.
 struct StateRows {
     float *h[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};

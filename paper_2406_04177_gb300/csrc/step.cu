@@ -1076,7 +1076,7 @@ vga_status sim_step_explicit(vga_sim *s, int64_t n_steps) {
     // 4.0 at 262,000; by the two-kernel sparse pass before 3.4, 3.7 and 6.2; one launch for the call, to which the rule
     // does not let them, 1.4 and 1.5 at half marked.)
     if (sparse && s->kernel_variant == 5 && s->act.n_active * 8 >= s->n * 5) sparse = false;
-    if (sparse && small_ok(s, s->act)) {  // the whole call as one launch, or a few
+    if (sparse && small_ok(s, s->act) && small_step_ok(s)) {  // the whole call as one launch, or a few
         StateRows rows;
         for (int c = 0; c < 5; ++c) {
             rows.h[c] = s->comp(c);
