@@ -1089,7 +1089,13 @@ vga_status vga_pngm_step(vga_pngm *pg, double *d_m, int64_t n_steps, int32_t sch
     int dev = 0, sms = 0;
     VGA_CUDA(cudaGetDevice(&dev));
     VGA_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const int G = (int)std::max<int64_t>(1, std::min<int64_t>(std::min(sms, kPcgThreads), grid_for(q, kPcgThreads / 4)));
+    // Alone, a block for 64 rows up to every SM.  With a stream of its own a handle leaves room for others, whose
+    // launches take their turn where the blocks do not fit: a block for 256 rows up to an eighth of the SMs.  us per solve,
+    // 1 / 4 / 8 / 16 threads with a handle and a stream each, and with the first rule there too (one block per solve before
+    // either): q = 30,719 972 / 259 / 131 / 132, 630 / 599 / 602 / 601 (6086 / 1553 / 771 / 405); q = 1,939
+    // 528 / 137 / 72 / 39, 567 / 146 / 140 / 137 (669 / 174 / 90 / 48).
+    const int64_t most = st ? std::min<int64_t>(sms / 8, grid_for(q, kPcgThreads)) : std::min<int64_t>(sms, grid_for(q, kPcgThreads / 4));
+    const int G = (int)std::max<int64_t>(1, std::min<int64_t>(most, kPcgThreads));
     // u, r, p, inverse diagonal, A p; then the words, zeroed; then the statistics
     const int64_t words = 2 * (int64_t)q + 8 * (int64_t)G + 8;
     VGA_TRY(ensure_work(pg, 5 * (int64_t)q + words + 8));

@@ -46,3 +46,32 @@ def test_several_streams_at_once():
     for s in sims + [ref]:
         s.close()
     g.close()
+
+
+def test_coarse_solves_leave_room_on_an_own_stream():
+    """4096 rows: 64 blocks on the default stream, 16 on another (block 20 is there or not).  Solves stop at a residual of
+    1e-12; with equal volumes the masses are then within 1e-12 of the solution per step, whatever the order of the sums."""
+    shape = (48, 48, 48)
+    g = vga.Graph(np.zeros(shape, dtype=np.uint8))
+    labels, q = synth.block_primitives(shape, g.export(labels=False, nbr=False)["voxel_of_node"], 3)
+    m0 = torch.rand(q, generator=torch.Generator(device="cuda").manual_seed(2), device="cuda", dtype=torch.float64)
+    torch.cuda.synchronize()
+    p = synth.diffusion_params()
+    args = (3, vga.VGA_SCHEME_IMPLICIT_PCG, p["D"], p["dt"])
+    out = []
+    for stream in (None, torch.cuda.Stream()):
+        pg = vga.Pngm(g, labels, q, stream=stream)
+        m = m0.clone()
+        torch.cuda.synchronize()
+        pg.step(m, *args)
+        out.append(m.cpu().numpy())
+        pg.set_wait_test(20, 4096)
+        if stream is None:
+            with pytest.raises(vga.VgaError) as e:
+                pg.step(m, *args)
+            assert e.value.name == "VGA_ERR_TIMEOUT"
+        else:
+            pg.step(m, *args)
+        pg.close()
+    assert np.linalg.norm(out[0] - out[1]) <= 2 * 3 * 1e-12 * np.linalg.norm(out[0])
+    g.close()
