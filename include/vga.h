@@ -444,7 +444,10 @@ vga_status vga_batch_free(vga_batch *b);
  * around every kernel it launches and accumulates the elapsed times per kernel kind; reading them
  * synchronises the stream.  The fused passes of one explicit step call are timed as one span and
  * counted as that many launches (an event pair between two passes would keep the second from being
- * scheduled during the first's tail), so ms / launches is their live mean per pass.  Kinds: */
+ * scheduled during the first's tail), so ms / launches is their live mean per pass.
+ * While timing is on, the step calls and sweeps of small graphs run by launches per pass instead of one
+ * launch (see vga_sim_set_activity_skip): the times are those of kernels that an untimed run does not use
+ * there.  Kinds: */
 #define VGA_KERNEL_FUSED_STEP 0    /* explicit pass: diffuse stored transformed DOM, transform */
 #define VGA_KERNEL_TRANSFORM 1     /* transformation-only pass (first pass of a step call) */
 #define VGA_KERNEL_DIFFUSE 2       /* diffusion-only pass (last pass of a step call) */

@@ -115,6 +115,7 @@ static vga_status harvest_timing(vga_sim *s) {
 // leaves behind.
 vga_status sim_device_error(vga_sim *s, int32_t h) {
     if (h != 0) {
+        s->report->err = 0;  // reported: a call that fails before its own copy arrives must not see it
         cudaMemsetAsync(s->d_err, 0, sizeof(int32_t), s->stream);
         small_reset(s);
         return fail(VGA_ERR_TIMEOUT, h == 3   ? "a bounded device wait timed out (small-graph launch)"
