@@ -612,7 +612,7 @@ BATCH_CHECK_STEPS = 200
 
 def bench_batched(vga, a, held=None, count=64, nsteps=5000):
     """64 subvolumes, side U{64..192}, porosity U(10%, 35%), rates log-uniform in [0.5, 1.5] x the
-    paper's, 5000 steps in persistent graph-captured launches (launch shape autotuned).  For the FP64
+    paper's, 5000 steps in graph-captured launches (launch shape autotuned).  For the FP64
     comparison the same batch then runs BATCH_CHECK_STEPS steps from the initial masses and the
     states of a size-stratified sample of instances are kept in `held`."""
     import synth

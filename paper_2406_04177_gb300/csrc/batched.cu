@@ -121,8 +121,8 @@ __device__ __forceinline__ void batch_sparse_pass(const BatchArgs &a, const Stat
 // One sparse fused pass as a launch of its own (the default launch shape): 1024 nodes per block, no
 // grid barrier, scheduled in the tail of the pass before it (programmatic dependent launch).  The
 // persistent form below keeps every block for the whole launch and makes it wait at a grid barrier
-// after every pass.  Per pass: 12 subvolumes, 8.2 M nodes: 33.7 us (persistent 46.4); 40
-// subvolumes, 24.5 M nodes: 97 us (126); 6 subvolumes, 0.53 M nodes: 4.7 us (6.5).
+// after every pass.  Per pass: 12 subvolumes, 8.1 M nodes: 33.4 us (persistent 44.0); 64
+// subvolumes, 31.2 M nodes: 125 us (153); 6 subvolumes, 0.53 M nodes: 4.7 us (6.5).
 template <int TR, int PREC, int TF, bool AHEAD>
 __global__ void __launch_bounds__(kSparseThreads, 6) k_batch_sparse_pass(BatchArgs a, int bi, int ahead) {
     __shared__ SparseShared sm;

@@ -13,10 +13,10 @@
 // Neighbours in the same block come from shared memory.  The launch is cooperative (every block is
 // resident, one per SM) and every wait is bounded: one that gives up sets the simulation's error flag,
 // and the blocks leave.
-// Per pass, 17% porosity, unit conductances, against launches: 64^3 1.13 us (2.2), 96^3 1.40 (2.6), 128^3, 0.30 M
-// nodes, 2.14 (2.6; four nodes per thread, where it is bound by instruction issue: 16 warps per SM). Backward
-// sweep per step with recomputation, 8^3 blocks, without / with dL/dX^0: 64^3 3.2 / 3.8 us (9.2 by launches), 96^3
-// 4.2 / 5.1, 128^3 7.2 / - (13.2).  The line at four nodes per thread lies where registers end.
+// Per pass, 17% porosity, unit conductances, against launches: 64^3 1.13 us (2.4), 96^3 1.43 (2.5), 128^3, 0.30 M
+// nodes, 2.25 (2.9; four nodes per thread, where it is bound by instruction issue: 16 warps per SM, 56% of the
+// slots). Backward sweep per step with recomputation, 8^3 blocks, without / with dL/dX^0: 64^3 3.1 / 3.3 us, 96^3
+// 3.9 / 4.6, 128^3 6.7 / - (11.1 by launches).  The line at four nodes per thread lies where registers end.
 // The first transformation, the last diffusion-only pass, the checkpoint of a segment and the moves to and
 // from the compact state are part of the launch.  Several simulations at once: see small_step_ok.  The arithmetic and its order are those of
 // k_transform, sparse_pass.cuh and k_adjoint_vec, so states and adjoints are the same bits.  With dL/dX^0 the
