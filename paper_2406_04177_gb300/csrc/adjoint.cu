@@ -1434,13 +1434,17 @@ static vga_status adjoint_backward_impl(vga_sim *s, const double *d_lamN, double
         }
     }
     if (nseg > 1) a->last_recorded = false;  // the records now hold the first segment
-    if (d_lam0) {
+    auto lam_out = [&]() -> vga_status {
         StateIO io = io_from(a->lam[lb], a->lam[lb], npad);  // CO2 from lam[0]
         io.in[4] = a->lam[0].h + 4 * (size_t)npad;
         io.lin[4] = a->lam[0].l + 4 * (size_t)npad;
         k_lam_out<<<grid_for(s->n, kThreads), kThreads, 0, st>>>(s->n, d_lam0, io);
         VGA_CHECK_LAUNCH();
-    }
+        return VGA_OK;
+    };
+    // dL/dX^0 may go where dL/dX^N came from, so a sweep that may be repeated writes it when it has held
+    const bool out_last = d_lam0 && flag_dev;
+    if (d_lam0 && !out_last) VGA_TRY(lam_out());
     if (tacc) {
         k_reduce_tacc<<<(unsigned)(Ts / kThreads), kThreads, 0, st>>>(tacc, a->gpart);
         ++s->launches;
@@ -1466,6 +1470,10 @@ static vga_status adjoint_backward_impl(vga_sim *s, const double *d_lamN, double
     if (flag[0] || flag[1]) {
         *redo = true;
         return VGA_OK;
+    }
+    if (out_last) {
+        VGA_TRY(lam_out());
+        VGA_CUDA(cudaStreamSynchronize(st));
     }
     a->grad_ready = s->wmode == W_BLOCK && s->n_theta > 0;
     const double dt = s->params.dt;

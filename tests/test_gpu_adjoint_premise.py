@@ -69,6 +69,33 @@ def test_small_graph_with_negative_stocks(shape, state_gradient):
     g.close()
 
 
+@pytest.mark.parametrize("where", ["host", "in place"])
+def test_a_repeated_sweep_reads_its_input_again(where):
+    """The host form stages both gradients in one buffer, and a caller may pass one for both: the sweep that is
+    repeated must not have overwritten dL/dX^N."""
+    g = vga.Graph(np.zeros((9, 11, 13), dtype=np.uint8))
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    X, marked = _state(g.n, gen)
+    X[1] = 0.0
+    X[3] = torch.where(marked, -1e-3, 0.0)  # repeats, as above
+    lam = torch.randn((5, g.n), generator=gen, device="cuda", dtype=torch.float64)
+    sim = vga.Sim(g, synth.paper_params())
+    sim.set_masses(X)
+    sim.adjoint_forward(11, 4)
+    dx = torch.zeros_like(lam)
+    ref, _ = sim.adjoint_backward(lam, dx)
+    if where == "host":
+        out = np.zeros((5, g.n))
+        got, _ = sim.adjoint_backward(lam.cpu().numpy(), out)
+    else:
+        buf = lam.clone()
+        got, _ = sim.adjoint_backward(buf, buf)
+        out = buf.cpu().numpy()
+    assert got == ref and np.array_equal(out, dx.cpu().numpy())
+    sim.close()
+    g.close()
+
+
 @pytest.mark.parametrize("shape", [(9, 11, 13), (40, 44, 52), (79, 84, 85)])
 @pytest.mark.parametrize("state_gradient", [False, True])
 @pytest.mark.parametrize("value", [float("inf"), float("nan")])
