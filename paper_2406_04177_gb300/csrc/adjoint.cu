@@ -1251,8 +1251,8 @@ static vga_status adjoint_backward_impl(vga_sim *s, const double *d_lamN, double
     // small graphs: a segment's recomputation and its reverse steps are one launch each
     const bool may_lean = lean && sparse && !d_lam0 && !plain;
     // (with dL/dX^0 its sums are one per pair of nodes: k_adjoint_vec's, when each of its threads takes one pair)
-    const bool small = sparse && !plain && a->small_fwd && small_ok(s, a->act) && std::min(ckpt, N) <= kSmallSteps && small_reverse_ok(s, !may_lean) &&
-                       (may_lean || (kAdjK == 2 && (int64_t)Gt * kThreads * 2 >= s->n));
+    const bool small = sparse && !plain && a->small_fwd && small_ok(s, a->act) && std::min(ckpt, N) <= kSmallSteps &&
+                       small_reverse_ok(s, !may_lean) && (may_lean || (kAdjK == 2 && (int64_t)Gt * kThreads * 2 >= s->n));
     // Above a quarter of the nodes marked a lean step moves as much as a full one (36 B per node and about
     // 120 B per marked node against 66 B per node); on small graphs its second launch costs more than it
     // saves.  Backward sweep per step, recomputation included, 6% marked, 8^3 blocks: 0.57 M nodes 19.9 us

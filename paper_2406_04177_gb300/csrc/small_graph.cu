@@ -18,10 +18,10 @@
 // slots). Backward sweep per step with recomputation, 8^3 blocks, without / with dL/dX^0: 64^3 3.1 / 3.3 us, 96^3
 // 3.9 / 4.6, 128^3 6.7 / - (11.1 by launches).  The line at four nodes per thread lies where registers end.
 // The first transformation, the last diffusion-only pass, the checkpoint of a segment and the moves to and
-// from the compact state are part of the launch.  Several simulations at once: see small_step_ok.  The arithmetic and its order are those of
+// from the compact state are part of the launch.  The arithmetic and its order are those of
 // k_transform, sparse_pass.cuh and k_adjoint_vec, so states and adjoints are the same bits.  With dL/dX^0 the
 // gradient sums are also those of k_adjoint_vec, one per pair of consecutive nodes; without it they take
-// the nodes in another order.
+// the nodes in another order.  Several simulations at once: see small_step_ok.
 #include <cuda_runtime.h>
 
 #include <algorithm>
