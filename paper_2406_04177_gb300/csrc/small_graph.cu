@@ -334,38 +334,43 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_forward(SmallArgs a,
 
     // pass 0: the transformation alone, of every node as in k_transform: the mask tells of the state it was built from, and
     // since then an implicit solve, a call at the stability bound or a negative FOM nearby may have left an unmarked node with
-    // a DOM below zero, which the transformation clamps at the cost of the biomass (nothing else changes there, so the
-    // store is rare; the loads are 24 B per node and launch).  In the middle of a call unmarked nodes do not transform
-    // in any form: that adds zero to the pair.
+    // a DOM below zero, which the transformation clamps at the cost of the biomass.  At a node that still holds
+    // nothing but DOM it adds zero to the pair; in the middle of a call unmarked nodes do not transform in any form.
+    // (16 B more per node and launch, on their way together: a stored value's residual is below half an ulp of it, so
+    // none is left of a zero.)
+    uint32_t holds[K];
 #pragma unroll
     for (int k = 0; k < K; ++k) {
         const uint32_t i = node_of(i0, k);
+        holds[k] = 0u;
+        if (f.first && i < a.n && !((act >> k) & 1u)) {
+#pragma unroll
+            for (int c = 0; c < 5; ++c)
+                if (c != 1) holds[k] |= __float_as_uint(f.in.h[c][i]);
+            holds[k] |= unmarked_identity(x2[k].h) ? 0u : 1u;
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
         if ((act >> k) & 1u) continue;
-        if (!f.first || i >= a.n) {
+        if (!holds[k]) {
             x2[k] = V{__fadd_rn(x2[k].h, 0.0f), __fadd_rn(x2[k].l, 0.0f)};
             continue;
         }
+        const uint32_t i = node_of(i0, k);
         V u[4];
-        res_t l[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int c = q > 0 ? q + 1 : 0;  // MB, SOM, FOM, CO2
             u[q].h = f.in.h[c][i];
-            l[q] = f.in.l[c][i];
-            u[q].l = res_decode(l[q], u[q].h);
+            u[q].l = res_decode(f.in.l[c][i], u[q].h);
         }
-        const V was[4] = {u[0], u[1], u[2], u[3]};
-        if (f.flag && !unmarked_identity(x2[k].h)) atomicOr(f.flag, 1);
+        if (f.flag) atomicOr(f.flag, 1);
         transform<TR, PREC>(u[0], x2[k], u[1], u[2], u[3], a.p);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            vround<PREC>(u[q]);
             const int c = q > 0 ? q + 1 : 0;
-            const bool moved = __float_as_uint(u[q].h) != __float_as_uint(was[q].h) || res_encode(u[q].l, u[q].h) != l[q];
-            if (moved && f.out.h[c]) {
-                f.out.h[c][i] = u[q].h;
-                f.out.l[c][i] = res_encode(u[q].l, u[q].h);
-            }
+            if (f.out.h[c]) vstore<PREC>(f.out.h[c], f.out.l[c], i, u[q]);
         }
     }
     publish(0, 0, false, true);
